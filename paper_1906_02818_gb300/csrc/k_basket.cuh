@@ -85,6 +85,8 @@ __global__ void __launch_bounds__(kLaunchBlock, 1) basket_fp32_kernel(const __gr
             }
             NormalReader rd;
             rd.init(n, a.run.rk);
+            PathStream ps;
+            ps.init(n, a.run.rk);
             for (int i = 0; i < M; ++i) {
                 // log-Euler accumulates L z straight into the state (|y| = O(1):
                 // ~65 roundings of <= 3e-8 per step, ~2e-6 rms over 252 steps);
@@ -102,13 +104,13 @@ __global__ void __launch_bounds__(kLaunchBlock, 1) basket_fp32_kernel(const __gr
                 // next block of four normals is drawn before this block's
                 // products (independent work while the SFU results arrive).
                 float4 znext = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (EXACT) znext = normals4(static_cast<uint64_t>(i) * (D / 4), n, a.run.rk);
+                if (EXACT) znext = ps.normals(static_cast<uint32_t>(i) * (D / 4), a.run.rk).f4();
 #pragma unroll
                 for (int kb = 0; kb < D / 4 + (D % 4 ? 1 : 0); ++kb) {
                     float zz[4];
                     if (EXACT) {
                         const float4 z4 = znext;
-                        if (kb + 1 < D / 4) znext = normals4(static_cast<uint64_t>(i) * (D / 4) + kb + 1, n, a.run.rk);
+                        if (kb + 1 < D / 4) znext = ps.normals(static_cast<uint32_t>(i) * (D / 4) + kb + 1, a.run.rk).f4();
                         zz[0] = z4.x; zz[1] = z4.y; zz[2] = z4.z; zz[3] = z4.w;
                     } else {
 #pragma unroll
@@ -187,7 +189,7 @@ const void *basket_select_impl(const BasketArgs &a)
 {
     const bool stats = a.pay.need_avg || a.pay.need_max || a.pay.need_min;
     const bool save = a.run.save != nullptr;
-    const bool exact = (a.d == D) && (D % 4 == 0);
+    const bool exact = (a.d == D) && (D % 4 == 0) && blocks_fit_32(a.run.steps, D);
     if (save) return basket_fn<D, SCHEME, false, true, false>();
     if (stats) return exact ? basket_fn<D, SCHEME, true, false, true>() : basket_fn<D, SCHEME, true, false, false>();
     return exact ? basket_fn<D, SCHEME, false, false, true>() : basket_fn<D, SCHEME, false, false, false>();

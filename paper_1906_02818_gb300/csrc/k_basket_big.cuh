@@ -109,8 +109,8 @@ using tc::wait_or_fail;
 // One worker's 16 normals of a Z panel (columns c0 .. c0 + 15 of its path
 // row at step i), rounded to the operand type and stored swizzled.
 template <int PREC>
-__device__ __forceinline__ void draw_panel(uint32_t pan, int row, int grp, int c0, int i, int d, bool valid, uint64_t n,
-                                           int exact4, const RoundKeys &rk, NormalReader &rd)
+__device__ __forceinline__ void draw_panel(uint32_t pan, int row, int grp, int c0, int i, int d, bool valid,
+                                           const PathStream &ps, int exact4, const RoundKeys &rk, NormalReader &rd)
 {
     using Ly = L2<PREC>;
     float z[16];
@@ -118,10 +118,10 @@ __device__ __forceinline__ void draw_panel(uint32_t pan, int row, int grp, int c
     for (int l = 0; l < 16; ++l) z[l] = 0.0f;
     if (valid && c0 < d) {
         if (exact4 && c0 + 16 <= d) {
-            const uint64_t q = (static_cast<uint64_t>(i) * d + c0) >> 2;
+            const uint32_t q = static_cast<uint32_t>(i) * (d >> 2) + (c0 >> 2);
 #pragma unroll
             for (int bq = 0; bq < 4; ++bq) {
-                const float4 v = normals4(q + bq, n, rk);
+                const float4 v = ps.normals(q + bq, rk).f4();
                 z[4 * bq] = v.x; z[4 * bq + 1] = v.y; z[4 * bq + 2] = v.z; z[4 * bq + 3] = v.w;
             }
         } else {
@@ -284,12 +284,14 @@ __global__ void __launch_bounds__(kThreads, 1) basket_big_kernel(const __grid_co
             const uint64_t n = static_cast<uint64_t>(a.run.path_offset + (valid ? nl : 0));
             NormalReader rd;
             rd.init(n, a.run.rk);
+            PathStream ps;
+            ps.init(n, a.run.rk);
             for (int i = 0; i < M; ++i, ++g) {
                 for (int hh = 0; hh < 2; ++hh) {
                     const bool ok = g == 0 || wait_or_fail(&s_fail, zfree + 8 * hh, static_cast<uint32_t>((g - 1) & 1), cap);
                     if (ok && !s_fail) {
                         for (int p = hh ? half : 0; p < (hh ? NP : half); ++p)
-                            draw_panel<PREC>(zt + p * Ly::kPanelBytes, row, grp, p * kPanel + grp * 16, i, d, valid, n,
+                            draw_panel<PREC>(zt + p * Ly::kPanelBytes, row, grp, p * kPanel + grp * 16, i, d, valid, ps,
                                              a.exact4, a.run.rk, rd);
                         tc::fence_proxy_async();
                     }

@@ -88,10 +88,10 @@ struct Stats {
     float sum, umax, umin;
 };
 
-// Draws Z_i of path n (row `row`) into the tile at `tile`; returns the
+// Draws Z_i of the path of ps / rd (row `row`) into the tile at `tile`; returns the
 // dequantisation factor of the row (1 unless E4M3).
 template <int PREC, bool EXACT>
-__device__ __forceinline__ float draw_row(uint32_t tile, int row, int i, int d, uint64_t n,
+__device__ __forceinline__ float draw_row(uint32_t tile, int row, int i, int d, const PathStream &ps,
                                           const RoundKeys &rk, NormalReader &rd, bool valid)
 {
     using Ly = Layout<PREC>;
@@ -100,8 +100,8 @@ __device__ __forceinline__ float draw_row(uint32_t tile, int row, int i, int d, 
 #pragma unroll
             for (int l = 0; l < 8; ++l) z[l] = 0.0f;
         } else if (EXACT) {
-            const uint64_t q = static_cast<uint64_t>(i) * (kN / 4) + c0 / 4;
-            const float4 a = normals4(q, n, rk), b = normals4(q + 1, n, rk);
+            const uint32_t q = static_cast<uint32_t>(i) * (kN / 4) + c0 / 4;
+            const float4 a = ps.normals(q, rk).f4(), b = ps.normals(q + 1, rk).f4();
             z[0] = a.x; z[1] = a.y; z[2] = a.z; z[3] = a.w; z[4] = b.x; z[5] = b.y; z[6] = b.z; z[7] = b.w;
         } else {
 #pragma unroll
@@ -209,6 +209,8 @@ __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_consta
         const uint64_t n = static_cast<uint64_t>(a.run.path_offset + (valid ? nl : 0));
         NormalReader rd;
         rd.init(n, a.run.rk);
+        PathStream ps;
+        ps.init(n, a.run.rk);
         float x[kN];
 #pragma unroll
         for (int j = 0; j < kN; ++j) x[j] = (SCHEME == MC_LOG_EULER) ? 0.0f : c.s0[j];
@@ -216,7 +218,7 @@ __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_consta
 
         float deq_cur = 1.0f, deq_next = 1.0f;
         if (!aborted) {
-            deq_cur = draw_row<PREC, EXACT>(zt[0], t, 0, d, n, a.run.rk, rd, valid);
+            deq_cur = draw_row<PREC, EXACT>(zt[0], t, 0, d, ps, a.run.rk, rd, valid);
             tc::fence_proxy_async();
         }
         __syncthreads();
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_consta
         }
         for (int i = 0; i < M && !aborted; ++i) {
             if (i + 1 < M) {
-                deq_next = draw_row<PREC, EXACT>(zt[(i + 1) & 1], t, i + 1, d, n, a.run.rk, rd, valid);
+                deq_next = draw_row<PREC, EXACT>(zt[(i + 1) & 1], t, i + 1, d, ps, a.run.rk, rd, valid);
                 tc::fence_proxy_async();
             }
             const bool ok = tc::mbar_wait_bounded(mbar, phase & 1u, a.wait_cap);
@@ -394,12 +396,14 @@ __global__ void __launch_bounds__(kThreads, 8) basket_tc_acc_kernel(const __grid
         const uint64_t n = static_cast<uint64_t>(a.run.path_offset + (valid ? nl : 0));
         NormalReader rd;
         rd.init(n, a.run.rk);
+        PathStream ps;
+        ps.init(n, a.run.rk);
         Stats st{0.0f, -INFINITY, INFINITY};
         bool ok = true;
         for (int i = 0; i < M; ++i) {
             // s_g[(i + 1) & 1] was last read before the previous step's barrier
             if (STATS || i + 1 == M) set_g(i + 1);
-            if (!aborted) draw_row<PREC, EXACT>(zt, t, i, d, n, a.run.rk, rd, valid);
+            if (!aborted) draw_row<PREC, EXACT>(zt, t, i, d, ps, a.run.rk, rd, valid);
             tc::fence_proxy_async();
             tc::fence_before_sync();  // this thread's accumulator reads precede the next MMA
             if (__syncthreads_or(ok ? 0 : 1)) aborted = true;
@@ -508,7 +512,7 @@ template <int PREC, int SCHEME>
 const void *basket_tc_select(const TcArgs &a, int *smem)
 {
     const bool stats = a.pay.need_avg || a.pay.need_max || a.pay.need_min;
-    const bool exact = a.d == tcb::kN;
+    const bool exact = a.d == tcb::kN && blocks_fit_32(a.run.steps, tcb::kN);
     if constexpr (PREC != MC_FP8E4M3 && SCHEME == MC_LOG_EULER) {
         // TMEM running sum: Z tile + factor tile + barriers + payoff slots
         // (~27 KB with the static arrays and the per-block reservation: at

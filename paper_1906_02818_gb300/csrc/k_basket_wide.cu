@@ -67,13 +67,15 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
         const uint64_t rn = static_cast<uint64_t>(a.run.path_offset + (rvalid ? rnl : 0));
         NormalReader rd;
         rd.init(rn, a.run.rk);
+        PathStream ps;
+        ps.init(rn, a.run.rk);
         for (int i = 0; i < M; ++i) {
             __syncthreads();  // previous step done with zs
             for (int k = rq * (D / 8); k < (rq + 1) * (D / 8); k += 4) {
                 float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (rvalid && k < d) {
                     if (a.exact4) {
-                        z = normals4((static_cast<uint64_t>(i) * d + k) >> 2, rn, a.run.rk);
+                        z = ps.normals((static_cast<uint32_t>(i) * (d >> 2)) + (k >> 2), a.run.rk).f4();
                     } else {
                         const uint64_t j0 = static_cast<uint64_t>(i) * d + k;
                         z.x = rd.get(j0);

@@ -59,11 +59,13 @@ __global__ void __launch_bounds__(kThreads) corr_path_kernel(const __grid_consta
         for (int k = 0; k < kD; ++k) W[k] = 0.0f;
         if (EXACT) {
             const int nb = d >> 2;
+            PathStream ps;
+            ps.init(n, a.run.rk);
             for (int i = 0; i < M; ++i) {
 #pragma unroll
                 for (int kb = 0; kb < kD / 4; ++kb) {
                     if (kb < nb) {
-                        const float4 z = normals4(static_cast<uint64_t>(i) * nb + kb, n, a.run.rk);
+                        const float4 z = ps.normals(static_cast<uint32_t>(i) * nb + kb, a.run.rk).f4();
                         W[4 * kb] += z.x;
                         W[4 * kb + 1] += z.y;
                         W[4 * kb + 2] += z.z;
@@ -245,7 +247,7 @@ __global__ void corr_finish_kernel(int d, int B, const double *nb, const double 
 // in registers across the launch).
 constexpr int kAsianStride = kD + 4;  // staged row stride (floats; 16-B aligned rows)
 
-__device__ __forceinline__ void asian_draw(bool exact, int i, int d, uint64_t n, const RoundKeys &rk,
+__device__ __forceinline__ void asian_draw(bool exact, int i, int d, const PathStream &ps, const RoundKeys &rk,
                                            NormalReader &rd, float (&W)[kD])
 {
     if (exact) {
@@ -253,7 +255,7 @@ __device__ __forceinline__ void asian_draw(bool exact, int i, int d, uint64_t n,
 #pragma unroll
         for (int kb = 0; kb < kD / 4; ++kb) {
             if (kb < nb) {
-                const float4 z = normals4(static_cast<uint64_t>(i) * nb + kb, n, rk);
+                const float4 z = ps.normals(static_cast<uint32_t>(i) * nb + kb, rk).f4();
                 W[4 * kb] += z.x;
                 W[4 * kb + 1] += z.y;
                 W[4 * kb + 2] += z.z;
@@ -303,9 +305,11 @@ __global__ void __launch_bounds__(kThreads) corr_asian_kernel(const __grid_const
         for (int k = 0; k < kD; ++k) W[k] = 0.0f;
         NormalReader rd;
         rd.init(n, a.run.rk);
+        PathStream ps;
+        ps.init(n, a.run.rk);
         float sumU = 0.0f;
         for (int i = 0; i < M; ++i) {
-            asian_draw(EXACT, i, d, n, a.run.rk, rd, W);
+            asian_draw(EXACT, i, d, ps, a.run.rk, rd, W);
             const float fi = static_cast<float>(i + 1);
             float U = 0.0f;
 #pragma unroll
@@ -328,7 +332,7 @@ __global__ void __launch_bounds__(kThreads) corr_asian_kernel(const __grid_const
         for (int k = 0; k < kD; ++k) W[k] = 0.0f;
         rd.init(n, a.run.rk);
         for (int i = 0; any && i < M; ++i) {
-            asian_draw(EXACT, i, d, n, a.run.rk, rd, W);
+            asian_draw(EXACT, i, d, ps, a.run.rk, rd, W);
             const float fi = static_cast<float>(i + 1);
             float *vr = sv + t * kAsianStride, *wr = sw + t * kAsianStride;
 #pragma unroll
@@ -382,17 +386,19 @@ __global__ void __launch_bounds__(128) corr_wsum_kernel(const __grid_constant__ 
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t p = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; p < a.run.paths; p += stride) {
         const uint64_t n = static_cast<uint64_t>(a.run.path_offset + p);
+        PathStream ps;
+        ps.init(n, a.run.rk);
         for (int c0 = 0; c0 < d; c0 += kWChunk) {
             float W[kWChunk];
 #pragma unroll
             for (int k = 0; k < kWChunk; ++k) W[k] = 0.0f;
             if (EXACT) {  // d % 4 == 0: step i's normals are blocks i d/4 .. i d/4 + d/4 - 1
-                const uint64_t nb = static_cast<uint64_t>(d >> 2);
+                const uint32_t nb = static_cast<uint32_t>(d >> 2);
                 for (int i = 0; i < M; ++i) {
 #pragma unroll
                     for (int kb = 0; kb < kWChunk / 4; ++kb) {
                         if (c0 + 4 * kb < d) {
-                            const float4 z = normals4(static_cast<uint64_t>(i) * nb + (c0 >> 2) + kb, n, a.run.rk);
+                            const float4 z = ps.normals(static_cast<uint32_t>(i) * nb + (c0 >> 2) + kb, a.run.rk).f4();
                             W[4 * kb] += z.x;
                             W[4 * kb + 1] += z.y;
                             W[4 * kb + 2] += z.z;

@@ -78,9 +78,11 @@ __global__ void __launch_bounds__(kBlock, 2) factor_kernel(const __grid_constant
             for (int e = 0; e < kA; ++e) x[p][e] = SCHEME == MC_LOG_EULER ? 0.0f : a.s0[a0 + e];
         float sum = 0.0f, umax = -INFINITY, umin = INFINITY, uT = 0.0f;  // lanes 0..3 of warp gw = 0: path `lane`
         NormalReader rd[kP];
-        if (!EXACT) {
+        PathStream ps[kP];
 #pragma unroll
-            for (int p = 0; p < kP; ++p) rd[p].init(n[p], a.run.rk);
+        for (int p = 0; p < kP; ++p) {
+            if (EXACT) ps[p].init(n[p], a.run.rk);
+            else rd[p].init(n[p], a.run.rk);
         }
         for (int i = 0; i < M; ++i) {
             const uint64_t base = static_cast<uint64_t>(i) * stride;
@@ -116,9 +118,9 @@ __global__ void __launch_bounds__(kBlock, 2) factor_kernel(const __grid_constant
             for (int p = 0; p < kP; ++p) {
                 float eps[kA];
                 if (EXACT) {
-                    const uint64_t q = (base + k + a0) / 4;
-                    const float4 e0 = a0 < d ? normals4(q, n[p], a.run.rk) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const float4 e1 = a0 + 4 < d ? normals4(q + 1, n[p], a.run.rk) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const uint32_t q = static_cast<uint32_t>((base + k + a0) / 4);
+                    const float4 e0 = a0 < d ? ps[p].normals(q, a.run.rk).f4() : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float4 e1 = a0 + 4 < d ? ps[p].normals(q + 1, a.run.rk).f4() : make_float4(0.f, 0.f, 0.f, 0.f);
                     eps[0] = e0.x; eps[1] = e0.y; eps[2] = e0.z; eps[3] = e0.w;
                     eps[4] = e1.x; eps[5] = e1.y; eps[6] = e1.z; eps[7] = e1.w;
                 } else {

@@ -28,12 +28,10 @@ __device__ __forceinline__ void accumulate_payoffs(AccSlot *s_acc, const PayoffS
     }
 }
 
-// Four uniforms of Philox block q of stream n (the same map as the normals).
-__device__ __forceinline__ float4 uniforms4(uint64_t q, uint64_t n, const RoundKeys &rk)
+// Four uniforms of Philox block q of a stream (the same map as the normals).
+__device__ __forceinline__ float4 uniforms4(uint32_t q, const PathStream &ps, const RoundKeys &rk)
 {
-    const uint4 x = philox4x32_10(make_uint4(static_cast<uint32_t>(q), static_cast<uint32_t>(q >> 32),
-                                             static_cast<uint32_t>(n), static_cast<uint32_t>(n >> 32)),
-                                  rk);
+    const uint4 x = ps.block(q, rk);
     return make_float4(u01(x.x), u01(x.y), u01(x.z), u01(x.w));
 }
 
@@ -73,13 +71,16 @@ __global__ void __launch_bounds__(kBlock, 8) gbm1d_kernel(const __grid_constant_
             const int64_t save_len = (static_cast<int64_t>(M / a.run.save_every) + 1) * a.run.paths;
             if (SAVE && GBMC_IN_BOUNDS(nl, save_len, kDbgGbm1dSave)) a.run.save[nl] = a.s0;
             const int nq = (M + 3) >> 2;
+            PathStream ps, pb;
+            ps.init(n, a.run.rk);
+            if (BRIDGE) pb.init(kBridgeDomain + n, a.run.rk);
             for (int q = 0; q < nq; ++q) {
-                const float4 z4 = normals4(static_cast<uint64_t>(q), n, a.run.rk);
+                const float4 z4 = ps.normals(static_cast<uint32_t>(q), a.run.rk).f4();
                 const float zz[4] = {z4.x, z4.y, z4.z, z4.w};
                 float4 ub[2];
                 if (BRIDGE) {  // uniforms 8q .. 8q + 7: (max, min) of steps 4q .. 4q + 3
-                    ub[0] = uniforms4(2 * static_cast<uint64_t>(q), kBridgeDomain + n, a.run.rk);
-                    ub[1] = uniforms4(2 * static_cast<uint64_t>(q) + 1, kBridgeDomain + n, a.run.rk);
+                    ub[0] = uniforms4(2 * static_cast<uint32_t>(q), pb, a.run.rk);
+                    ub[1] = uniforms4(2 * static_cast<uint32_t>(q) + 1, pb, a.run.rk);
                 }
 #pragma unroll
                 for (int l = 0; l < 4; ++l) {

@@ -78,9 +78,11 @@ __global__ void __launch_bounds__(kBlock) gbm1d_greeks_kernel(const __grid_const
         float dE[3] = {0.0f, 0.0f, 0.0f}, dA[3] = {0.0f, 0.0f, 0.0f};
         if (valid) {
             const uint64_t n = static_cast<uint64_t>(a.run.path_offset + nl);
+            PathStream ps;
+            ps.init(n, a.run.rk);
             float y = 0.0f, W = 0.0f, sS = 0.0f, sSt = 0.0f, sSW = 0.0f;
             for (int q = 0; q < (M + 3) / 4; ++q) {
-                const float4 z4 = normals4(static_cast<uint64_t>(q), n, a.run.rk);
+                const float4 z4 = ps.normals(static_cast<uint32_t>(q), a.run.rk).f4();
                 const float zz[4] = {z4.x, z4.y, z4.z, z4.w};
 #pragma unroll
                 for (int l = 0; l < 4; ++l) {

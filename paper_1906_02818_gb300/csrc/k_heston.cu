@@ -38,8 +38,10 @@ __global__ void __launch_bounds__(kBlock) heston_kernel(const __grid_constant__ 
                 if (GBMC_IN_BOUNDS(a.run.paths + nl, save_len, kDbgHestonSave)) a.run.save[a.run.paths + nl] = a.v0;
             }
             const int nq = (M + 1) >> 1;
+            PathStream ps;
+            ps.init(n, a.run.rk);
             for (int q = 0; q < nq; ++q) {
-                const float4 z4 = normals4(static_cast<uint64_t>(q), n, a.run.rk);
+                const float4 z4 = ps.normals(static_cast<uint32_t>(q), a.run.rk).f4();
                 const float z1s[2] = {z4.x, z4.z}, z2s[2] = {z4.y, z4.w};
 #pragma unroll
                 for (int l = 0; l < 2; ++l) {

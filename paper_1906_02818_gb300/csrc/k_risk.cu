@@ -63,10 +63,12 @@ __global__ void __launch_bounds__(256) label_kernel(int64_t npts, const float *_
         if (!(sk >= H)) {  // already at or above the barrier on the current date: worthless
             for (int path = threadIdx.x; path < paths; path += blockDim.x) {
                 const uint64_t n = tag(4, (static_cast<uint64_t>(p) << 16) | static_cast<uint64_t>(path));
+                PathStream ps;
+                ps.init(n, rk);
                 float y = 0.0f, zs = 0.0f;
                 bool alive = true;
                 for (int q = 0; q < (M + 3) / 4; ++q) {
-                    const float4 z = normals4(static_cast<uint64_t>(q), n, rk);
+                    const float4 z = ps.normals(static_cast<uint32_t>(q), rk).f4();
                     const float zz[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
                     for (int l = 0; l < 4; ++l) {
@@ -155,10 +157,12 @@ __global__ void __launch_bounds__(256) nested_kernel(const __grid_constant__ Ris
     const uint64_t domain = Sp ? 3 : 5;
     for (int path = threadIdx.x; path < a.inner; path += blockDim.x) {
         const uint64_t n = tag(domain, base_idx | static_cast<uint64_t>(path));
+        PathStream ps;
+        ps.init(n, a.rk);
         float y = 0.0f, mx = -INFINITY;  // log2(S/S1) and its running maximum over the dates
         int jn = 0;                      // next option to mature
         for (int q = 0; q < (maxrem + 3) / 4; ++q) {
-            const float4 z = normals4(static_cast<uint64_t>(q), n, a.rk);
+            const float4 z = ps.normals(static_cast<uint32_t>(q), a.rk).f4();
             const float zz[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
             for (int l = 0; l < 4; ++l) {

@@ -17,9 +17,9 @@ __global__ void __launch_bounds__(256) philox_words_kernel(uint64_t n, uint64_t 
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < blocks; i += stride) {
         const uint64_t q = q0 + static_cast<uint64_t>(i);
-        if (GBMC_IN_BOUNDS(i, blocks, kDbgPhiloxOut)) out[i] = philox4x32_10(make_uint4(static_cast<uint32_t>(q), static_cast<uint32_t>(q >> 32),
-                                          static_cast<uint32_t>(n), static_cast<uint32_t>(n >> 32)),
-                               rk);
+        PathStream ps;
+        ps.init(n, rk, static_cast<uint32_t>(q >> 32));
+        if (GBMC_IN_BOUNDS(i, blocks, kDbgPhiloxOut)) out[i] = ps.block(static_cast<uint32_t>(q), rk);
     }
 }
 
@@ -34,7 +34,9 @@ __global__ void __launch_bounds__(256) normals_kernel(uint64_t n, uint64_t j0, i
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nblk; i += stride) {
         const uint64_t q = qa + static_cast<uint64_t>(i);
-        const float4 z = normals4(q, n, rk);
+        PathStream ps;
+        ps.init(n, rk, static_cast<uint32_t>(q >> 32));
+        const float4 z = ps.normals(static_cast<uint32_t>(q), rk).f4();
         const float v[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
         for (int l = 0; l < 4; ++l) {

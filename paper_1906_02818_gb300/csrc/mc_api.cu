@@ -444,7 +444,7 @@ int big_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const PayoffSe
     BigArgs &b = P->bg;
     b.run = run;
     b.d = d;
-    b.exact4 = d % 4 == 0;
+    b.exact4 = d % 4 == 0 && blocks_fit_32(c->steps, d);
     b.greeks = greeks ? 1 : 0;
     b.bimg = P->bimg;
     b.Lp = P->dLp;
@@ -513,7 +513,7 @@ int factor_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const Payof
     f.k = k;
     f.G = G;
     f.scheme = c->scheme;
-    f.exact4 = (k % 4 == 0 && d % 4 == 0) ? 1 : 0;
+    f.exact4 = (k % 4 == 0 && d % 4 == 0 && blocks_fit_32(c->steps, k + d)) ? 1 : 0;
     f.Bp = P->dcol;
     f.ep = P->dcol + static_cast<size_t>(k) * dp;
     f.drift = f.ep + dp;
@@ -1111,7 +1111,7 @@ static int corr_greeks_wide(const mc_model *m, const mc_sim_cfg *c, const mc_pay
     a.run.steps = c->steps;
     a.run.save_every = 1;
     a.d = d;
-    a.exact4 = d % 4 == 0 ? 1 : 0;
+    a.exact4 = d % 4 == 0 && blocks_fit_32(c->steps, d) ? 1 : 0;
     a.kind = pay->kind;
     a.strike = static_cast<float>(pay->strike);
     // batches of kchunk paths (a multiple of 16) for the batch-means errors
@@ -1234,7 +1234,7 @@ int mc_corr_greeks(const mc_model *m, const mc_sim_cfg *c, const mc_payoff *pay,
     a.run.steps = c->steps;
     a.run.save_every = 1;
     a.d = d;
-    a.exact4 = d % 4 == 0 ? 1 : 0;
+    a.exact4 = d % 4 == 0 && blocks_fit_32(c->steps, d) ? 1 : 0;
     a.kind = pay->kind;
     a.strike = static_cast<float>(pay->strike);
     const int occ = corr_occupancy(a);

@@ -42,6 +42,10 @@ inline void set_seed(PathRun &r, uint64_t seed)
     r.rk = round_keys(r.k0, r.k1);
 }
 
+// Whether the Philox blocks of a path of `steps` steps all have index high
+// word 0 (PathStream's default); runs beyond that read through NormalReader.
+inline bool blocks_fit_32(int64_t steps, int64_t normals_per_step) { return steps * normals_per_step <= (int64_t(1) << 34); }
+
 // Single-asset GBM.  log-Euler: y = log2(S/S0) += a + b z with
 // a = log2(e) (r - sigma^2/2) dt, b = log2(e) sigma sqrt(dt).
 // Euler: S <- S + S (a + b z) with a = r dt, b = sigma sqrt(dt).
