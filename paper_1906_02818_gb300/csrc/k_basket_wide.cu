@@ -1,19 +1,22 @@
-// FP32 contraction for large baskets (64 < d <= 512), the reference
-// precision of the tensor-core kernels: the multivariate Euler step of
-// Sec. II.A.2 for a tile of 64 paths as a register-tiled SIMT product.
+// FP32 large baskets (64 < d <= 512) and the pathwise Greeks of every FP32
+// basket: European payoffs under log-Euler, the multivariate Euler step of
+// Sec. II.A.2 summed over the steps (Segments, mc_device.cuh: the terminal
+// log-prices need the contraction of the summed normals only).
 //   * CTA = 64 paths x D assets (D = 128, 256 or 512, zero-padded), 512
-//     threads; thread (pg, ag) owns paths 4 pg .. 4 pg + 3 and the assets
-//     128 j + 4 ag .. + 3 (j < D / 128): 4 x D / 32 running sums in registers
-//     as asset pairs, acc[p][a] = sum over steps of (Lhat z)_a, Lhat =
-//     log2(e) sqrt(dt) diag(sigma) Lrho, accumulated by packed FP32x2 FMAs
-//     (one instruction for two assets of one path; each lane an FP32 fma).
-//   * per step: the CTA draws the 64 x d normals into shared memory
-//     (z[k][path], consecutive threads on consecutive paths), then streams
-//     Lhat^T in chunks of 16 rows (cp.async double buffer) and accumulates;
-//     128-asset blocks that lie above the chunk (zero in the lower-triangular
+//     threads.  Drawing: thread (path t mod 64, t / 64) sums every eighth
+//     Philox block of its path over the steps, four blocks at a time in
+//     registers, into W[k][path] in shared memory.
+//   * Contraction, once per tile: thread (pg, ag) owns paths 4 pg .. 4 pg + 3
+//     and the assets 128 j + 4 ag .. + 3 (j < D / 128): 4 x D / 32 sums in
+//     registers as asset pairs (packed FP32x2 FMAs, one instruction for two
+//     assets of one path, each lane an FP32 fma), Lhat = log2(e) sqrt(dt)
+//     diag(sigma) Lrho streamed k-major in chunks of 16 rows (cp.async double
+//     buffer); 128-asset blocks above the chunk (zero in the lower-triangular
 //     factor) are skipped.
-//   * at the end of the tile: log2(S_a / S0_a) = M drift_a + acc, the basket,
+//   * Epilogue: log2(S_a / S0_a) = M drift_a + (Lhat W)_a, the basket,
 //     European payoffs and the pathwise delta / vega / rho of payoff 0.
+// Bound by drawing; the contraction, which ran every step before, is 5 % of
+// a tile at d = 512 and 252 steps.
 #include "mc_kernels.cuh"
 
 namespace gbmc {
@@ -22,6 +25,7 @@ namespace {
 constexpr int kP = 64;       // paths per CTA
 constexpr int kThreads = 512;
 constexpr int kKC = 16;      // factor rows per chunk
+constexpr int kDraw = 4;     // Philox blocks a thread sums at a time
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
 {
@@ -51,8 +55,33 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
     for (int i = t; i < (2 * d + 1) * 2; i += kThreads) s_g[i >> 1][i & 1] = 0.0f;
     const int64_t ntiles = (a.run.paths + kP - 1) / kP;
     const int nchunks = (d + kKC - 1) / kKC;
+    const Segments seg(M, d);
+    // rows past d of the last chunk meet zero rows of the factor: finite, and written once
+    for (int i = d * kP + t; i < nchunks * kKC * kP; i += kThreads) zs[i] = 0.0f;
 
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        // drawing: path t % 64, blocks t / 64, t / 64 + 8, ... of each segment
+        const int rp = t & (kP - 1);
+        const uint32_t rq = static_cast<uint32_t>(t) >> 6;
+        const int64_t rnl = tile * kP + rp;
+        const uint64_t rn = static_cast<uint64_t>(a.run.path_offset + (rnl < a.run.paths ? rnl : 0));
+        for (uint32_t p = 0; p < seg.period && seg.count(p) > 0; ++p) {
+            const int o = seg.lane(p);
+            const uint32_t nblk = static_cast<uint32_t>(o + d + 3) >> 2;
+            for (uint32_t g = rq; g < nblk; g += 8 * kDraw) {
+                f32x2 w[2 * kDraw];
+                sum_blocks<kDraw>(w, rn, a.run.rk, a.wide, seg.first_block(p) + g, 8, seg.count(p), seg.blocks, NoRounding{});
+#pragma unroll
+                for (int e = 0; e < 4 * kDraw; ++e) {
+                    const int k = static_cast<int>(4 * (g + 8 * (e >> 2))) + (e & 3) - o;
+                    if (k >= 0 && k < d) {
+                        const float v = (e & 1) ? hi_of(w[e >> 1]) : lo_of(w[e >> 1]);
+                        zs[k * kP + rp] = p == 0 ? v : zs[k * kP + rp] + v;
+                    }
+                }
+            }
+            if (p + 1 < seg.period) __syncthreads();  // a column's sums of two segments lie with different threads
+        }
         f32x2 acc2[4][J][2];  // [path][asset group][asset pair]
 #pragma unroll
         for (int p = 0; p < 4; ++p)
@@ -60,66 +89,36 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
             for (int j = 0; j < J; ++j)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) acc2[p][j][e] = pack2(0.0f, 0.0f);
-        // RNG mapping: path t % 64, normals [q*D/8, (q+1)*D/8) with q = t / 64
-        const int rp = t & (kP - 1), rq = t >> 6;
-        const int64_t rnl = tile * kP + rp;
-        const bool rvalid = rnl < a.run.paths;
-        const uint64_t rn = static_cast<uint64_t>(a.run.path_offset + (rvalid ? rnl : 0));
-        NormalReader rd;
-        rd.init(rn, a.run.rk);
-        PathStream ps;
-        ps.init(rn, a.run.rk);
-        for (int i = 0; i < M; ++i) {
-            __syncthreads();  // previous step done with zs
-            for (int k = rq * (D / 8); k < (rq + 1) * (D / 8); k += 4) {
-                float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (rvalid && k < d) {
-                    if (a.exact4) {
-                        z = ps.normals((static_cast<uint32_t>(i) * (d >> 2)) + (k >> 2), a.run.rk).f4();
-                    } else {
-                        const uint64_t j0 = static_cast<uint64_t>(i) * d + k;
-                        z.x = rd.get(j0);
-                        z.y = k + 1 < d ? rd.get(j0 + 1) : 0.f;
-                        z.z = k + 2 < d ? rd.get(j0 + 2) : 0.f;
-                        z.w = k + 3 < d ? rd.get(j0 + 3) : 0.f;
-                    }
-                }
-                zs[(k + 0) * kP + rp] = z.x;
-                zs[(k + 1) * kP + rp] = z.y;
-                zs[(k + 2) * kP + rp] = z.z;
-                zs[(k + 3) * kP + rp] = z.w;
+        // first factor chunk
+        for (int e = t * 4; e < kKC * D; e += kThreads * 4) cp_async16(Ls + e, a.Lp + e);
+        cp_async_commit();
+        for (int c = 0; c < nchunks; ++c) {
+            cp_async_wait_all();
+            __syncthreads();  // chunk c (and, at c = 0, the summed normals) visible
+            const float *Lc = Ls + (c & 1) * kKC * D;
+            if (c + 1 < nchunks) {  // prefetch the next chunk into the other buffer
+                float *dst = Ls + ((c + 1) & 1) * kKC * D;
+                const float *src = a.Lp + static_cast<size_t>(c + 1) * kKC * D;
+                for (int e = t * 4; e < kKC * D; e += kThreads * 4) cp_async16(dst + e, src + e);
+                cp_async_commit();
             }
-            // first factor chunk
-            for (int e = t * 4; e < kKC * D; e += kThreads * 4) cp_async16(Ls + e, a.Lp + e);
-            cp_async_commit();
-            for (int c = 0; c < nchunks; ++c) {
-                cp_async_wait_all();
-                __syncthreads();  // chunk c (and, at c = 0, the normals) visible
-                const float *Lc = Ls + (c & 1) * kKC * D;
-                if (c + 1 < nchunks) {  // prefetch the next chunk into the other buffer
-                    float *dst = Ls + ((c + 1) & 1) * kKC * D;
-                    const float *src = a.Lp + static_cast<size_t>(c + 1) * kKC * D;
-                    for (int e = t * 4; e < kKC * D; e += kThreads * 4) cp_async16(dst + e, src + e);
-                    cp_async_commit();
-                }
-                const int k0 = c * kKC;
+            const int k0 = c * kKC;
 #pragma unroll 4
-                for (int kk = 0; kk < kKC; ++kk) {
-                    const float4 zv = *reinterpret_cast<const float4 *>(zs + (k0 + kk) * kP + 4 * pg);
-                    const f32x2 zz[4] = {pack2(zv.x, zv.x), pack2(zv.y, zv.y), pack2(zv.z, zv.z), pack2(zv.w, zv.w)};
+            for (int kk = 0; kk < kKC; ++kk) {
+                const float4 zv = *reinterpret_cast<const float4 *>(zs + (k0 + kk) * kP + 4 * pg);
+                const f32x2 zz[4] = {pack2(zv.x, zv.x), pack2(zv.y, zv.y), pack2(zv.z, zv.z), pack2(zv.w, zv.w)};
 #pragma unroll
-                    for (int j = 0; j < J; ++j) {
-                        if (128 * j + 127 < k0) continue;  // block above the diagonal chunk: zero
-                        const ulonglong2 lv = *reinterpret_cast<const ulonglong2 *>(Lc + kk * D + 128 * j + 4 * ag);
+                for (int j = 0; j < J; ++j) {
+                    if (128 * j + 127 < k0) continue;  // block above the diagonal chunk: zero
+                    const ulonglong2 lv = *reinterpret_cast<const ulonglong2 *>(Lc + kk * D + 128 * j + 4 * ag);
 #pragma unroll
-                        for (int p = 0; p < 4; ++p) {
-                            acc2[p][j][0] = ffma2(lv.x, zz[p], acc2[p][j][0]);
-                            acc2[p][j][1] = ffma2(lv.y, zz[p], acc2[p][j][1]);
-                        }
+                    for (int p = 0; p < 4; ++p) {
+                        acc2[p][j][0] = ffma2(lv.x, zz[p], acc2[p][j][0]);
+                        acc2[p][j][1] = ffma2(lv.y, zz[p], acc2[p][j][1]);
                     }
                 }
-                __syncthreads();  // everyone done with chunk c before it is overwritten
             }
+            __syncthreads();  // everyone done with chunk c before it is overwritten
         }
         // ---- epilogue ----
         float Ux[4] = {0.f, 0.f, 0.f, 0.f};

@@ -445,6 +445,7 @@ int big_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const PayoffSe
     b.run = run;
     b.d = d;
     b.exact4 = d % 4 == 0 && blocks_fit_32(c->steps, d);
+    b.wide = !blocks_fit_32(c->steps, d);
     b.greeks = greeks ? 1 : 0;
     b.bimg = P->bimg;
     b.Lp = P->dLp;

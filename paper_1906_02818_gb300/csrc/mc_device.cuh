@@ -240,6 +240,75 @@ struct NormalReader {
 };
 
 // ---------------------------------------------------------------------------
+// Summed normals.  Under log-Euler with constant coefficients the terminal
+// log-prices of a basket depend on a path's normals only through
+// W_k = sum_i z_{i d + k}, so payoffs on the terminal value alone need one
+// contraction per path, of W, instead of one per step.  Steps that share
+// their position inside a Philox block (all of them when 4 | d, every second
+// or fourth otherwise) form a segment: the same blocks of each, added up in
+// registers without a select, so that a step of any width costs its blocks.
+// ---------------------------------------------------------------------------
+struct Segments {
+    uint32_t period;  // steps until a step starts again at the same place of a block: 1, 2 or 4
+    uint32_t blocks;  // Philox blocks of `period` steps
+    int steps, d;
+
+    __device__ __forceinline__ Segments(int steps_, int d_)
+        : period((d_ & 3) == 0 ? 1u : (d_ & 1) == 0 ? 2u : 4u), blocks(period * static_cast<uint32_t>(d_) / 4u), steps(steps_),
+          d(d_)
+    {
+    }
+    // Segment p: the steps p, p + period, ...; their first normal is lane `lane` of their first block `block`.
+    __device__ __forceinline__ int count(uint32_t p) const
+    {
+        return static_cast<int>((static_cast<uint32_t>(steps) + period - 1u - p) / period);
+    }
+    __device__ __forceinline__ uint32_t first_block(uint32_t p) const { return p * static_cast<uint32_t>(d) >> 2; }
+    __device__ __forceinline__ int lane(uint32_t p) const { return static_cast<int>(p * static_cast<uint32_t>(d) & 3u); }
+};
+
+// w = the sums over `count` steps, `blocks` Philox blocks apart, of the
+// normals of blocks b, b + stride, ... (NB of them) of stream n, each normal
+// passed through `round` (the operand rounding of the reduced precisions).
+// wide: a block index may pass 2^32.
+struct NoRounding {
+    __device__ __forceinline__ f32x2 operator()(f32x2 z) const { return z; }
+};
+template <int NB, class Round>
+__device__ __forceinline__ void sum_blocks(f32x2 (&w)[2 * NB], uint64_t n, const RoundKeys &rk, bool wide, uint64_t b,
+                                           uint32_t stride, int count, uint32_t blocks, const Round &round)
+{
+#pragma unroll
+    for (int j = 0; j < 2 * NB; ++j) w[j] = pack2(0.0f, 0.0f);
+    if (!wide) {
+        PathStream ps;
+        ps.init(n, rk);
+        uint32_t q = static_cast<uint32_t>(b);
+        for (int s = 0; s < count; ++s, q += blocks)
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                const Normals4 z = ps.normals(q + stride * j, rk);
+                w[2 * j] = fadd2(w[2 * j], round(z.a));
+                w[2 * j + 1] = fadd2(w[2 * j + 1], round(z.b));
+            }
+    } else {
+        for (int s = 0; s < count; ++s)
+#pragma unroll 1
+            for (int j = 0; j < NB; ++j) {
+                const float4 z = normals4(static_cast<uint64_t>(s) * blocks + b + stride * j, n, rk);
+                const f32x2 za = round(pack2(z.x, z.y)), zb = round(pack2(z.z, z.w));
+#pragma unroll
+                for (int k = 0; k < NB; ++k) {
+                    if (k == j) {
+                        w[2 * k] = fadd2(w[2 * k], za);
+                        w[2 * k + 1] = fadd2(w[2 * k + 1], zb);
+                    }
+                }
+            }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Payoffs (undiscounted) on the monitored statistics of U.
 // ---------------------------------------------------------------------------
 struct PayoffSet {

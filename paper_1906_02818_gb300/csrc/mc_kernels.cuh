@@ -127,6 +127,7 @@ struct BigArgs {
     PathRun run;
     int d;
     int exact4;             // d % 4 == 0: each 16-normal group is 4 whole Philox blocks
+    bool wide;              // a path's Philox blocks pass 2^32
     int greeks;
     const uint8_t *bimg;    // tensor cores: pre-swizzled factor chunks
     const float *Lp;        // FP32: k-major dense log2(e) sqrt(dt) diag(sigma) Lrho, [D x D]
