@@ -240,12 +240,17 @@ int mc_risk(const mc_portfolio *pf, const mc_risk_cfg *cf, mc_risk_result *res, 
     a.rk = rk;
     a.scen_off = cf->scen_offset;
     if (cf->method == MC_RISK_NESTED) {
-        double *d_contrib;
+        double *d_contrib, *d_part;
+        int dev = 0, sms = 0;
+        RK_CUDA(cudaGetDevice(&dev));
+        RK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const int bsl = nested_slices(d, cf->base_paths, sms), isl = nested_slices(ns * d, cf->inner_paths, sms);
         RK_CUDA(B.alloc(&d_contrib, ns * d));
+        RK_CUDA(B.alloc(&d_part, std::max(nested_part_doubles(d, bsl), nested_part_doubles(ns * d, isl))));
         a.inner = cf->base_paths;
-        RK_CUDA(launch_nested(a, 1, nullptr, nullptr, s));  // base values at S0, full maturities
+        RK_CUDA(launch_nested(a, 1, nullptr, nullptr, d_part, bsl, s));  // base values at S0, full maturities
         a.inner = cf->inner_paths;
-        RK_CUDA(launch_nested(a, ns, d_Sp, d_contrib, s));
+        RK_CUDA(launch_nested(a, ns, d_Sp, d_contrib, d_part, isl, s));
         RK_CUDA(launch_sum_under(ns, d, d_contrib, d_pnl, s));
     } else {
         mc_mlp *net = cf->surrogate;

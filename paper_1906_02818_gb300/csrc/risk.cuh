@@ -33,7 +33,12 @@ cudaError_t launch_labels(int64_t npts, const float *pts, int paths, float steps
                           float *labels, float *inputs, float *dlabels, cudaStream_t s);
 cudaError_t launch_outer(int64_t nscen, int64_t off, int d, const float *Lc, const float *drift, const float *s0,
                          const RoundKeys &rk, float *Sp, cudaStream_t s);
-cudaError_t launch_nested(const RiskArgs &a, int64_t nscen, const float *Sp, double *contrib, cudaStream_t s);
+// Inner paths of nscen scenarios (Sp == nullptr: the base date) in `slices`
+// CTAs per (scenario, underlying); part: nested_part_doubles scratch.
+int nested_slices(int64_t pairs, int inner, int sms);
+size_t nested_part_doubles(int64_t pairs, int slices);
+cudaError_t launch_nested(const RiskArgs &a, int64_t nscen, const float *Sp, double *contrib, double *part, int slices,
+                          cudaStream_t s);
 cudaError_t launch_sum_under(int64_t nscen, int d, const double *contrib, double *pnl, cudaStream_t s);
 cudaError_t launch_features(const RiskArgs &a, int64_t nscen, const float *Sp, float *x, cudaStream_t s);
 cudaError_t launch_pnl(const RiskArgs &a, int64_t nscen, const float *Sp, const float *y, double *pnl, cudaStream_t s);
