@@ -42,10 +42,9 @@ constexpr uint64_t kBridgeDomain = uint64_t(1) << 56;  // stream of path n's bri
 // yp, y of log2(S/S0) the maximum of the Brownian bridge is drawn as
 // (yp + y + sqrt((y - yp)^2 - cb lg2 U)) / 2 with cb = 2 dt sigma^2 log2(e)
 // (Sec. VI.A.1; the formula in log2 units) and the minimum with the root
-// subtracted; U = uniforms 2i and 2i + 1 of the bridge stream.  Eight
-// blocks per SM (32 registers, an 8-byte spill): left free, the compiler
-// takes 48 registers, 5 blocks fit, and the 2^20 x 64 call runs 76.3 us
-// instead of 73.8 us.
+// subtracted; U = uniforms 2i and 2i + 1 of the bridge stream.  Bound by
+// drawing; a European payoff under log-Euler only adds its path's normals up,
+// and no step is tested against M but in the last block.  Eight blocks per SM.
 template <int SCHEME, bool STATS, bool SAVE, bool BRIDGE>
 __global__ void __launch_bounds__(kBlock, 8) gbm1d_kernel(const __grid_constant__ Gbm1dArgs a)
 {
@@ -70,44 +69,58 @@ __global__ void __launch_bounds__(kBlock, 8) gbm1d_kernel(const __grid_constant_
             float bmax = 0.0f, bmin = 0.0f;                    // bridge extremes of y
             const int64_t save_len = (static_cast<int64_t>(M / a.run.save_every) + 1) * a.run.paths;
             if (SAVE && GBMC_IN_BOUNDS(nl, save_len, kDbgGbm1dSave)) a.run.save[nl] = a.s0;
-            const int nq = (M + 3) >> 2;
+            const int nq = M >> 2, rest = M & 3;  // whole Philox blocks, normals of the last one
             PathStream ps, pb;
             ps.init(n, a.run.rk);
             if (BRIDGE) pb.init(kBridgeDomain + n, a.run.rk);
-            for (int q = 0; q < nq; ++q) {
-                const float4 z4 = ps.normals(static_cast<uint32_t>(q), a.run.rk).f4();
-                const float zz[4] = {z4.x, z4.y, z4.z, z4.w};
-                float4 ub[2];
-                if (BRIDGE) {  // uniforms 8q .. 8q + 7: (max, min) of steps 4q .. 4q + 3
-                    ub[0] = uniforms4(2 * static_cast<uint32_t>(q), pb, a.run.rk);
-                    ub[1] = uniforms4(2 * static_cast<uint32_t>(q) + 1, pb, a.run.rk);
+            if (SCHEME == MC_LOG_EULER && !STATS && !SAVE) {
+                // European: the terminal price depends on the normals' sum alone
+                f32x2 w = pack2(0.0f, 0.0f);
+                for (int q = 0; q < nq; ++q) {
+                    const Normals4 z = ps.normals(static_cast<uint32_t>(q), a.run.rk);
+                    w = fadd2(w, fadd2(z.a, z.b));
                 }
-#pragma unroll
-                for (int l = 0; l < 4; ++l) {
-                    const int i = 4 * q + l;
-                    if (i < M) {
-                        const float yp = y;
-                        if (SCHEME == MC_LOG_EULER) y += fmaf(a.b, zz[l], a.a);
-                        else y = fmaf(y, fmaf(a.b, zz[l], a.a), y);
-                        if (BRIDGE) {
-                            const float4 u = ub[l >> 1];
-                            const float umx = (l & 1) ? u.z : u.x, umn = (l & 1) ? u.w : u.y;
-                            const float dy = y - yp, d2 = dy * dy;
-                            const float rmax = sqrt_approx(fmaf(-a.cb, lg2_approx(umx), d2));
-                            const float rmin = sqrt_approx(fmaf(-a.cb, lg2_approx(umn), d2));
-                            bmax = fmaxf(bmax, 0.5f * (yp + y + rmax));
-                            bmin = fminf(bmin, 0.5f * (yp + y - rmin));
-                        }
-                        if (STATS || SAVE) {
-                            const float S = (SCHEME == MC_LOG_EULER) ? a.s0 * ex2_approx(y) : y;
-                            if (STATS) st.add(S);
-                            if (SAVE && ((i + 1) % a.run.save_every) == 0) {
-                                const int64_t o = static_cast<int64_t>((i + 1) / a.run.save_every) * a.run.paths + nl;
-                                if (GBMC_IN_BOUNDS(o, save_len, kDbgGbm1dSave)) a.run.save[o] = S;
-                            }
+                if (rest) {
+                    const Normals4 z = ps.normals(static_cast<uint32_t>(nq), a.run.rk);
+                    w = fadd2(w, pack2(lo_of(z.a) + (rest > 2 ? lo_of(z.b) : 0.0f), rest > 1 ? hi_of(z.a) : 0.0f));
+                }
+                y = fmaf(a.b, lo_of(w) + hi_of(w), static_cast<float>(M) * a.a);
+            } else {
+                auto step = [&](int i, float z, float umx, float umn) {
+                    const float yp = y;
+                    if (SCHEME == MC_LOG_EULER) y += fmaf(a.b, z, a.a);
+                    else y = fmaf(y, fmaf(a.b, z, a.a), y);
+                    if (BRIDGE) {
+                        const float dy = y - yp, d2 = dy * dy;
+                        const float rmax = sqrt_approx(fmaf(-a.cb, lg2_approx(umx), d2));
+                        const float rmin = sqrt_approx(fmaf(-a.cb, lg2_approx(umn), d2));
+                        bmax = fmaxf(bmax, 0.5f * (yp + y + rmax));
+                        bmin = fminf(bmin, 0.5f * (yp + y - rmin));
+                    }
+                    if (STATS || SAVE) {
+                        const float S = (SCHEME == MC_LOG_EULER) ? a.s0 * ex2_approx(y) : y;
+                        if (STATS) st.add(S);
+                        if (SAVE && ((i + 1) % a.run.save_every) == 0) {
+                            const int64_t o = static_cast<int64_t>((i + 1) / a.run.save_every) * a.run.paths + nl;
+                            if (GBMC_IN_BOUNDS(o, save_len, kDbgGbm1dSave)) a.run.save[o] = S;
                         }
                     }
-                }
+                };
+                // block q: steps 4q .. 4q + cnt - 1; bridge uniforms 8q .. 8q + 7: (max, min) of each
+                auto block = [&](int q, int cnt) {
+                    const float4 z = ps.normals(static_cast<uint32_t>(q), a.run.rk).f4();
+                    float4 u0 = make_float4(1.0f, 1.0f, 1.0f, 1.0f), u1 = u0;
+                    if (BRIDGE) {
+                        u0 = uniforms4(2 * static_cast<uint32_t>(q), pb, a.run.rk);
+                        u1 = uniforms4(2 * static_cast<uint32_t>(q) + 1, pb, a.run.rk);
+                    }
+                    step(4 * q, z.x, u0.x, u0.y);
+                    if (cnt > 1) step(4 * q + 1, z.y, u0.z, u0.w);
+                    if (cnt > 2) step(4 * q + 2, z.z, u1.x, u1.y);
+                    if (cnt > 3) step(4 * q + 3, z.w, u1.z, u1.w);
+                };
+                for (int q = 0; q < nq; ++q) block(q, 4);
+                if (rest) block(nq, rest);
             }
             uT = (SCHEME == MC_LOG_EULER) ? a.s0 * ex2_approx(y) : y;
             avg = st.sum * inv_m;
@@ -153,7 +166,11 @@ const void *basket_select(int D, const BasketArgs &a)
     case 4: return basket_select_d<4>(a);
     case 8: return basket_select_d<8>(a);
     case 16: return basket_select_d<16>(a);
+    case 24: return basket_select_d<24>(a);
     case 32: return basket_select_d<32>(a);
+    case 40: return basket_select_d<40>(a);
+    case 48: return basket_select_d<48>(a);
+    case 56: return basket_select_d<56>(a);
     case 64: return basket_select_d<64>(a);
     default: return nullptr;
     }
@@ -176,11 +193,19 @@ cudaError_t launch_gbm1d(const Gbm1dArgs &a, int grid, int block, cudaStream_t s
 
 int gbm1d_occupancy(const Gbm1dArgs &a, int block) { return occupancy_of(gbm1d_select(a), block); }
 
-int basket_fp32_width(int d)
+// Widths every eight assets from 16 up: a contraction padded from 50 assets to
+// 64 runs 2080 products for 1275 (56: 1596).
+int basket_fp32_width(int d, bool wide)
 {
-    for (int D : {4, 8, 16, 32, 64})
+    if (wide) return d <= 64 ? 64 : 0;
+    for (int D : {4, 8, 16, 24, 32, 40, 48, 56, 64})
         if (d <= D) return D;
     return 0;
+}
+
+bool basket_fp32_sums(const BasketArgs &a)
+{
+    return a.scheme == MC_LOG_EULER && !a.run.save && !a.pay.need_avg && !a.pay.need_max && !a.pay.need_min;
 }
 
 size_t basket_const_bytes(int D)
@@ -189,7 +214,11 @@ size_t basket_const_bytes(int D)
     case 4: return sizeof(BasketConst<4>);
     case 8: return sizeof(BasketConst<8>);
     case 16: return sizeof(BasketConst<16>);
+    case 24: return sizeof(BasketConst<24>);
     case 32: return sizeof(BasketConst<32>);
+    case 40: return sizeof(BasketConst<40>);
+    case 48: return sizeof(BasketConst<48>);
+    case 56: return sizeof(BasketConst<56>);
     case 64: return sizeof(BasketConst<64>);
     default: return 0;
     }
@@ -211,7 +240,11 @@ void basket_const_offsets(int D, size_t *L, size_t *drift, size_t *ws0, size_t *
     case 4: offsets_of<4>(L, drift, ws0, w, s0); break;
     case 8: offsets_of<8>(L, drift, ws0, w, s0); break;
     case 16: offsets_of<16>(L, drift, ws0, w, s0); break;
+    case 24: offsets_of<24>(L, drift, ws0, w, s0); break;
     case 32: offsets_of<32>(L, drift, ws0, w, s0); break;
+    case 40: offsets_of<40>(L, drift, ws0, w, s0); break;
+    case 48: offsets_of<48>(L, drift, ws0, w, s0); break;
+    case 56: offsets_of<56>(L, drift, ws0, w, s0); break;
     default: offsets_of<64>(L, drift, ws0, w, s0); break;
     }
 }

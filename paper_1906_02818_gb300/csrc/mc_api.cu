@@ -626,7 +626,8 @@ int plan_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const mc_payo
         const bool tcpath = c->precision != MC_FP32;
         if (tcpath && save)
             return fail(MC_EUNSUPPORTED, "paths are materialised by the FP32 contraction only");
-        const int D = tcpath ? 64 : basket_fp32_width(d);
+        const bool wide = !blocks_fit_32(c->steps, d);
+        const int D = tcpath ? 64 : basket_fp32_width(d, wide);
         if (!D) return fail(MC_EUNSUPPORTED, "FP32 contraction supports d <= 64 (got %d)", d);
         P->D = D;
         const size_t dd = static_cast<size_t>(d) * d;
@@ -690,15 +691,32 @@ int plan_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const mc_payo
             resident = basket_tc_occupancy(P->prec, ta) * di.sms;
         } else {
             P->kk = K_BASKET_FP32;
-            // Large runs: one block per SM, as many rounds of paths as 640
-            // threads need, the block trimmed (to whole warps) so that those
-            // rounds cover the paths on every SM; small runs (or a trimmed
-            // block under 16 warps): blocks of 128, 5 per SM, to spread them.
-            const int64_t per_round = static_cast<int64_t>(640) * di.sms;
-            const int64_t rounds = (c->paths + per_round - 1) / per_round;
-            const int64_t per_sm = (c->paths + rounds * di.sms - 1) / (rounds * di.sms);
-            const int trimmed = static_cast<int>(std::min<int64_t>(640, (per_sm + 31) / 32 * 32));
-            P->block = (c->paths >= 2 * per_round || trimmed >= 512) && c->paths >= per_round ? trimmed : 128;
+            BasketArgs &b = P->bk;
+            b.run = run;
+            b.d = d;
+            b.scheme = c->scheme;
+            b.wide = wide;
+            b.pay = ps;
+            b.red = red;
+            // The stepping kernel: one block per SM, as large (in whole warps)
+            // as an equal share of each round of paths asks for: two paths per
+            // thread where the width allows it and an SM has more than 256,
+            // else one, of up to 640 threads.  Runs of less than a round, or
+            // of so few paths that the block would fall under 16 warps: blocks
+            // of 128, to spread them.
+            const int64_t per_sm = (c->paths + di.sms - 1) / di.sms;
+            const int most = wide || save ? 0 : basket_threads2(D);
+            if (basket_fp32_sums(b)) {
+                P->block = kBasketSumBlock;
+            } else if (most > 0 && per_sm > 256) {
+                b.two = true;
+                const int64_t rounds = (per_sm + 2 * most - 1) / (2 * most);
+                P->block = static_cast<int>((per_sm + 2 * rounds - 1) / (2 * rounds) + 31) / 32 * 32;
+            } else {
+                const int64_t rounds = (per_sm + 639) / 640;
+                const int trimmed = static_cast<int>(((per_sm + rounds - 1) / rounds + 31) / 32 * 32);
+                P->block = (per_sm >= 1280 || trimmed >= 512) && per_sm >= 640 ? trimmed : 128;
+            }
             MC_CUDA(launch_scale_factor(d, P->dL, P->dsig, cfac, sdt, m->r, dt, c->scheme, P->dLp, P->ddrift, s));
             std::vector<float> Lp(tri), drift(d);
             MC_CUDA(cudaMemcpyAsync(&status, P->dstatus, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -729,12 +747,6 @@ int plan_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const mc_payo
                 cW[a] = static_cast<float>(w);
                 cS[a] = static_cast<float>(m->s0[a]);
             }
-            BasketArgs &b = P->bk;
-            b.run = run;
-            b.d = d;
-            b.scheme = c->scheme;
-            b.pay = ps;
-            b.red = red;
             resident = basket_fp32_occupancy(D, b, P->block) * di.sms;
         }
     }
@@ -745,6 +757,10 @@ int plan_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const mc_payo
         P->grid = static_cast<int>(tiles < resident ? tiles : resident);
     } else {
         size_grid(c->paths, P->block, resident, &P->grid, &ppt);
+        if (P->kk == K_BASKET_FP32 && P->bk.two) {  // whole rounds of two paths per thread, on every SM
+            P->grid = static_cast<int>(std::min<int64_t>(di.sms, (c->paths + P->block - 1) / P->block));
+            ppt = static_cast<int>((c->paths + static_cast<int64_t>(P->grid) * P->block - 1) / (static_cast<int64_t>(P->grid) * P->block));
+        }
     }
     P->g1.run.ppt = ppt;
     P->bk.run.ppt = ppt;

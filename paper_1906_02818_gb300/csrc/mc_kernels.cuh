@@ -81,10 +81,17 @@ struct BasketConst {
     float s0[D];
 };
 
+constexpr int kBasketSumBlock = 128;   // block of the summed-normals kernel
+// The largest block of two paths per thread: what the registers of D assets of
+// state leave (0: one path per thread only; at 64 assets two would leave an SM
+// eight warps: 9.5 ms against 8.1 ms for 2^18 paths x 252 steps).
+__host__ __device__ constexpr int basket_threads2(int D) { return D > 56 ? 0 : D > 40 ? 352 : D > 32 ? 384 : 512; }
 struct BasketArgs {
     PathRun run;
     int d;
     int scheme;
+    bool wide;  // a path's Philox blocks pass 2^32
+    bool two;   // two paths per thread
     PayoffSet pay;
     ReduceArgs red;
 };
@@ -337,7 +344,8 @@ int gbm1d_occupancy(const Gbm1dArgs &a, int block);
 cudaError_t launch_basket_fp32(int D, const BasketArgs &a, const void *cst, int grid, int block,
                                cudaStream_t s);
 int basket_fp32_occupancy(int D, const BasketArgs &a, int block);
-int basket_fp32_width(int d);        // smallest instantiated D >= d (0 if none)
+int basket_fp32_width(int d, bool wide);  // smallest instantiated D >= d (0 if none); wide: the one that takes such runs
+bool basket_fp32_sums(const BasketArgs &a);  // the summed-normals kernel takes it
 size_t basket_const_bytes(int D);    // sizeof(BasketConst<D>)
 void basket_const_offsets(int D, size_t *L, size_t *drift, size_t *ws0, size_t *w, size_t *s0);
 
