@@ -114,7 +114,7 @@ typedef struct {
     int64_t path_offset;   /* global index of the first path (for sharding / resume) */
     uint64_t seed;         /* Philox key */
     int32_t precision;     /* mc_precision of the correlation contraction */
-    int32_t ckpt_every;    /* adjoint checkpoint stride in steps (0 = 32) */
+    int32_t ckpt_every;    /* adjoint checkpoint stride in steps (0: the library chooses) */
     int32_t monitoring;    /* mc_monitoring of the barrier payoffs */
 } mc_sim_cfg;
 
@@ -228,7 +228,8 @@ int32_t mc_greek_count(const mc_model *model);
  * simulation, Sec. VI.A.2), with their standard errors, on the same paths as
  * the prices.  d/dr includes the -T * price term of the discount factor.
  *   MC_HESTON: reverse-mode adjoint kernel; the path state is checkpointed
- *     every cfg->ckpt_every steps (0 = 32, at most 64) in device scratch and
+ *     every cfg->ckpt_every steps (0: 8, or 32 where checkpoints of 8 would
+ *     pass 1 GiB; at most 64) in device scratch and
  *     each segment is recomputed from its checkpoint during the backward
  *     sweep.  d sqrt(v+)/dv is taken as 0 where v <= 0.
  *   MC_GBM, d == 1: MC_LOG_EULER (the adjoint of log S is constant along

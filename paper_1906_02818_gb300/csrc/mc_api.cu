@@ -1033,8 +1033,8 @@ int mc_greeks(const mc_model *m, const mc_sim_cfg *c, const mc_payoff *pays, int
     }
     if (m->kind == MC_GBM && c->scheme != MC_LOG_EULER)
         return fail(MC_EUNSUPPORTED, "GBM Greeks are computed for the log-Euler scheme");
-    const int K = c->ckpt_every ? c->ckpt_every : 32;
-    if (m->kind == MC_HESTON && (K < 1 || K > 64)) return fail(MC_EINVAL, "ckpt_every = %d outside [1, 64]", K);
+    int K = c->ckpt_every;
+    if (m->kind == MC_HESTON && K > 64) return fail(MC_EINVAL, "ckpt_every = %d outside [1, 64]", K);
     const int G = mc_greek_count(m);
     const int nv = np * (G + 1);
     if (nv * 2 * 4 * static_cast<int>(sizeof(AccSlot)) > 48 * 1024) return fail(MC_EINVAL, "too many payoffs for one Greeks launch");
@@ -1069,13 +1069,15 @@ int mc_greeks(const mc_model *m, const mc_sim_cfg *c, const mc_payoff *pays, int
         a.xi = static_cast<float>(m->xi);
         a.rho = static_cast<float>(m->rho);
         a.rhoc = static_cast<float>(std::sqrt(1.0 - m->rho * m->rho));
-        a.K = K;
     }
     a.pay = ps;
     const int block = greeks_block();
-    const int occ = greeks_occupancy(a.model, np);
-    if (occ <= 0) return fail(MC_ECUDA, "Greeks kernel cannot be resident");
     int grid = 0, ppt = 1;
+    if (m->kind == MC_HESTON && K == 0)
+        K = heston_stride(c->steps, std::min<int64_t>((c->paths + block - 1) / block, int64_t(16) * di.sms) * block);
+    a.K = K;
+    const int occ = greeks_occupancy(a.model, K, np);
+    if (occ <= 0) return fail(MC_ECUDA, "Greeks kernel cannot be resident");
     size_grid(c->paths, block, occ * di.sms, &grid, &ppt);
     a.run.ppt = ppt;
 

@@ -403,6 +403,34 @@ __device__ __forceinline__ void warp_accumulate(AccSlot *s_acc, int np, int p, f
     }
 }
 
+// The same for eight values at a time (v[j] to p0 + j < np): the sixteen sums
+// (values and squares) share one exchange tree, in which a lane hands over the
+// half of its values that it does not go on with, 16 shuffles instead of 80;
+// every sum adds the lanes in the order of warp_sum, so the bits are the same,
+// and the slots are updated by sixteen lanes at once.
+__device__ __forceinline__ void warp_accumulate8(AccSlot *s_acc, int np, int p0, const float (&v)[8])
+{
+    const int lane = threadIdx.x & 31;
+    float a[16];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        a[2 * j] = v[j];
+        a[2 * j + 1] = v[j] * v[j];
+    }
+#pragma unroll
+    for (int h = 8, o = 16; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int j = 0; j < h; ++j) {
+            const float keep = up ? a[j + h] : a[j], give = up ? a[j] : a[j + h];
+            a[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+    const int e = lane >> 1, p = p0 + (e >> 1);  // this lane pair's sum
+    if ((lane & 1) == 0 && p < np) s_acc[((threadIdx.x >> 5) * np + p) * 2 + (e & 1)] += static_cast<double>(a[0]);
+}
+
 // Called by every thread of the block after its last path.  s_acc holds
 // nwarps*np*2 slots; s_red is scratch for 32 doubles.
 __device__ inline void block_finish(AccSlot *s_acc, double *s_red, int np, const ReduceArgs &ra)

@@ -176,7 +176,8 @@ struct GreeksArgs {
     ReduceArgs red;     // n_payoff * (1 + G) values per path
 };
 cudaError_t launch_greeks(const GreeksArgs &a, int grid, cudaStream_t s);
-int greeks_occupancy(int model, int n_payoff);
+int greeks_occupancy(int model, int K, int n_payoff);
+int heston_stride(int steps, int64_t threads);
 int greeks_block();
 
 // Correction level of the two-level precision estimator (k_mlmc.cu): d <= 64
