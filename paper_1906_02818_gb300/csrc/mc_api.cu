@@ -247,6 +247,46 @@ void dev_free_raw(void *p)
     g_live_blocks.erase(it);
 }
 
+// Pinned blocks in which a pricing kernel leaves its results for the host: a
+// synchronising call then waits for its kernel alone, not for a copy behind
+// it.  At most kHostBlocks idle ones are kept; mc_release_cache frees them.
+struct HostBlock {
+    mc_result res[MC_MAX_PAYOFFS];
+};
+constexpr size_t kHostBlocks = 16;
+std::vector<HostBlock *> g_host_blocks;  // guarded by g_cache_mu
+
+HostBlock *host_block_take()
+{
+    {
+        std::lock_guard<std::mutex> g(g_cache_mu);
+        if (!g_host_blocks.empty()) {
+            HostBlock *b = g_host_blocks.back();
+            g_host_blocks.pop_back();
+            return b;
+        }
+    }
+    void *p = nullptr;
+    if (cudaHostAlloc(&p, sizeof(HostBlock), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;  // the caller falls back to a copy
+    }
+    return static_cast<HostBlock *>(p);
+}
+
+void host_block_give(HostBlock *b)  // no launch may still write it
+{
+    if (!b) return;
+    {
+        std::lock_guard<std::mutex> g(g_cache_mu);
+        if (g_host_blocks.size() < kHostBlocks) {
+            g_host_blocks.push_back(b);
+            return;
+        }
+    }
+    cudaFreeHost(b);
+}
+
 template <class T>
 cudaError_t dev_alloc(T **p, size_t n)
 {
@@ -337,6 +377,9 @@ std::vector<gbmc::DebugReader> &debug_readers()
 }  // namespace
 
 void gbmc::debug_register(DebugReader fn) { debug_readers().push_back(fn); }
+
+cudaError_t gbmc::scratch_alloc(void **p, size_t bytes) { return dev_alloc_raw(p, bytes); }
+void gbmc::scratch_free(void *p) { dev_free_raw(p); }
 
 int gbmc::set_last_error(int code, const char *msg)
 {
@@ -810,10 +853,28 @@ int mc_release_cache(void)
 {
     std::lock_guard<std::mutex> g(g_cache_mu);
     release_cached(-1);
+    for (HostBlock *b : g_host_blocks) cudaFreeHost(b);
+    g_host_blocks.clear();
     return MC_OK;
 }
 
 const char *mc_last_error(void) { return g_err.c_str(); }
+
+// A set-up plan whose last set-up work may still be running on `stream`.
+static int plan_new(const mc_model *model, const mc_sim_cfg *cfg, const mc_payoff *payoffs, int32_t n_payoff,
+                    mc_plan **plan, cudaStream_t stream)
+{
+    if (n_payoff < 1) return fail(MC_EINVAL, "n_payoff must be >= 1");
+    mc_plan *P = new (std::nothrow) mc_plan();
+    if (!P) return fail(MC_ENOMEM, "host allocation failed");
+    const int rc = plan_setup(P, model, cfg, payoffs, n_payoff, nullptr, 0, stream);
+    if (rc) {
+        delete P;
+        return rc;
+    }
+    *plan = P;
+    return MC_OK;
+}
 
 int mc_plan_create(const mc_model *model, const mc_sim_cfg *cfg, const mc_payoff *payoffs, int32_t n_payoff,
                    mc_plan **plan, void *stream)
@@ -821,14 +882,9 @@ int mc_plan_create(const mc_model *model, const mc_sim_cfg *cfg, const mc_payoff
     gbmc::NvtxRange nvtx_("gbmc: plan set-up");
     if (!plan) return fail(MC_EINVAL, "plan is NULL");
     *plan = nullptr;
-    if (n_payoff < 1) return fail(MC_EINVAL, "n_payoff must be >= 1");
-    mc_plan *P = new (std::nothrow) mc_plan();
-    if (!P) return fail(MC_ENOMEM, "host allocation failed");
-    int rc = plan_setup(P, model, cfg, payoffs, n_payoff, nullptr, 0, static_cast<cudaStream_t>(stream));
-    if (rc) {
-        delete P;
-        return rc;
-    }
+    mc_plan *P = nullptr;
+    const int rc = plan_new(model, cfg, payoffs, n_payoff, &P, static_cast<cudaStream_t>(stream));
+    if (rc) return rc;
     cudaError_t e = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) {
         delete P;
@@ -922,16 +978,25 @@ int mc_price(const mc_model *model, const mc_sim_cfg *cfg, const mc_payoff *payo
     gbmc::NvtxRange nvtx_("gbmc: mc_price");
     if (!out) return fail(MC_EINVAL, "out is NULL");
     mc_plan *P = nullptr;
-    int rc = mc_plan_create(model, cfg, payoffs, n_payoff, &P, stream);
-    if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    rc = plan_launch(P, P->dout, s);
+    int rc = plan_new(model, cfg, payoffs, n_payoff, &P, s);
+    if (rc) return rc;
+    // The results go straight to pinned host memory.
+    HostBlock *hb = host_block_take();
+    mc_result *dst = hb ? hb->res : P->dout;
     std::vector<mc_result> tmp(n_payoff);
+    rc = plan_launch(P, dst, s);
     if (!rc) {
-        cudaError_t e = cudaMemcpyAsync(tmp.data(), P->dout, n_payoff * sizeof(mc_result), cudaMemcpyDeviceToHost, s);
+        cudaError_t e = cudaSuccess;
+        if (!hb) e = cudaMemcpyAsync(tmp.data(), P->dout, n_payoff * sizeof(mc_result), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) rc = fail(MC_ECUDA, "mc_price: %s", cudaGetErrorString(e));
         else P->idle = true;
+        if (hb && !rc) std::memcpy(tmp.data(), hb->res, n_payoff * sizeof(mc_result));
+    }
+    if (hb) {
+        if (P->idle) host_block_give(hb);
+        else if (cudaDeviceSynchronize() == cudaSuccess) cudaFreeHost(hb);
     }
     if (!rc && P->err) {
         unsigned int e = 0;

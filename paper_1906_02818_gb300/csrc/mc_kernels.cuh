@@ -329,6 +329,11 @@ struct CorrWide {
 };
 cudaError_t launch_corr_wide(const CorrArgs &a, const CorrWide &w, int grid, cudaStream_t s);
 
+// Device scratch from the cache of set-up blocks (mc_api.cu); a block goes back
+// only when no launch can still use it.
+cudaError_t scratch_alloc(void **p, size_t bytes);
+void scratch_free(void *p);
+
 // Records the thread-local message returned by mc_last_error(); returns code.
 int set_last_error(int code, const char *msg);
 // The argument checks of mc_price (model, simulation configuration, payoff
