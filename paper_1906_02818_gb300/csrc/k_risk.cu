@@ -13,7 +13,7 @@
 //   features_kernel  network inputs of every (scenario, option) pair;
 //   pnl_kernel       one scenario per CTA: portfolio PnL from the revalued
 //                    options (FP64 sum over options);
-//   tail_kernel      one CTA: bitonic sort of the losses, VaR and CVaR.
+//   tail_*_kernel    VaR by radix selection of the losses, CVaR.
 // Random streams: the stream index carries a domain tag in its top byte
 // (2 outer scenarios, 3 inner paths, 4 labels, 5 base values) so that the
 // domains never share normals.
@@ -375,57 +375,129 @@ __global__ void sum_under_kernel(int64_t nscen, int d, const double *contrib, do
 }
 
 // ------------------------------ VaR / CVaR -------------------------------
-// One CTA of 1024 threads: losses l = -pnl padded to a power of two with
-// -inf, bitonic sort descending in global memory (work), then
-// VaR = the k-th largest loss, k = ceil((1 - alpha) n), and CVaR = the mean of
-// the losses strictly above VaR (VaR itself if there is none).
-__global__ void __launch_bounds__(1024) tail_kernel(int64_t n, const double *pnl, double *work, int64_t npow2,
-                                                    double alpha, double *res)
+// Losses l = -pnl: VaR = the k-th largest loss, k = ceil((1 - alpha) n), and
+// CVaR = the mean of the losses strictly above VaR (VaR itself if there is
+// none).  VaR by radix selection from the top: each pass histograms the next
+// kTailBits bits of the losses' ordered keys among those that share the digits
+// found so far, and its last CTA picks the digit that holds the k-th; then one
+// pass adds up what lies above.  Seven reads of n values over the SMs, in
+// launches of a few microseconds; a sort of all losses in one CTA took 6.5 ms
+// of a 2^16-scenario run.
+constexpr int kTailBits = 11, kTailBins = 1 << kTailBits, kTailPasses = 6;  // 5 x 11 + 9 bits
+constexpr int kTailBlock = 512, kTailMaxGrid = 304;
+struct TailState {
+    unsigned long long prefix;       // the digits found
+    unsigned int k;                  // rank among the losses that share them, from the largest
+    unsigned int ticket[kTailPasses + 1];
+    unsigned int hist[kTailPasses][kTailBins];
+    double sum[kTailMaxGrid], count[kTailMaxGrid];
+};
+
+// Ascending unsigned order of the keys is ascending order of the doubles.
+__device__ __forceinline__ unsigned long long loss_key(double l)
 {
-    for (int64_t i = threadIdx.x; i < npow2; i += blockDim.x) work[i] = i < n ? -pnl[i] : -INFINITY;
+    const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(l));
+    return (u >> 63) ? ~u : u | 0x8000000000000000ull;
+}
+
+// Whether this CTA is the last of the launch to arrive (the others' writes are then visible).
+__device__ __forceinline__ bool last_cta(unsigned int *ticket)
+{
+    __shared__ unsigned int s_last;
+    __threadfence();
     __syncthreads();
-    for (int64_t k = 2; k <= npow2; k <<= 1) {
-        for (int64_t j = k >> 1; j > 0; j >>= 1) {
-            for (int64_t i = threadIdx.x; i < npow2; i += blockDim.x) {
-                const int64_t l = i ^ j;
-                if (l > i) {
-                    const bool desc = (i & k) == 0;
-                    const double x = work[i], y = work[l];
-                    if (desc ? (x < y) : (x > y)) {
-                        work[i] = y;
-                        work[l] = x;
-                    }
-                }
-            }
-            __syncthreads();
-        }
+    if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1u : 0u;
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last != 0u;
+}
+
+__global__ void __launch_bounds__(kTailBlock) tail_pass_kernel(int64_t n, const double *__restrict__ pnl, int pass,
+                                                               unsigned int k0, TailState *st)
+{
+    __shared__ unsigned int h[kTailBins];
+    __shared__ unsigned int scan[kTailBlock];
+    const int t = threadIdx.x;
+    const int below = 64 - kTailBits * pass;                             // bits below the digits found
+    const int width = below < kTailBits ? below : kTailBits, shift = below - width;
+    const unsigned long long prefix = pass ? st->prefix : 0ull;
+    for (int b = t; b < kTailBins; b += kTailBlock) h[b] = 0u;
+    __syncthreads();
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(kTailBlock) + t; i < n; i += static_cast<int64_t>(gridDim.x) * kTailBlock) {
+        const unsigned long long key = loss_key(-pnl[i]);
+        if (pass == 0 || (key >> below) == prefix) atomicAdd(&h[(key >> shift) & ((1ull << width) - 1ull)], 1u);
     }
-    __shared__ double s_red[32];
-    int64_t kk = static_cast<int64_t>(ceil((1.0 - alpha) * static_cast<double>(n) - 1e-9));
-    if (kk < 1) kk = 1;
-    const double var = work[kk - 1];
+    __syncthreads();
+    for (int b = t; b < kTailBins; b += kTailBlock)
+        if (h[b]) atomicAdd(&st->hist[pass][b], h[b]);
+    if (!last_cta(&st->ticket[pass])) return;
+    // thread t: the bins from kTailBins - 1 - 4 t down; counts from the top
+    constexpr int kPer = kTailBins / kTailBlock;
+    unsigned int c[kPer], own = 0u;
+    for (int j = 0; j < kPer; ++j) {
+        c[j] = *reinterpret_cast<volatile unsigned int *>(&st->hist[pass][kTailBins - 1 - kPer * t - j]);
+        own += c[j];
+    }
+    scan[t] = own;
+    __syncthreads();
+    for (int o = 1; o < kTailBlock; o <<= 1) {
+        const unsigned int v = t >= o ? scan[t - o] : 0u;
+        __syncthreads();
+        scan[t] += v;
+        __syncthreads();
+    }
+    const unsigned int k = pass ? st->k : k0;
+    unsigned int above = scan[t] - own;
+    __syncthreads();
+    if (above < k && k <= above + own)
+        for (int j = 0; j < kPer; ++j) {
+            if (k <= above + c[j]) {
+                st->prefix = (prefix << width) | static_cast<unsigned long long>(kTailBins - 1 - kPer * t - j);
+                st->k = k - above;
+                break;
+            }
+            above += c[j];
+        }
+}
+
+__global__ void __launch_bounds__(kTailBlock) tail_sum_kernel(int64_t n, const double *__restrict__ pnl, TailState *st, double *res)
+{
+    __shared__ double s_red[2][kTailBlock / 32];
+    const unsigned long long key = st->prefix;
+    const double var = __longlong_as_double(static_cast<long long>((key >> 63) ? key & 0x7fffffffffffffffull : ~key));
     double t = 0.0, c = 0.0;
-    for (int64_t i = threadIdx.x; i < kk; i += blockDim.x) {
-        if (work[i] > var) { t += work[i]; c += 1.0; }
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(kTailBlock) + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * kTailBlock) {
+        const double l = -pnl[i];
+        if (l > var) {
+            t += l;
+            c += 1.0;
+        }
     }
     t = warp_sum_d(t);
     c = warp_sum_d(c);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) { s_red[warp] = t; }
-    __syncthreads();
-    double tot = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < 32; ++w) tot += s_red[w];
-    __syncthreads();
-    if (lane == 0) s_red[warp] = c;
+    if ((threadIdx.x & 31) == 0) {
+        s_red[0][threadIdx.x >> 5] = t;
+        s_red[1][threadIdx.x >> 5] = c;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double cnt = 0.0;
-        for (int w = 0; w < 32; ++w) cnt += s_red[w];
-        res[0] = var;
-        res[1] = cnt > 0.0 ? tot / cnt : var;
-        res[2] = cnt;
+        t = c = 0.0;
+        for (int w = 0; w < kTailBlock / 32; ++w) {
+            t += s_red[0][w];
+            c += s_red[1][w];
+        }
+        st->sum[blockIdx.x] = t;
+        st->count[blockIdx.x] = c;
     }
+    if (!last_cta(&st->ticket[kTailPasses]) || threadIdx.x != 0) return;
+    t = c = 0.0;
+    for (unsigned int g = 0; g < gridDim.x; ++g) {
+        t += *reinterpret_cast<volatile double *>(&st->sum[g]);
+        c += *reinterpret_cast<volatile double *>(&st->count[g]);
+    }
+    res[0] = var;
+    res[1] = c > 0.0 ? t / c : var;
+    res[2] = c;
 }
 
 }  // namespace
@@ -493,10 +565,21 @@ cudaError_t launch_pnl(const RiskArgs &a, int64_t nscen, const float *Sp, const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_tail(int64_t n, const double *pnl, double *work, int64_t npow2, double alpha, double *res,
-                        cudaStream_t s)
+size_t tail_scratch_bytes() { return sizeof(TailState); }
+
+cudaError_t launch_tail(int64_t n, const double *pnl, void *scratch, double alpha, double *res, cudaStream_t s)
 {
-    tail_kernel<<<1, 1024, 0, s>>>(n, pnl, work, npow2, alpha, res);
+    TailState *st = static_cast<TailState *>(scratch);
+    int64_t k = static_cast<int64_t>(std::ceil((1.0 - alpha) * static_cast<double>(n) - 1e-9));
+    if (k < 1) k = 1;
+    cudaError_t e = cudaMemsetAsync(st, 0, sizeof(TailState), s);
+    if (e != cudaSuccess) return e;
+    const int grid = static_cast<int>(std::min<int64_t>(kTailMaxGrid, (n + 2 * kTailBlock - 1) / (2 * kTailBlock)));
+    for (int pass = 0; pass < kTailPasses; ++pass) {
+        tail_pass_kernel<<<grid, kTailBlock, 0, s>>>(n, pnl, pass, static_cast<unsigned int>(k), st);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    tail_sum_kernel<<<grid, kTailBlock, 0, s>>>(n, pnl, st, res);
     return cudaGetLastError();
 }
 

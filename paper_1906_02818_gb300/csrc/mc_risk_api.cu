@@ -37,18 +37,28 @@ namespace {
 
 int fail(int code, const char *msg) { return set_last_error(code, msg); }
 
+// The buffers of one call: from the cache of scratch blocks, so that repeated
+// calls neither allocate nor free (19 of each per mc_risk, and a cudaFree
+// waits for the device); blocks over kKeep are allocated and freed instead.
 struct DevBufs {
-    std::vector<void *> ptrs;
+    static constexpr size_t kKeep = size_t(64) << 20;
+    std::vector<void *> cached, own;
+    bool idle = false;  // set once the call's stream has been synchronised
     template <class T>
     cudaError_t alloc(T **p, size_t n)
     {
-        cudaError_t e = cudaMalloc(reinterpret_cast<void **>(p), n * sizeof(T) + 16);
-        if (e == cudaSuccess) ptrs.push_back(*p);
+        const size_t bytes = n * sizeof(T) + 16;
+        void *q = nullptr;
+        const cudaError_t e = bytes <= kKeep ? scratch_alloc(&q, bytes) : cudaMalloc(&q, bytes);
+        if (e == cudaSuccess) (bytes <= kKeep ? cached : own).push_back(q);
+        *p = static_cast<T *>(q);
         return e;
     }
     ~DevBufs()
     {
-        for (void *p : ptrs) cudaFree(p);
+        if (!idle && !cached.empty()) cudaDeviceSynchronize();
+        for (void *p : cached) scratch_free(p);
+        for (void *p : own) cudaFree(p);
     }
 };
 
@@ -91,16 +101,16 @@ int mc_tail(const double *dev_pnl, int64_t n, double alpha, mc_risk_result *res,
     if (n < 1 || n > (int64_t(1) << 24)) return fail(MC_EINVAL, "n outside [1, 2^24]");
     if (!(alpha > 0.0 && alpha < 1.0)) return fail(MC_EINVAL, "alpha must lie in (0, 1)");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int64_t np2 = 1;
-    while (np2 < n) np2 <<= 1;
     DevBufs B;
-    double *d_work, *d_res;
-    RK_CUDA(B.alloc(&d_work, np2));
+    unsigned char *d_work;
+    double *d_res;
+    RK_CUDA(B.alloc(&d_work, tail_scratch_bytes()));
     RK_CUDA(B.alloc(&d_res, 3));
-    RK_CUDA(launch_tail(n, dev_pnl, d_work, np2, alpha, d_res, s));
+    RK_CUDA(launch_tail(n, dev_pnl, d_work, alpha, d_res, s));
     double r3[3];
     RK_CUDA(cudaMemcpyAsync(r3, d_res, sizeof r3, cudaMemcpyDeviceToHost, s));
     RK_CUDA(cudaStreamSynchronize(s));
+    B.idle = true;
     res->var = r3[0];
     res->cvar = r3[1];
     res->n_tail = static_cast<int64_t>(r3[2]);
@@ -173,16 +183,15 @@ int mc_risk(const mc_portfolio *pf, const mc_risk_cfg *cf, mc_risk_result *res, 
     DevBufs B;
     int *d_under, *d_kind, *d_rem, *d_start, *d_status;
     float *d_K, *d_H, *d_s0, *d_sig, *d_Lc, *d_drift, *d_Sp;
-    double *d_pos, *d_base, *d_corr, *d_L, *d_pnl, *d_work, *d_res;
+    double *d_pos, *d_base, *d_corr, *d_L, *d_pnl, *d_res;
+    unsigned char *d_work;
     const int64_t ns = cf->n_scen;
-    int64_t np2 = 1;
-    while (np2 < ns) np2 <<= 1;
     RK_CUDA(B.alloc(&d_under, no)); RK_CUDA(B.alloc(&d_kind, no)); RK_CUDA(B.alloc(&d_rem, no));
     RK_CUDA(B.alloc(&d_start, d + 1)); RK_CUDA(B.alloc(&d_status, 1));
     RK_CUDA(B.alloc(&d_K, no)); RK_CUDA(B.alloc(&d_H, no)); RK_CUDA(B.alloc(&d_s0, d)); RK_CUDA(B.alloc(&d_sig, d));
     RK_CUDA(B.alloc(&d_Lc, d * d)); RK_CUDA(B.alloc(&d_drift, d)); RK_CUDA(B.alloc(&d_Sp, ns * d));
     RK_CUDA(B.alloc(&d_pos, no)); RK_CUDA(B.alloc(&d_base, no)); RK_CUDA(B.alloc(&d_corr, d * d));
-    RK_CUDA(B.alloc(&d_L, d * d)); RK_CUDA(B.alloc(&d_pnl, ns)); RK_CUDA(B.alloc(&d_work, np2)); RK_CUDA(B.alloc(&d_res, 3));
+    RK_CUDA(B.alloc(&d_L, d * d)); RK_CUDA(B.alloc(&d_pnl, ns)); RK_CUDA(B.alloc(&d_work, tail_scratch_bytes())); RK_CUDA(B.alloc(&d_res, 3));
     std::vector<float> h_s0(d), h_sig(d);
     for (int u = 0; u < d; ++u) {
         h_s0[u] = static_cast<float>(pf->s0[u]);
@@ -272,13 +281,14 @@ int mc_risk(const mc_portfolio *pf, const mc_risk_cfg *cf, mc_risk_result *res, 
             RK_CUDA(launch_pnl(a, nc, d_Sp + s0 * d, d_y, d_pnl + s0, s));
         }
     }
-    RK_CUDA(launch_tail(ns, d_pnl, d_work, np2, cf->alpha, d_res, s));
+    RK_CUDA(launch_tail(ns, d_pnl, d_work, cf->alpha, d_res, s));
     double r3[3];
     std::vector<double> base(no);
     RK_CUDA(cudaMemcpyAsync(r3, d_res, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
     RK_CUDA(cudaMemcpyAsync(base.data(), d_base, no * sizeof(double), cudaMemcpyDeviceToHost, s));
     if (host_pnl) RK_CUDA(cudaMemcpyAsync(host_pnl, d_pnl, ns * sizeof(double), cudaMemcpyDeviceToHost, s));
     RK_CUDA(cudaStreamSynchronize(s));
+    B.idle = true;
     if (cf->method == MC_RISK_SURROGATE && cf->surrogate_precision == MC_BF16) {
         const int rc = mlp_check_timeout(cf->surrogate, s);
         if (rc) return rc;

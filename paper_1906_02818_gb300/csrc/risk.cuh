@@ -42,7 +42,8 @@ cudaError_t launch_nested(const RiskArgs &a, int64_t nscen, const float *Sp, dou
 cudaError_t launch_sum_under(int64_t nscen, int d, const double *contrib, double *pnl, cudaStream_t s);
 cudaError_t launch_features(const RiskArgs &a, int64_t nscen, const float *Sp, float *x, cudaStream_t s);
 cudaError_t launch_pnl(const RiskArgs &a, int64_t nscen, const float *Sp, const float *y, double *pnl, cudaStream_t s);
-cudaError_t launch_tail(int64_t n, const double *pnl, double *work, int64_t npow2, double alpha, double *res,
-                        cudaStream_t s);
+// res: VaR, CVaR, losses above VaR; scratch: tail_scratch_bytes().
+size_t tail_scratch_bytes();
+cudaError_t launch_tail(int64_t n, const double *pnl, void *scratch, double alpha, double *res, cudaStream_t s);
 
 }  // namespace gbmc
