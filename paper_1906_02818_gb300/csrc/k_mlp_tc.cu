@@ -248,23 +248,25 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bf16_kernel(const Args a)
                 const bool last = l == NL - 1;
                 const float *bias = a.params + a.b_off[l];
                 float acc_out = 0.0f;
-                for (int cc = 0; cc < ncol; cc += 16) {
-                    float v[16];
-                    if (live) {
-                        tc::tmem_ld16(taddr + cc, v);
-                        tc::tmem_wait_ld();
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) v[e] = 0.0f;
-                    }
+                // 16 columns at a time; the next 16 leave tensor memory while
+                // these go through the activation (two warps per SM quarter
+                // share a tile's epilogue: too few to hide that latency, which
+                // a load used at once exposed eight times per layer)
+                auto columns = [&](int cc, float (&v)[16], float (&ahead)[16]) {
                     const int c = col0 + cc;
+                    float4 b4[4];
+#pragma unroll
+                    for (int e4 = 0; e4 < 4; ++e4) b4[e4] = __ldg(reinterpret_cast<const float4 *>(bias + c) + e4);
+                    if (live) {
+                        tc::tmem_wait_ld16(v);
+                        if (cc + 16 < ncol) tc::tmem_ld16(taddr + cc + 16, ahead);
+                    }
 #pragma unroll
                     for (int e4 = 0; e4 < 4; ++e4) {
-                        const float4 b4 = __ldg(reinterpret_cast<const float4 *>(bias + c) + e4);
-                        v[4 * e4] = silu_tanh(v[4 * e4] + b4.x);
-                        v[4 * e4 + 1] = silu_tanh(v[4 * e4 + 1] + b4.y);
-                        v[4 * e4 + 2] = silu_tanh(v[4 * e4 + 2] + b4.z);
-                        v[4 * e4 + 3] = silu_tanh(v[4 * e4 + 3] + b4.w);
+                        v[4 * e4] = silu_tanh(v[4 * e4] + b4[e4].x);
+                        v[4 * e4 + 1] = silu_tanh(v[4 * e4 + 1] + b4[e4].y);
+                        v[4 * e4 + 2] = silu_tanh(v[4 * e4 + 2] + b4[e4].z);
+                        v[4 * e4 + 3] = silu_tanh(v[4 * e4 + 3] + b4[e4].w);
                     }
                     if (!last) {
                         const uint32_t pan = A + (c / kKc) * kPanelBytes;
@@ -282,6 +284,14 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bf16_kernel(const Args a)
                             acc_out = fmaf(w4.w, v[4 * e4 + 3], acc_out);
                         }
                     }
+                };
+                float va[16], vb[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) va[e] = vb[e] = 0.0f;
+                if (live) tc::tmem_ld16(taddr, va);
+                for (int cc = 0; cc < ncol; cc += 32) {
+                    columns(cc, va, vb);
+                    if (cc + 16 < ncol) columns(cc + 16, vb, va);
                 }
                 if (!last) {
                     tc::fence_proxy_async();
