@@ -132,17 +132,16 @@ __global__ void __launch_bounds__(kThreads) corr_path_kernel(const __grid_consta
 }
 
 // Batch k of B: the FP64 sum of the partials of CTAs k, k + B, k + 2B, ...
-__global__ void corr_batch_kernel(const float *partials, const double *counts, int G, int B, double *Hb,
-                                  double *nb)
+__global__ void __launch_bounds__(256) corr_batch_kernel(const float *__restrict__ partials, const double *__restrict__ counts,
+                                                         int G, int B, double *__restrict__ Hb, double *__restrict__ nb)
 {
-    const int k = blockIdx.x;
-    for (int e = threadIdx.x; e < kD * kD; e += blockDim.x) {
-        double s = 0.0;
-        for (int c = k; c < G; c += B) s += static_cast<double>(partials[static_cast<size_t>(c) * kD * kD + e]);
-        Hb[static_cast<size_t>(k) * kD * kD + e] = s;
-    }
-    if (threadIdx.x == 0) {
-        double s = 0.0;
+    const int k = blockIdx.x, e = blockIdx.y * blockDim.x + threadIdx.x;
+    double s = 0.0;
+#pragma unroll 4
+    for (int c = k; c < G; c += B) s += static_cast<double>(partials[static_cast<size_t>(c) * kD * kD + e]);
+    Hb[static_cast<size_t>(k) * kD * kD + e] = s;
+    if (e == 0) {
+        s = 0.0;
         for (int c = k; c < G; c += B) s += counts[c];
         nb[k] = s;
     }
@@ -150,12 +149,17 @@ __global__ void corr_batch_kernel(const float *partials, const double *counts, i
 
 // Block k < B: batch k; block B: all paths.  FP64, d <= 64, one CTA each.
 // Outputs per block: dP/dLrho (lower, d-stride) and dP/dcorr (symmetric).
+// The two triangular solves run right-looking, four lanes to a row (column),
+// with the factor's reciprocal diagonal: 64 dependent steps of one product and
+// up to 16 independent FMAs per lane, where one thread per row ran 2000
+// dependent FMAs and 64 divisions (403 us at d = 64).
 __global__ void __launch_bounds__(256) corr_adjoint_kernel(int d, int B, const double *Hb, const double *nb,
                                                             const double *L, const double *cfac, double *out_dl,
                                                             double *out_drho)
 {
     extern __shared__ double sm[];
-    double *sL = sm, *sG = sm + d * d, *sA = sm + 2 * d * d;   // Lrho, Lbar then S, A then P then X
+    const int ld = d + 1;  // padded rows: the second solve walks columns
+    double *sL = sm, *sG = sL + d * ld, *sA = sG + d * ld, *sr = sA + d * ld;  // Lrho, Lbar then S, A then P then X, 1 / Lrho_ii
     const int k = blockIdx.x, tid = threadIdx.x;
     double n = 0.0;
     if (k < B) n = nb[k];
@@ -170,45 +174,69 @@ __global__ void __launch_bounds__(256) corr_adjoint_kernel(int d, int B, const d
             else for (int q = 0; q < B; ++q) h += Hb[static_cast<size_t>(q) * kD * kD + i * kD + j];
         }
         const double g = cfac[i] * h * inv_n;   // Lbar = dP/dLrho
-        sG[e] = g;
+        sG[i * ld + j] = g;
         odl[e] = g;
-        sL[e] = L[e];
+        sL[i * ld + j] = L[e];
     }
     __syncthreads();
+    if (tid < d) sr[tid] = 1.0 / sL[tid * ld + tid];
     // A = Lrho^T Lbar, then P = Phi(A)
     for (int e = tid; e < d * d; e += blockDim.x) {
         const int i = e / d, j = e % d;
-        double s = 0.0;
+        double s0 = 0.0, s1 = 0.0;
         if (j <= i) {
-            for (int q = i; q < d; ++q) s = fma(sL[q * d + i], sG[q * d + j], s);
-            if (j == i) s *= 0.5;
+            int q = i;
+            for (; q + 1 < d; q += 2) {
+                s0 = fma(sL[q * ld + i], sG[q * ld + j], s0);
+                s1 = fma(sL[(q + 1) * ld + i], sG[(q + 1) * ld + j], s1);
+            }
+            if (q < d) s0 = fma(sL[q * ld + i], sG[q * ld + j], s0);
+            s0 += s1;
+            if (j == i) s0 *= 0.5;
         }
-        sA[e] = s;
+        sA[i * ld + j] = s0;
     }
     __syncthreads();
-    // X = P Lrho^-1 (rows, in place): x_ij = (p_ij - sum_{q > j} x_iq L_qj) / L_jj, j = i .. 0
-    if (tid < d) {
-        const int i = tid;
-        for (int j = i; j >= 0; --j) {
-            double s = sA[i * d + j];
-            for (int q = j + 1; q <= i; ++q) s = fma(-sA[i * d + q], sL[q * d + j], s);
-            sA[i * d + j] = s / sL[j * d + j];
+    const int row = tid >> 2, lane = tid & 3;  // four lanes of one warp per row (column), d <= 64 of them
+    double w[kD / 4];                          // entries 4 e + lane
+    // X = P Lrho^-1: x_ij = p_ij / L_jj, then p_iq -= x_ij L_jq for q < j, j = d - 1 .. 0 (zero past i)
+#pragma unroll
+    for (int e = 0; e < kD / 4; ++e) w[e] = (row < d && 4 * e + lane < d) ? sA[row * ld + 4 * e + lane] : 0.0;
+#pragma unroll
+    for (int j = kD - 1; j >= 0; --j) {
+        if (j < d) {
+            const double x = __shfl_sync(0xffffffffu, w[j >> 2], j & 3, 4) * sr[j];
+            if (lane == (j & 3)) w[j >> 2] = x;
+#pragma unroll
+            for (int e = 0; e <= (j >> 2); ++e)
+                if (4 * e + lane < j) w[e] = fma(-x, sL[j * ld + 4 * e + lane], w[e]);
         }
     }
     __syncthreads();
-    // S = Lrho^-T X (columns, into sG): s_ij = (x_ij - sum_{q > i} L_qi s_qj) / L_ii, i = d-1 .. 0
-    if (tid < d) {
-        const int j = tid;
-        for (int i = d - 1; i >= 0; --i) {
-            double s = sA[i * d + j];
-            for (int q = i + 1; q < d; ++q) s = fma(-sL[q * d + i], sG[q * d + j], s);
-            sG[i * d + j] = s / sL[i * d + i];
+#pragma unroll
+    for (int e = 0; e < kD / 4; ++e)
+        if (row < d && 4 * e + lane < d) sA[row * ld + 4 * e + lane] = w[e];
+    __syncthreads();
+    // S = Lrho^-T X, column `row`: s_ij = x_ij / L_ii, then x_qj -= L_iq s_ij for q < i, i = d - 1 .. 0
+#pragma unroll
+    for (int e = 0; e < kD / 4; ++e) w[e] = (row < d && 4 * e + lane < d) ? sA[(4 * e + lane) * ld + row] : 0.0;
+#pragma unroll
+    for (int i = kD - 1; i >= 0; --i) {
+        if (i < d) {
+            const double x = __shfl_sync(0xffffffffu, w[i >> 2], i & 3, 4) * sr[i];
+            if (lane == (i & 3)) w[i >> 2] = x;
+#pragma unroll
+            for (int e = 0; e <= (i >> 2); ++e)
+                if (4 * e + lane < i) w[e] = fma(-x, sL[i * ld + 4 * e + lane], w[e]);
         }
     }
+#pragma unroll
+    for (int e = 0; e < kD / 4; ++e)
+        if (row < d && 4 * e + lane < d) sG[(4 * e + lane) * ld + row] = w[e];
     __syncthreads();
     for (int e = tid; e < d * d; e += blockDim.x) {
         const int i = e / d, j = e % d;
-        odr[e] = (i == j) ? 0.0 : sG[i * d + j] + sG[j * d + i];
+        odr[e] = (i == j) ? 0.0 : sG[i * ld + j] + sG[j * ld + i];
     }
 }
 
@@ -589,7 +617,7 @@ int corr_occupancy(const CorrArgs &a)
 
 int corr_block() { return kThreads; }
 
-size_t corr_adjoint_smem(int d) { return 3 * static_cast<size_t>(d) * d * sizeof(double); }
+size_t corr_adjoint_smem(int d) { return (3 * static_cast<size_t>(d) * (d + 1) + d) * sizeof(double); }
 
 cudaError_t launch_corr(const CorrArgs &a, const CorrConst &c, int grid, int batches, const double *L,
                         const double *cfac, double *Hb, double *nb, double *out_dl, double *out_drho,
@@ -604,7 +632,7 @@ cudaError_t launch_corr(const CorrArgs &a, const CorrConst &c, int grid, int bat
     }
     cudaError_t e = cudaLaunchKernel(corr_select(a), dim3(grid), dim3(kThreads), args, dyn, s);
     if (e != cudaSuccess) return e;
-    corr_batch_kernel<<<batches, 256, 0, s>>>(a.partials, a.counts, grid, batches, Hb, nb);
+    corr_batch_kernel<<<dim3(batches, kD * kD / 256), 256, 0, s>>>(a.partials, a.counts, grid, batches, Hb, nb);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const size_t smem = corr_adjoint_smem(a.d);
     if (smem > 48 * 1024) {
@@ -615,7 +643,7 @@ cudaError_t launch_corr(const CorrArgs &a, const CorrConst &c, int grid, int bat
     corr_adjoint_kernel<<<batches + 1, 256, smem, s>>>(a.d, batches, Hb, nb, L, cfac, out_dl, out_drho);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int dd2 = 2 * a.d * a.d;
-    corr_finish_kernel<<<(dd2 + 255) / 256, 256, 0, s>>>(a.d, batches, nb, out_dl, out_drho, res_dl, res_drho);
+    corr_finish_kernel<<<(dd2 + 31) / 32, 32, 0, s>>>(a.d, batches, nb, out_dl, out_drho, res_dl, res_drho);
     return cudaGetLastError();
 }
 

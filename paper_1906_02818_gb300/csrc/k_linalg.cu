@@ -53,10 +53,12 @@ __global__ void __launch_bounds__(kCholSmallBlock) cholesky_small_kernel(int d, 
 {
     __shared__ double W[kCholSmallD][kCholSmallD + 1];
     __shared__ uint16_t tri[kCholTri];  // (ii << 6) | jj, jj <= ii, row by row
+    __shared__ double s_diag[kCholSmallD];  // A's diagonal for the pivot checks: a load in the column loop's serial chain otherwise
     __shared__ double s_inv;
     __shared__ int s_fail;
     const int t = threadIdx.x;
     for (int idx = t; idx < d * d; idx += blockDim.x) W[idx / d][idx % d] = A[idx];
+    for (int k = t; k < d; k += blockDim.x) s_diag[k] = A[k * d + k];
     for (int ii = t; ii < kCholSmallD - 1; ii += blockDim.x)
         for (int jj = 0; jj <= ii; ++jj) tri[ii * (ii + 1) / 2 + jj] = static_cast<uint16_t>((ii << 6) | jj);
     if (t == 0) {
@@ -86,7 +88,7 @@ __global__ void __launch_bounds__(kCholSmallBlock) cholesky_small_kernel(int d, 
         // entry 0 is (k + 1, k + 1), updated above by this same thread
         if (t == 0 && k + 1 < d) {
             const double p = W[k + 1][k + 1];
-            if (!pivot_ok(p, A[(k + 1) * d + (k + 1)], d)) {
+            if (!pivot_ok(p, s_diag[k + 1], d)) {
                 s_fail = 1;
             } else {
                 const double r = rsqrt_refined(p);
@@ -105,11 +107,14 @@ __global__ void __launch_bounds__(kCholSmallBlock) cholesky_small_kernel(int d, 
 }
 
 // Blocked right-looking Cholesky for d > 64, spread over the SMs (FP64 issue
-// on this part is a few FMAs per clock per SM, so one CTA is slow): for each
+// on this part is two FMAs per clock per SM, so one CTA is slow): for each
 // 32-column block K, (1) one CTA factors the diagonal block in shared memory,
-// (2) one thread per row below it solves the panel row against it, (3) one
-// CTA per 32 x 32 block of the trailing lower triangle subtracts the panel
-// product.  Pivots are checked against the original diagonal as above.
+// (2) the panel rows are solved against it, four lanes to a row, (3) one CTA
+// per 32 x 32 block of the trailing lower triangle subtracts the panel
+// product.  Pivots are checked against the original diagonal as above.  (1)
+// and (2) are chains of dependent FP64 operations and set the time: a panel
+// row by one thread, and a pivot check that loads in the chain, took 64 us and
+// 50 us of a block's 130 us; d = 512 took 2.1 ms.
 constexpr int kCholNb = 32;
 
 __global__ void chol_copy_kernel(int64_t n, const double *__restrict__ A, double *__restrict__ W, int *status)
@@ -120,41 +125,49 @@ __global__ void chol_copy_kernel(int64_t n, const double *__restrict__ A, double
     if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
 }
 
-// (1) the diagonal block W[k0 .. k0 + nb)^2, in place (lower part)
+// (1) the diagonal block W[k0 .. k0 + nb)^2, in place (lower part), and the
+// reciprocals of its diagonal (rdiag).  As in cholesky_small_kernel: dense walk
+// of the trailing triangle, whose first entry, the next pivot, thread 0
+// updates and turns into the next reciprocal square root without waiting.
 __global__ void __launch_bounds__(256) chol_diag_kernel(int d, int k0, int nb, const double *__restrict__ A,
-                                                        double *__restrict__ W, int *status)
+                                                        double *__restrict__ W, double *__restrict__ rdiag, int *status)
 {
     __shared__ double T[kCholNb][kCholNb + 1];
-    __shared__ double s_inv;
+    __shared__ uint16_t tri[kCholNb * (kCholNb - 1) / 2];  // (ii << 6) | jj, jj <= ii, row by row
+    __shared__ double s_diag[kCholNb], s_inv[kCholNb];
     __shared__ int s_fail;
     const int t = threadIdx.x;
     for (int e = t; e < nb * nb; e += blockDim.x) T[e / nb][e % nb] = W[static_cast<int64_t>(k0 + e / nb) * d + k0 + e % nb];
+    if (t < nb) s_diag[t] = A[static_cast<int64_t>(k0 + t) * d + k0 + t];
+    if (t < kCholNb - 1)
+        for (int jj = 0; jj <= t; ++jj) tri[t * (t + 1) / 2 + jj] = static_cast<uint16_t>((t << 6) | jj);
     if (t == 0) s_fail = 0;
     __syncthreads();
-    for (int k = 0; k < nb; ++k) {
-        if (t == 0) {
-            const double p = T[k][k];
-            const int64_t g = static_cast<int64_t>(k0 + k) * d + (k0 + k);
-            if (!pivot_ok(p, A[g], d)) {
-                s_fail = 1;
-            } else {
-                const double r = rsqrt_refined(p);
-                T[k][k] = p * r;
-                s_inv = r;
-            }
+    auto pivot = [&](int k) {  // thread 0
+        const double p = T[k][k];
+        if (!pivot_ok(p, s_diag[k], d)) {
+            s_fail = 1;
+        } else {
+            const double r = rsqrt_refined(p);
+            T[k][k] = p * r;
+            s_inv[k] = r;
         }
+    };
+    if (t == 0) pivot(0);
+    for (int k = 0; k < nb; ++k) {
         __syncthreads();
         if (s_fail) break;
-        const double inv = s_inv;
+        const double inv = s_inv[k];
         for (int i = k + 1 + t; i < nb; i += blockDim.x) T[i][k] *= inv;
         __syncthreads();
-        const int m = nb - k - 1;
-        for (int e = t; e < m * m; e += blockDim.x) {
-            const int i = k + 1 + e / m, j = k + 1 + e % m;
-            if (j <= i) T[i][j] -= T[i][k] * T[j][k];
+        const int m = nb - k - 1, n = m * (m + 1) / 2;
+        for (int e = t; e < n; e += blockDim.x) {
+            const int code = tri[e], i = k + 1 + (code >> 6), j = k + 1 + (code & 63);
+            T[i][j] -= T[i][k] * T[j][k];
         }
-        __syncthreads();
+        if (t == 0 && k + 1 < nb) pivot(k + 1);
     }
+    __syncthreads();
     if (s_fail) {
         if (t == 0) *status = 1;
         return;
@@ -163,20 +176,39 @@ __global__ void __launch_bounds__(256) chol_diag_kernel(int d, int k0, int nb, c
         const int i = e / nb, j = e % nb;
         if (j <= i) W[static_cast<int64_t>(k0 + i) * d + k0 + j] = T[i][j];
     }
+    if (t < nb) rdiag[t] = 1.0 / T[t][t];
 }
 
-// (2) rows i >= k0 + nb of the panel: L_ij = (W_ij - sum_{c < j} L_ic L_jc) / L_jj, j in the block
-__global__ void chol_panel_kernel(int d, int k0, int nb, double *__restrict__ W)
+// (2) rows i >= k0 + nb of the panel (nb = kCholNb: only the last block is
+// narrower, and it has no panel): x_j = w_j / L_jj, then w_c -= x_j L_cj for
+// c > j, j = 0 .. 31, four lanes to a row (lane q holds the columns 4 e + q).
+__global__ void __launch_bounds__(64) chol_panel_kernel(int d, int k0, const double *__restrict__ rdiag, double *__restrict__ W)
 {
-    const int i = k0 + nb + blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= d) return;
-    double *Ri = W + static_cast<int64_t>(i) * d + k0;
-    for (int j = 0; j < nb; ++j) {
-        const double *Rj = W + static_cast<int64_t>(k0 + j) * d + k0;
-        double s = Ri[j];
-        for (int c = 0; c < j; ++c) s = fma(-Ri[c], Rj[c], s);
-        Ri[j] = s / Rj[j];
+    __shared__ double Lt[kCholNb][kCholNb];  // Lt[j][c] = L_cj for c > j, else 0
+    __shared__ double s_r[kCholNb];
+    const int t = threadIdx.x, q = t & 3;
+    for (int e = t; e < kCholNb * kCholNb; e += 64) {
+        const int c = e / kCholNb, j = e % kCholNb;
+        Lt[j][c] = c > j ? W[static_cast<int64_t>(k0 + c) * d + k0 + j] : 0.0;
     }
+    if (t < kCholNb) s_r[t] = rdiag[t];
+    __syncthreads();
+    const int i = k0 + kCholNb + blockIdx.x * 16 + (t >> 2);
+    const bool in = i < d;
+    double *Ri = W + static_cast<int64_t>(in ? i : k0) * d + k0;
+    double w[kCholNb / 4];
+#pragma unroll
+    for (int e = 0; e < kCholNb / 4; ++e) w[e] = in ? Ri[4 * e + q] : 0.0;
+#pragma unroll
+    for (int j = 0; j < kCholNb; ++j) {
+        const double x = __shfl_sync(0xffffffffu, w[j >> 2], j & 3, 4) * s_r[j];
+        if (q == (j & 3)) w[j >> 2] = x;
+#pragma unroll
+        for (int e = j >> 2; e < kCholNb / 4; ++e) w[e] = fma(-x, Lt[j][4 * e + q], w[e]);  // zero factors for c <= j
+    }
+    if (in)
+#pragma unroll
+        for (int e = 0; e < kCholNb / 4; ++e) Ri[4 * e + q] = w[e];
 }
 
 // (3) the trailing lower triangle, one CTA per 32 x 32 block (bi >= bj) of
@@ -247,9 +279,10 @@ cudaError_t launch_cholesky(int d, const double *A, double *L, int *status, cuda
     chol_copy_kernel<<<g, 256, 0, s>>>(n, A, L, status);
     for (int k0 = 0; k0 < d; k0 += kCholNb) {
         const int nb = std::min(kCholNb, d - k0), rest = d - k0 - nb;
-        chol_diag_kernel<<<1, 256, 0, s>>>(d, k0, nb, A, L, status);
+        double *rdiag = L + d - kCholNb;  // row 0's last entries: above the diagonal (d > 64), zeroed at the end
+        chol_diag_kernel<<<1, 256, 0, s>>>(d, k0, nb, A, L, rdiag, status);
         if (rest > 0) {
-            chol_panel_kernel<<<(rest + 127) / 128, 128, 0, s>>>(d, k0, nb, L);
+            chol_panel_kernel<<<(rest + 15) / 16, 64, 0, s>>>(d, k0, rdiag, L);
             const int nbl = (rest + kCholNb - 1) / kCholNb;
             chol_update_kernel<<<nbl * (nbl + 1) / 2, 256, 0, s>>>(d, k0, nb, L);
         }
