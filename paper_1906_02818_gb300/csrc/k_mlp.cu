@@ -207,6 +207,35 @@ __global__ void smallk_kernel(int M, int N, int K, const float *__restrict__ A, 
     }
 }
 
+// The same for N a multiple of 4 and every row with bias and activation
+// (bias_rows >= M): four outputs of a row per thread, B row-major.
+__global__ void __launch_bounds__(256) smallk4_kernel(int M, int N, int K, const float *__restrict__ A, int lda,
+                                                      const float *__restrict__ B, int ldb, const float *__restrict__ bias,
+                                                      float *__restrict__ Z, float *__restrict__ H, int ldc, int act)
+{
+    const int g = N / 4, rows = static_cast<int>(blockDim.x) / g;
+    const int r = static_cast<int>(threadIdx.x) / g, n = 4 * (static_cast<int>(threadIdx.x) % g);
+    if (r >= rows) return;
+    const float4 b4 = bias ? *reinterpret_cast<const float4 *>(bias + n) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int64_t m = static_cast<int64_t>(blockIdx.x) * rows + r; m < M; m += static_cast<int64_t>(gridDim.x) * rows) {
+        const float *a = A + m * lda;
+        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (int k = 0; k < K; ++k) {
+            const float ak = a[k];
+            const float4 w = *reinterpret_cast<const float4 *>(B + static_cast<int64_t>(k) * ldb + n);
+            s.x = fmaf(ak, w.x, s.x);
+            s.y = fmaf(ak, w.y, s.y);
+            s.z = fmaf(ak, w.z, s.z);
+            s.w = fmaf(ak, w.w, s.w);
+        }
+        s = make_float4(s.x + b4.x, s.y + b4.y, s.z + b4.z, s.w + b4.w);
+        if (Z) *reinterpret_cast<float4 *>(Z + m * ldc + n) = s;
+        if (H)
+            *reinterpret_cast<float4 *>(H + m * ldc + n) =
+                act ? make_float4(silu_f(s.x), silu_f(s.y), silu_f(s.z), silu_f(s.w)) : s;
+    }
+}
+
 // One output column (N = 1, e.g. the network's scalar output layer): a warp
 // per row, lanes over k, then a fixed-order warp sum.
 __global__ void rowvec_kernel(int M, int K, const float *__restrict__ A, int lda, const float *__restrict__ B, int ldb,
@@ -555,6 +584,161 @@ __global__ void dact_bwd_kernel(int64_t n, int K, int C, const float *__restrict
     }
 }
 
+// Element-wise steps over rows of C floats, C a multiple of 4 (the tensor-core
+// training path: a multiple of 64), four columns at a time.  The grid strides
+// by whole rows of column groups (vec_grid), so a thread's columns never
+// change: no division per element, and column sums gather in registers.
+// One pass per layer and direction; they are bound by the traffic of the
+// stacked rows.  With an index division per element, the bias, activation and
+// tangents apart, and column sums read back down strided columns, they were
+// 45 % of a 0.71 ms step of 4096 samples.
+struct F4 {
+    float v[4];
+};
+__device__ __forceinline__ F4 ld4(const float *p)
+{
+    const float4 q = *reinterpret_cast<const float4 *>(p);
+    return F4{{q.x, q.y, q.z, q.w}};
+}
+__device__ __forceinline__ void st4(float *p, const F4 &q) { *reinterpret_cast<float4 *>(p) = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]); }
+
+constexpr int kVecBlock = 256;
+// Blocks for `rows` rows of C floats: a multiple of what makes the grid's
+// threads whole rows, at most about four per SM.
+int vec_grid(int64_t rows, int C)
+{
+    const int g = C / 4;
+    int unit = g;
+    for (int b = kVecBlock; unit % 2 == 0 && b % 2 == 0; b /= 2) unit /= 2;  // g / gcd(g, 256): 256 is a power of two
+    const int64_t want = std::min<int64_t>(640, (rows * g + kVecBlock - 1) / kVecBlock);
+    return static_cast<int>((want + unit - 1) / unit * unit);
+}
+
+// Rows r < n of a layer's stacked pre-activations: Z += b (if b), H = silu(Z);
+// the tangent rows: Z = W0's row of the direction in layer 0 (W0 set), H =
+// silu'(z) Z with z the sample's primal pre-activation.
+__global__ void __launch_bounds__(kVecBlock) act_rows_kernel(int64_t n, int C, const float *__restrict__ b,
+                                                             const float *__restrict__ W0, const DirSet ds,
+                                                             float *__restrict__ Z, float *__restrict__ H)
+{
+    const int64_t tot = n * C, step = static_cast<int64_t>(gridDim.x) * kVecBlock * 4;
+    const int64_t e0 = (static_cast<int64_t>(blockIdx.x) * kVecBlock + threadIdx.x) * 4;
+    const int c = static_cast<int>(e0 % C);
+    F4 bias{}, w0[kMaxDirs] = {};
+    if (b) bias = ld4(b + c);
+#pragma unroll
+    for (int k = 0; k < kMaxDirs; ++k)
+        if (W0 && k < ds.K) w0[k] = ld4(W0 + static_cast<int64_t>(ds.dir[k]) * C + c);
+    for (int64_t e = e0; e < tot; e += step) {
+        F4 z = ld4(Z + e), h, g;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            z.v[q] = b ? z.v[q] + bias.v[q] : z.v[q];
+            h.v[q] = silu_f(z.v[q]);
+            g.v[q] = silu_grad_f(z.v[q]);
+        }
+        if (b) {
+            st4(Z + e, z);
+            st4(H + e, h);
+        }
+#pragma unroll
+        for (int k = 0; k < kMaxDirs; ++k) {
+            if (k >= ds.K) break;
+            const int64_t o = (1 + k) * tot + e;
+            F4 dz = W0 ? w0[k] : ld4(Z + o);
+            if (W0) st4(Z + o, dz);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) dz.v[q] = g.v[q] * dz.v[q];
+            st4(H + o, dz);
+        }
+    }
+}
+
+// dact_bwd_kernel's arithmetic, and per block the column sums of the parts it
+// writes: psum[(part gridDim.x + block) C + c], part 0 the primal rows, 1 + k
+// direction k (those only if all_parts).
+__global__ void __launch_bounds__(kVecBlock) dact_bwd_vec_kernel(int64_t n, int K, int C, const float *__restrict__ Abar,
+                                                                 const float *__restrict__ Zs, float *__restrict__ Zbar,
+                                                                 float *__restrict__ psum, int all_parts)
+{
+    extern __shared__ float s_col[];  // [C]
+    const int64_t tot = n * C, step = static_cast<int64_t>(gridDim.x) * kVecBlock * 4;
+    const int64_t e0 = (static_cast<int64_t>(blockIdx.x) * kVecBlock + threadIdx.x) * 4;
+    const int c = static_cast<int>(e0 % C);
+    F4 sum[1 + kMaxDirs] = {};
+    for (int64_t e = e0; e < tot; e += step) {
+        const F4 z = ld4(Zs + e), a0 = ld4(Abar + e);
+        F4 zb, d1, d2;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float sg = 1.0f / (1.0f + expf(-z.v[q]));
+            d1.v[q] = sg * (1.0f + z.v[q] * (1.0f - sg));
+            d2.v[q] = sg * (1.0f - sg) * (2.0f + z.v[q] * (1.0f - 2.0f * sg));
+            zb.v[q] = a0.v[q] * d1.v[q];
+        }
+#pragma unroll
+        for (int k = 0; k < kMaxDirs; ++k) {
+            if (k >= K) break;
+            const int64_t o = (1 + k) * tot + e;
+            const F4 ak = ld4(Abar + o), zk = ld4(Zs + o);
+            F4 out;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                zb.v[q] = fmaf(ak.v[q] * d2.v[q], zk.v[q], zb.v[q]);
+                out.v[q] = ak.v[q] * d1.v[q];
+                sum[1 + k].v[q] += out.v[q];
+            }
+            st4(Zbar + o, out);
+        }
+        st4(Zbar + e, zb);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sum[0].v[q] += zb.v[q];
+    }
+    // threads with the same columns, in thread order: g threads apart when g <= 256
+    const int g = C / 4, parts = all_parts ? 1 + K : 1;
+    for (int p = 0; p < parts; ++p) {
+        for (int i = threadIdx.x; i < C; i += kVecBlock) s_col[i] = 0.0f;
+        __syncthreads();
+        for (int r = 0; r * g < kVecBlock + g; ++r) {  // one run of g consecutive threads at a time: distinct columns
+            const int first = r * g;
+            if (static_cast<int>(threadIdx.x) >= first && static_cast<int>(threadIdx.x) < first + g) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float v = 0.0f;
+#pragma unroll
+                    for (int k = 0; k <= kMaxDirs; ++k)
+                        if (k == p) v = sum[k].v[q];
+                    s_col[c + q] += v;
+                }
+            }
+            __syncthreads();
+        }
+        float *dst = psum + (static_cast<int64_t>(p) * gridDim.x + blockIdx.x) * C;
+        for (int i = threadIdx.x; i < C; i += kVecBlock) dst[i] = s_col[i];
+        __syncthreads();
+    }
+}
+
+// out[c] (part 0) and gW0[dir_k C + c] += (part 1 + k): the blocks' column sums
+// in block order, a warp of columns per block.
+__global__ void __launch_bounds__(256) col_parts_kernel(int blocks, int C, const float *__restrict__ psum, const DirSet ds,
+                                                        float *__restrict__ out, float *__restrict__ gW0)
+{
+    __shared__ float s_part[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x * 32 + lane, p = blockIdx.y;
+    float s = 0.0f;
+    if (c < C)
+        for (int b = w; b < blocks; b += 8) s += psum[(static_cast<int64_t>(p) * blocks + b) * C + c];
+    s_part[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && c < C) {
+        s = 0.0f;
+        for (int q = 0; q < 8; ++q) s += s_part[q][lane];
+        if (p == 0) out[c] = s;
+        else gW0[static_cast<int64_t>(ds.dir[p - 1]) * C + c] += s;
+    }
+}
+
 // Layer 0's weight gradient from the tangents: row j_k of dW_0 gains the
 // column sums of direction k's adjoint rows (dh_0^k = e_{j_k}).
 __global__ void dir_rows_kernel(int64_t n, int C, const float *__restrict__ Zbar, const DirSet ds, float *__restrict__ gW0)
@@ -595,6 +779,8 @@ void launch_tiled(int M, int N, int K, const float *A, int lda, const float *B, 
         gemm4_kernel<TA, TB><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, bias, Z, H, ldc, act, kchunk, bias_rows);
 }
 
+bool aligned16(const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }  // NULL is
+
 // C = op(A) op(B) with the epilogue of store_out (bias and activation on
 // rows m < bias_rows; every row when bias_rows < 0).
 template <bool TA, bool TB>
@@ -605,6 +791,11 @@ cudaError_t gemm(int M, int N, int K, const float *A, int lda, const float *B, i
     if (!TA && N == 1) {
         rowvec_kernel<<<grid_for(static_cast<int64_t>(M) * 32), 256, 0, s>>>(M, K, A, lda, B, ldb, bias, Z, H, ldc, act,
                                                                              bias_rows);
+    } else if (!TA && !TB && K <= kSmallK && bias_rows >= M && N % 4 == 0 && N <= 1024 && ldb % 4 == 0 && ldc % 4 == 0 &&
+               aligned16(B) && aligned16(bias) && aligned16(Z) && aligned16(H)) {
+        const int rows = std::max(1, 1024 / N);  // 256 threads, or N / 4 of them past 1024 columns
+        smallk4_kernel<<<static_cast<int>(std::min<int64_t>(1216, (M + rows - 1) / rows)), 256, 0, s>>>(M, N, K, A, lda, B, ldb,
+                                                                                                     bias, Z, H, ldc, act);
     } else if (!TA && K <= kSmallK) {
         smallk_kernel<TB><<<grid_for(static_cast<int64_t>(M) * N), 256, 0, s>>>(M, N, K, A, lda, B, ldb, bias, Z, H,
                                                                                 ldc, act, bias_rows);
@@ -994,21 +1185,6 @@ cudaError_t mlp_loss_grad_tc(const MlpLayout &L, const float *params, const floa
     return cudaGetLastError();
 }
 
-namespace {
-// Rows r < n of a layer's stacked pre-activations: Z += b, H = silu(Z).
-__global__ void bias_act_rows_kernel(int64_t n, int C, const float *__restrict__ b, float *__restrict__ Z,
-                                     float *__restrict__ H)
-{
-    const int64_t tot = n * C;
-    for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < tot;
-         e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const float z = Z[e] + b[e % C];
-        Z[e] = z;
-        H[e] = silu_f(z);
-    }
-}
-}  // namespace
-
 size_t mlp_train_floats_d_tc(const MlpLayout &L, int64_t n, int K)
 {
     const int nl = static_cast<int>(L.sizes.size()) - 1, W = L.sizes[1];
@@ -1019,6 +1195,7 @@ size_t mlp_train_floats_d_tc(const MlpLayout &L, int64_t n, int K)
     f += 2 * static_cast<size_t>(W) * Rt;                                                   // H^T, Zbar^T
     f += static_cast<size_t>(nl - 2) * W * W;                                               // W_l^T
     f += static_cast<size_t>(std::max(kTcMaxSlices, kMaxSlices)) * W * W;                   // split-K partials
+    f += static_cast<size_t>(K + 1) * vec_grid(n, W) * W;                                   // column sums of Zbar
     return f + 64;
 }
 
@@ -1055,6 +1232,7 @@ cudaError_t mlp_loss_grad_d_tc(const MlpLayout &L, const float *params, const fl
     float *Abar = take(static_cast<size_t>(Rt) * W), *Zbar = take(static_cast<size_t>(Rt) * W);
     float *Ht = take(static_cast<size_t>(W) * Rt), *Zt = take(static_cast<size_t>(W) * Rt);
     for (int l = 1; l < nl - 1; ++l) WT[l] = take(static_cast<size_t>(W) * W);
+    float *psum = take(static_cast<size_t>(K + 1) * vec_grid(n, W) * W);
     float *ws = p;
     cudaError_t e;
     const dim3 tb(32, 8);
@@ -1093,12 +1271,11 @@ cudaError_t mlp_loss_grad_d_tc(const MlpLayout &L, const float *params, const fl
                                    static_cast<int>(n));
             if (e != cudaSuccess) return e;
             if (l == 0 && K > 0)
-                tangent_first_kernel<<<grid_for(K * n * out), 256, 0, s>>>(n, out, params + L.w_off[0], ds, Zs[0], Hs[0]);
+                act_rows_kernel<<<vec_grid(n, W), kVecBlock, 0, s>>>(n, W, nullptr, params + L.w_off[0], ds, Zs[0], Hs[0]);
         } else {
             const auto r = product(Hs[l - 1], W, WT[l], W, R, W, W, 1, Zs[l]);
             if ((e = r.first) != cudaSuccess) return e;
-            bias_act_rows_kernel<<<grid_for(n * W), 256, 0, s>>>(n, W, params + L.b_off[l], Zs[l], Hs[l]);
-            if (K > 0) tangent_act_kernel<<<grid_for(K * n * W), 256, 0, s>>>(n, K, W, Zs[l], Hs[l]);
+            act_rows_kernel<<<vec_grid(n, W), kVecBlock, 0, s>>>(n, W, params + L.b_off[l], nullptr, ds, Zs[l], Hs[l]);
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -1125,8 +1302,10 @@ cudaError_t mlp_loss_grad_d_tc(const MlpLayout &L, const float *params, const fl
             sum_slices_t_kernel<<<grid_for(static_cast<int64_t>(W) * W), 256, 0, s>>>(W, W, r.second, ws,
                                                                                      grad + L.w_off[l]);
         }
-        if (l == 0 && K > 0) dir_rows_kernel<<<dim3(out, K), 256, 0, s>>>(n, out, Zbar, ds, grad + L.w_off[0]);
-        colsum_kernel<<<out, 256, 0, s>>>(static_cast<int>(n), out, Zbar, grad + L.b_off[l]);
+        if (l == nl - 1) colsum_kernel<<<out, 256, 0, s>>>(static_cast<int>(n), out, Zbar, grad + L.b_off[l]);
+        else  // the column sums that dact_bwd_vec_kernel left when it wrote Zbar
+            col_parts_kernel<<<dim3((W + 31) / 32, l == 0 ? 1 + K : 1), 256, 0, s>>>(vec_grid(n, W), W, psum, ds,
+                                                                                   grad + L.b_off[l], grad + L.w_off[0]);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (l > 0) {
             if (l == nl - 1) {
@@ -1137,7 +1316,7 @@ cudaError_t mlp_loss_grad_d_tc(const MlpLayout &L, const float *params, const fl
                 e = product(Zbar, W, params + L.w_off[l], W, R, W, W, 1, Abar).first;
             }
             if (e != cudaSuccess) return e;
-            dact_bwd_kernel<<<grid_for(n * in), 256, 0, s>>>(n, K, in, Abar, Zs[l - 1], Zbar);
+            dact_bwd_vec_kernel<<<vec_grid(n, W), kVecBlock, W * sizeof(float), s>>>(n, K, W, Abar, Zs[l - 1], Zbar, psum, l == 1);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     }
