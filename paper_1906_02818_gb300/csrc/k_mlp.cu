@@ -1050,6 +1050,7 @@ bool mlp_tc_supported(const MlpLayout &L)
 
 namespace {
 constexpr int kTcMaxSlices = 32;
+constexpr int kTcMaxSlicesD = 48;  // of the stacked rows: 96 CTAs of 256 columns at width 256
 int64_t round4(int64_t n) { return (n + 3) / 4 * 4; }
 }  // namespace
 
@@ -1061,7 +1062,6 @@ size_t mlp_train_floats_tc(const MlpLayout &L, int64_t n)
     for (int l = 0; l < nl; ++l) f += 2 * static_cast<size_t>(n) * L.sizes[l + 1];  // Z, H
     f += static_cast<size_t>(nl - 1) * W * nt;                                      // H^T of the hidden layers
     f += 3 * static_cast<size_t>(n) * W + 2 * static_cast<size_t>(W) * nt;           // dH, dZ[2], dZt[2]
-    f += static_cast<size_t>(nl - 2) * W * W;                                        // W_l^T
     const int in0 = L.sizes[0];
     f += static_cast<size_t>(std::max(kTcMaxSlices, kMaxSlices)) * std::max(W, in0) * W;  // split-K partials
     return f + 64;  // 16-byte alignment of the pieces
@@ -1083,7 +1083,7 @@ cudaError_t mlp_loss_grad_tc(const MlpLayout &L, const float *params, const floa
         p += (count + 3) / 4 * 4;
         return q;
     };
-    std::vector<float *> Zp(nl), Hp(nl), Ht(nl - 1), WT(nl - 1, nullptr);
+    std::vector<float *> Zp(nl), Hp(nl), Ht(nl - 1);
     for (int l = 0; l < nl; ++l) {
         Zp[l] = take(static_cast<size_t>(n) * L.sizes[l + 1]);
         Hp[l] = take(static_cast<size_t>(n) * L.sizes[l + 1]);
@@ -1092,7 +1092,6 @@ cudaError_t mlp_loss_grad_tc(const MlpLayout &L, const float *params, const floa
     float *dH = take(static_cast<size_t>(n) * W);
     float *dZ[2] = {take(static_cast<size_t>(n) * W), take(static_cast<size_t>(n) * W)};
     float *dZt[2] = {take(static_cast<size_t>(W) * nt), take(static_cast<size_t>(W) * nt)};
-    for (int l = 1; l < nl - 1; ++l) WT[l] = take(static_cast<size_t>(W) * W);
     float *ws = p;
     cudaError_t e;
     const dim3 tb(32, 8);
@@ -1104,9 +1103,6 @@ cudaError_t mlp_loss_grad_tc(const MlpLayout &L, const float *params, const floa
     TfGemmArgs base{};
     base.err = err;
     base.cap = cap;
-    // W_l^T (out x in, K-major over in) of the width -> width layers
-    for (int l = 1; l < nl - 1; ++l)
-        if ((e = transpose(W, W, params + L.w_off[l], W, WT[l], W)) != cudaSuccess) return e;
     // forward
     e = gemm<false, false>(static_cast<int>(n), W, n_in, x, n_in, params + L.w_off[0], W, params + L.b_off[0], Zp[0],
                            Hp[0], W, 1, s);
@@ -1115,7 +1111,7 @@ cudaError_t mlp_loss_grad_tc(const MlpLayout &L, const float *params, const floa
     for (int l = 1; l < nl - 1; ++l) {
         TfGemmArgs a = base;
         a.A = Hp[l - 1]; a.lda = W;
-        a.B = WT[l]; a.ldb = W;
+        a.B = params + L.w_off[l]; a.ldb = W; a.tb = true;
         a.M = n; a.N = W; a.K = W; a.kchunk = W;
         a.mode = kTfFwd;
         a.bias = params + L.b_off[l];
@@ -1192,9 +1188,7 @@ size_t mlp_train_floats_d_tc(const MlpLayout &L, int64_t n, int K)
     size_t f = 0;
     for (int l = 0; l < nl; ++l) f += 2 * static_cast<size_t>(round4(R * L.sizes[l + 1]));  // Z, H (stacked)
     f += 2 * static_cast<size_t>(Rt) * W;                                                   // Abar, Zbar
-    f += 2 * static_cast<size_t>(W) * Rt;                                                   // H^T, Zbar^T
-    f += static_cast<size_t>(nl - 2) * W * W;                                               // W_l^T
-    f += static_cast<size_t>(std::max(kTcMaxSlices, kMaxSlices)) * W * W;                   // split-K partials
+    f += static_cast<size_t>(std::max(kTcMaxSlicesD, kMaxSlices)) * W * W;                  // split-K partials
     f += static_cast<size_t>(K + 1) * vec_grid(n, W) * W;                                   // column sums of Zbar
     return f + 64;
 }
@@ -1224,31 +1218,26 @@ cudaError_t mlp_loss_grad_d_tc(const MlpLayout &L, const float *params, const fl
         p += (count + 3) / 4 * 4;
         return q;
     };
-    std::vector<float *> Zs(nl), Hs(nl), WT(nl - 1, nullptr);
+    std::vector<float *> Zs(nl), Hs(nl);
     for (int l = 0; l < nl; ++l) {
         Zs[l] = take(static_cast<size_t>(R) * L.sizes[l + 1]);
         Hs[l] = take(static_cast<size_t>(R) * L.sizes[l + 1]);
     }
     float *Abar = take(static_cast<size_t>(Rt) * W), *Zbar = take(static_cast<size_t>(Rt) * W);
-    float *Ht = take(static_cast<size_t>(W) * Rt), *Zt = take(static_cast<size_t>(W) * Rt);
-    for (int l = 1; l < nl - 1; ++l) WT[l] = take(static_cast<size_t>(W) * W);
     float *psum = take(static_cast<size_t>(K + 1) * vec_grid(n, W) * W);
     float *ws = p;
     cudaError_t e;
-    const dim3 tb(32, 8);
-    auto transpose = [&](int64_t rows, int cols, const float *src, int64_t lds, float *dst, int64_t ldd) {
-        const dim3 gt(static_cast<unsigned>((rows + 31) / 32), static_cast<unsigned>((cols + 31) / 32));
-        transpose_kernel<<<gt, tb, 0, s>>>(rows, cols, src, lds, dst, ldd);
-        return cudaGetLastError();
-    };
     TfGemmArgs base{};
     base.err = err;
     base.cap = cap;
     base.mode = kTfPart;
-    // C [M x N] = A [M x Kd] B [N x Kd]^T into P (row-major, ld N); split K when slices > 1
-    auto product = [&](const float *A, int64_t lda, const float *B, int64_t ldb, int64_t M, int N, int Kd, int slices,
-                       float *P) {
+    // C [M x N] = A [M x Kd] B [N x Kd]^T into P (row-major, ld N); A as [Kd x M] if ta, B as [Kd x N] if tb;
+    // split K when slices > 1
+    auto product = [&](bool ta, const float *A, int64_t lda, bool tb, const float *B, int64_t ldb, int64_t M, int N, int Kd,
+                       int slices, float *P) {
         TfGemmArgs a = base;
+        a.ta = ta;
+        a.tb = tb;
         a.A = A; a.lda = lda;
         a.B = B; a.ldb = ldb;
         a.M = M; a.N = N; a.K = Kd;
@@ -1258,8 +1247,6 @@ cudaError_t mlp_loss_grad_d_tc(const MlpLayout &L, const float *params, const fl
         cudaError_t r = tf32_gemm(a, sl, s);
         return std::make_pair(r, sl);
     };
-    for (int l = 1; l < nl - 1; ++l)
-        if ((e = transpose(W, W, params + L.w_off[l], W, WT[l], W)) != cudaSuccess) return e;
     // forward
     for (int l = 0; l < nl; ++l) {
         const int in = L.sizes[l], out = L.sizes[l + 1];
@@ -1273,7 +1260,7 @@ cudaError_t mlp_loss_grad_d_tc(const MlpLayout &L, const float *params, const fl
             if (l == 0 && K > 0)
                 act_rows_kernel<<<vec_grid(n, W), kVecBlock, 0, s>>>(n, W, nullptr, params + L.w_off[0], ds, Zs[0], Hs[0]);
         } else {
-            const auto r = product(Hs[l - 1], W, WT[l], W, R, W, W, 1, Zs[l]);
+            const auto r = product(false, Hs[l - 1], W, true, params + L.w_off[l], W, R, W, W, 1, Zs[l]);
             if ((e = r.first) != cudaSuccess) return e;
             act_rows_kernel<<<vec_grid(n, W), kVecBlock, 0, s>>>(n, W, params + L.b_off[l], nullptr, ds, Zs[l], Hs[l]);
         }
@@ -1293,14 +1280,12 @@ cudaError_t mlp_loss_grad_d_tc(const MlpLayout &L, const float *params, const fl
                                                grad + L.w_off[l], out, 0, s);
             if (e != cudaSuccess) return e;
         } else {
-            // dW_l^T [out x in] = Zbar^T H_{l-1}: both transposed to K-major over the stacked rows
-            if ((e = transpose(R, W, Zbar, W, Zt, Rt)) != cudaSuccess) return e;
-            if ((e = transpose(R, W, hin, W, Ht, Rt)) != cudaSuccess) return e;
-            const int slices0 = static_cast<int>(std::min<int64_t>(kTcMaxSlices, std::max<int64_t>(1, (R + 255) / 256)));
-            const auto r = product(Zt, Rt, Ht, Rt, W, W, static_cast<int>(R), slices0, ws);
+            // dW_l [in x out] = H_{l-1}^T Zbar over the stacked rows, both as they lie
+            const int slices0 = static_cast<int>(std::min<int64_t>(kTcMaxSlicesD, std::max<int64_t>(1, (R + 255) / 256)));
+            const auto r = product(true, hin, W, true, Zbar, W, W, W, static_cast<int>(R), slices0, ws);
             if ((e = r.first) != cudaSuccess) return e;
-            sum_slices_t_kernel<<<grid_for(static_cast<int64_t>(W) * W), 256, 0, s>>>(W, W, r.second, ws,
-                                                                                     grad + L.w_off[l]);
+            const int64_t count = static_cast<int64_t>(W) * W;
+            sum_slices_kernel<<<grid_for(count), 256, 0, s>>>(count, r.second, ws, grad + L.w_off[l]);
         }
         if (l == nl - 1) colsum_kernel<<<out, 256, 0, s>>>(static_cast<int>(n), out, Zbar, grad + L.b_off[l]);
         else  // the column sums that dact_bwd_vec_kernel left when it wrote Zbar
@@ -1313,7 +1298,7 @@ cudaError_t mlp_loss_grad_d_tc(const MlpLayout &L, const float *params, const fl
                                       nullptr, Abar, in, 0, s);
             } else {
                 // Abar [R x in] = Zbar W_l^T: B = W_l [in x out], K-major over out
-                e = product(Zbar, W, params + L.w_off[l], W, R, W, W, 1, Abar).first;
+                e = product(false, Zbar, W, false, params + L.w_off[l], W, R, W, W, 1, Abar).first;
             }
             if (e != cudaSuccess) return e;
             dact_bwd_vec_kernel<<<vec_grid(n, W), kVecBlock, W * sizeof(float), s>>>(n, K, W, Abar, Zs[l - 1], Zbar, psum, l == 1);

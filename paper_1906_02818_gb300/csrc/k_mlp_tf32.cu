@@ -1,7 +1,9 @@
 // Training GEMMs of the pricing surrogate on the 5th-generation tensor cores
 // (back-propagation through the network, Sec. I.A.3, on the DNN-layer
-// analogue of Sec. III.C): C[M x N] = A[M x K] B[N x K]^T with both operands
-// K-major FP32 in global memory, FP32 accumulation in tensor memory.
+// analogue of Sec. III.C): C[M x N] = A[M x K] B[N x K]^T, FP32 accumulation
+// in tensor memory.  Each operand lies in global memory as written (K-major)
+// or transposed (A [K x M], B [K x N]); the loaders transpose while staging,
+// so no product needs a transposed copy.
 //
 // Three-pass TF32 ("3xTF32"): each operand is split into hi = x with its low
 // 13 mantissa bits cleared (exact in TF32) and lo = x - hi (exact in FP32,
@@ -9,13 +11,17 @@
 // hi*hi + hi*lo + lo*hi; the dropped lo*lo term and the TF32 reading of lo
 // leave a relative error near 2^-21 per product, FP32-like.
 //
-// One CTA computes a 128 x 64 tile.  Eight loader warps load their share of
-// each 32-wide K chunk two chunks ahead into registers and stage it (A: 128
-// rows, B: 64 rows, 128-byte rows, 128-byte swizzle) as hi and lo planes in
-// one of two stages, then arrive on the stage's `full` mbarrier; one lane of
-// a ninth warp waits on it, issues the chunk's 12 MMAs (4 K-steps of 8, 3
-// passes) and commits them to the stage's `empty` mbarrier, on which the
-// loaders wait before refilling the stage.  The epilogue (loader warps)
+// One CTA computes a 128 x BN tile, BN = 256, 128 or 64 (tf32_gemm picks the
+// widest that still fills a good part of the SMs: a wider tile loads, splits
+// and stages A once where a 64-wide one does it four times for 256 columns).
+// Eight loader warps load their share of each 32-wide K chunk two chunks ahead
+// into registers and stage it (128-byte rows, 128-byte swizzle) as hi and lo
+// planes in one of two stages, then arrive on the stage's `full` mbarrier; one
+// lane of a ninth warp waits on it, issues the chunk's 12 MMAs (4 K-steps of
+// 8, 3 passes) and commits them to the stage's `empty` mbarrier, on which the
+// loaders wait before refilling the stage.  At BN = 256 the MMAs of a chunk
+// (1536 cycles) cover the loads of the next (48 KB); at 64 the tile is bound
+// by latency: 12288 x 256 x 256 took 33 us.  The epilogue (loader warps)
 // reads the accumulator (TMEM lane = row), writes the transposed output from
 // registers, stages the tile in shared memory for coalesced row-major
 // stores, and applies one of:
@@ -31,11 +37,19 @@
 namespace gbmc {
 namespace mtf {
 
-constexpr int kBM = 128, kBN = 64, kBK = 32, kThreads = 256;
+constexpr int kBM = 128, kBK = 32, kThreads = 256;
 constexpr int kATile = kBM * kBK * 4;                  // 16 KB per plane
-constexpr int kBTile = kBN * kBK * 4;                  // 8 KB per plane
-constexpr int kStage = 2 * kATile + 2 * kBTile;        // hi + lo of A and B
-constexpr int kSmem = 1024 + 2 * kStage + 64;          // align pad, 2 stages, barriers + TMEM slot
+template <int BN>
+struct Tile {
+    static constexpr int kBTile = BN * kBK * 4;                // per plane
+    static constexpr int kStage = 2 * kATile + 2 * kBTile;     // hi + lo of A and B
+    static constexpr int kCStride = BN + 4;                    // row stride of the staged output tile (floats)
+    static constexpr int kOut = kBM * kCStride * 4;
+    static constexpr int kBody = 2 * kStage > kOut ? 2 * kStage : kOut;
+    static constexpr int kSmem = 1024 + kBody + 64;            // align pad, 2 stages (then the output tile), barriers + TMEM slot
+    static constexpr int kALoads = kBM * 8 / kThreads;         // float4 of A per thread and chunk
+    static constexpr int kBLoads = BN * 8 / kThreads;          // float4 of B per thread and chunk
+};
 
 // Byte offset of 16-byte chunk `ch` (0..7) of row `row` in a 128-byte-row,
 // 128-byte-swizzled K-major tile (8-row groups of 1024 bytes).
@@ -74,15 +88,16 @@ __device__ __forceinline__ void st4(uint32_t addr, float a, float b, float c, fl
     asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-constexpr int kALoads = kBM * 8 / kThreads;  // float4 of A per thread and chunk
-constexpr int kBLoads = kBN * 8 / kThreads;  // float4 of B per thread and chunk
-constexpr int kCStride = kBN + 4;            // row stride of the staged output tile (floats)
-
-// One K chunk's share of this thread: A rows (idx >> 3), 16-byte column
-// chunk (idx & 7), idx = threadIdx.x + i kThreads.
+// One K chunk's share of this thread.  As written: row (idx >> 3), 16-byte
+// column chunk (idx & 7), idx = threadIdx.x + i kThreads.  Transposed: lane l
+// of warp w holds K column 16 (i & 1) + (l & 15) of rows (of the operand tile)
+// R w + 8 (i >> 1) + 4 (l >> 4) .. + 3, R = rows / 8: a warp's load covers 16
+// rows of memory by whole 32-byte sectors, and the 32 lanes' scalar stores of
+// one of its four values fall into distinct banks.
+template <int BN>
 struct Frag {
-    float4 a[kALoads];
-    float4 b[kBLoads];
+    float4 a[Tile<BN>::kALoads];
+    float4 b[Tile<BN>::kBLoads];
 };
 
 // K columns kk .. kk + 3 of row gr (zero past nrows or K).
@@ -101,17 +116,23 @@ __device__ __forceinline__ float4 ld_chunk(const float *__restrict__ X, int64_t 
     return v;
 }
 
-__device__ __forceinline__ void load_frag(Frag &f, const TfGemmArgs &a, int64_t m0, int n0, int ke, int k0)
+// Operand rows r .. r + 3 (r and nrows multiples of 4) at K column kk of a transposed operand.
+__device__ __forceinline__ float4 ld_chunk_t(const float *__restrict__ X, int64_t ld, int64_t nrows, int K, int64_t r, int kk)
 {
+    if (r >= nrows || kk >= K) return make_float4(0.f, 0.f, 0.f, 0.f);
+    return __ldg(reinterpret_cast<const float4 *>(X + static_cast<int64_t>(kk) * ld + r));
+}
+
+template <int LOADS, bool T>
+__device__ __forceinline__ void load_operand(float4 (&f)[LOADS], const float *__restrict__ X, int64_t ld, int64_t nrows, int ke,
+                                             int64_t r0, int k0)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int i = 0; i < kALoads; ++i) {
+    for (int i = 0; i < LOADS; ++i) {
         const int idx = threadIdx.x + i * kThreads;
-        f.a[i] = ld_chunk(a.A, a.lda, a.M, ke, m0 + (idx >> 3), k0 + 4 * (idx & 7));
-    }
-#pragma unroll
-    for (int i = 0; i < kBLoads; ++i) {
-        const int idx = threadIdx.x + i * kThreads;
-        f.b[i] = ld_chunk(a.B, a.ldb, a.N, ke, n0 + (idx >> 3), k0 + 4 * (idx & 7));
+        if (T) f[i] = ld_chunk_t(X, ld, nrows, ke, r0 + LOADS * 4 * warp + 8 * (i >> 1) + 4 * (lane >> 4), k0 + 16 * (i & 1) + (lane & 15));
+        else f[i] = ld_chunk(X, ld, nrows, ke, r0 + (idx >> 3), k0 + 4 * (idx & 7));
     }
 }
 
@@ -127,14 +148,31 @@ __device__ __forceinline__ void store4(const float4 v, uint32_t hi_base, uint32_
     st4(lo_base + off, l0, l1, l2, l3);
 }
 
-__device__ __forceinline__ void store_frag(const Frag &f, uint32_t a_hi, uint32_t a_lo, uint32_t b_hi, uint32_t b_lo)
+template <int LOADS, bool T>
+__device__ __forceinline__ void store_operand(const float4 (&f)[LOADS], uint32_t hi_base, uint32_t lo_base)
 {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int i = 0; i < kALoads; ++i) store4(f.a[i], a_hi, a_lo, threadIdx.x + i * kThreads);
+    for (int i = 0; i < LOADS; ++i) {
+        if (!T) {
+            store4(f[i], hi_base, lo_base, threadIdx.x + i * kThreads);
+            continue;
+        }
+        const float v[4] = {f[i].x, f[i].y, f[i].z, f[i].w};
+        const int k = 16 * (i & 1) + (lane & 15);
 #pragma unroll
-    for (int i = 0; i < kBLoads; ++i) store4(f.b[i], b_hi, b_lo, threadIdx.x + i * kThreads);
+        for (int j = 0; j < 4; ++j) {
+            const int row = LOADS * 4 * warp + 8 * (i >> 1) + 4 * (lane >> 4) + j;
+            float h, l;
+            split(v[j], h, l);
+            const uint32_t off = sw128(row, k >> 2) + 4 * (k & 3);
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(hi_base + off), "f"(h) : "memory");
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(lo_base + off), "f"(l) : "memory");
+        }
+    }
 }
 
+template <int BN, bool TA, bool TB>
 __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __grid_constant__ TfGemmArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -142,13 +180,15 @@ __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __gri
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const uint32_t raw = tc::smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
+    using T = Tile<BN>;
+    constexpr int kStage = T::kStage, kBTile = T::kBTile, kCStride = T::kCStride;
     // barriers: full[2] (loaders staged the chunk), empty[2] (its MMAs completed), done, tslot,
     // xbar (the test stall)
-    const uint32_t full = base + 2 * kStage, empty = full + 16, done = empty + 16, tslot = done + 8,
+    const uint32_t full = base + T::kBody, empty = full + 16, done = empty + 16, tslot = done + 8,
                    xbar = done + 16;
     uint32_t *tslot_ptr = reinterpret_cast<uint32_t *>(smem_raw + (tslot - raw));
     const int64_t m0 = static_cast<int64_t>(blockIdx.x) * kBM;
-    const int n0 = blockIdx.y * kBN;
+    const int n0 = blockIdx.y * BN;
     const int kb = blockIdx.z * a.kchunk;
     const int ke = min(a.K, kb + a.kchunk);
     const int nk = (ke - kb + kBK - 1) / kBK;
@@ -163,7 +203,7 @@ __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __gri
         tc::mbar_init(xbar, 1);
     }
     if (warp == 0) {
-        tc::tmem_alloc(tslot, kBN);
+        tc::tmem_alloc(tslot, BN);
         tc::tmem_relinquish();
     }
     tc::fence_before_sync();
@@ -180,7 +220,7 @@ __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __gri
     if (warp == kThreads / 32) {
         // ---------------- MMA issuer (one lane) ----------------
         if (lane == 0) {
-            const uint32_t idesc = idesc_tf32(kBM, kBN);
+            const uint32_t idesc = idesc_tf32(kBM, BN);
             for (int c = 0; c < nk; ++c) {
                 const int st = c & 1;
                 const uint32_t a_hi = base + st * kStage, a_lo = a_hi + kATile, b_hi = a_lo + kATile,
@@ -204,21 +244,28 @@ __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __gri
         }
     } else {
         // ---------------- loaders: chunk c into stage c & 1, two chunks ahead ----------------
-        auto step = [&](int c, Frag &f) {
+        auto load = [&](Frag<BN> &f, int k0) {
+            load_operand<T::kALoads, TA>(f.a, a.A, a.lda, a.M, ke, m0, k0);
+            load_operand<T::kBLoads, TB>(f.b, a.B, a.ldb, a.N, ke, n0, k0);
+        };
+        auto step = [&](int c, Frag<BN> &f) {
             const int st = c & 1;
             const uint32_t a_hi = base + st * kStage, a_lo = a_hi + kATile, b_hi = a_lo + kATile,
                            b_lo = b_hi + kBTile;
             // the stage is free once the MMAs of chunk c - 2 have read it
             if (c >= 2) tc::wait_or_fail(&s_fail, empty + 8 * st, ((c - 2) >> 1) & 1u, cap);
             tc::fence_after_sync();
-            if (!s_fail) store_frag(f, a_hi, a_lo, b_hi, b_lo);
-            if (c + 2 < nk) load_frag(f, a, m0, n0, ke, kb + (c + 2) * kBK);
+            if (!s_fail) {
+                store_operand<T::kALoads, TA>(f.a, a_hi, a_lo);
+                store_operand<T::kBLoads, TB>(f.b, b_hi, b_lo);
+            }
+            if (c + 2 < nk) load(f, kb + (c + 2) * kBK);
             tc::fence_proxy_async();
             tc::mbar_arrive(full + 8 * st);
         };
-        Frag f0, f1;
-        if (nk > 0) load_frag(f0, a, m0, n0, ke, kb);
-        if (nk > 1) load_frag(f1, a, m0, n0, ke, kb + kBK);
+        Frag<BN> f0, f1;
+        if (nk > 0) load(f0, kb);
+        if (nk > 1) load(f1, kb + kBK);
         for (int c = 0; c < nk; c += 2) {
             step(c, f0);
             if (c + 1 < nk) step(c + 1, f1);
@@ -238,7 +285,7 @@ __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __gri
 
     // epilogue (warps 0..7; the issuer warp only passes the barriers).
     // Part 1: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its rows), columns
-    // 32 (w / 4) .. + 31; applies the element-wise step, writes the transposed
+    // BN/2 (w / 4) .. + BN/2 - 1; applies the element-wise step, writes the transposed
     // output (lanes = consecutive rows: coalesced) and stages the tile in
     // shared memory (the operand stages are no longer read).
     const bool worker = warp < kThreads / 32;
@@ -247,10 +294,10 @@ __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __gri
     const int row = q * 32 + lane;
     const int64_t gr = m0 + row;
     float *sC = reinterpret_cast<float *>(smem_raw + (base - raw));
-    const uint32_t taddr = tmem + (static_cast<uint32_t>(q * 32) << 16) + half * 32;
+    const uint32_t taddr = tmem + (static_cast<uint32_t>(q * 32) << 16) + half * (BN / 2);
     if (worker) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
+#pragma unroll 1
+        for (int h = 0; h < BN / 32; ++h) {
             float v[16];
             if (live) {
                 tc::tmem_ld16(taddr + 16 * h, v);
@@ -259,7 +306,7 @@ __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __gri
 #pragma unroll
                 for (int e = 0; e < 16; ++e) v[e] = 0.0f;
             }
-            const int c0 = half * 32 + 16 * h;
+            const int c0 = half * (BN / 2) + 16 * h;
             const bool rok = live && gr < a.M;
             if (a.mode == kTfFwd) {
 #pragma unroll
@@ -285,9 +332,9 @@ __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __gri
         }
     }
     __syncthreads();
-    // part 2: row-major outputs, 16 threads per 64-column row (coalesced)
-    for (int i = 0; worker && i < kBM * kBN / 4 / kThreads; ++i) {
-        const int idx = t + i * kThreads, r = idx >> 4, c4 = idx & 15;
+    // part 2: row-major outputs, BN / 4 threads per row (coalesced)
+    for (int i = 0; worker && i < kBM * BN / 4 / kThreads; ++i) {
+        const int idx = t + i * kThreads, r = idx / (BN / 4), c4 = idx % (BN / 4);
         const int64_t g = m0 + r;
         const int n = n0 + 4 * c4;
         if (!live || g >= a.M || n >= a.N) continue;
@@ -318,25 +365,47 @@ __global__ void __launch_bounds__(kThreads + 32, 1) tf32_gemm_kernel(const __gri
     __syncthreads();
     if (warp == 0) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, kBN);
+        tc::tmem_dealloc(tmem, BN);
     }
     if (t == 0 && s_fail) atomicExch(a.err, 1u);
 }
 
 }  // namespace mtf
 
-size_t tf32_gemm_smem() { return mtf::kSmem; }
+namespace {
 
+template <int BN, bool TA, bool TB>
+cudaError_t launch(const TfGemmArgs &a, int slices, cudaStream_t s)
+{
+    using namespace mtf;
+    // per device (the current one): set on every launch
+    const cudaError_t e = cudaFuncSetAttribute(tf32_gemm_kernel<BN, TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               static_cast<int>(Tile<BN>::kSmem));
+    if (e != cudaSuccess) return e;
+    const dim3 grid(static_cast<unsigned>((a.M + kBM - 1) / kBM), static_cast<unsigned>((a.N + BN - 1) / BN),
+                    static_cast<unsigned>(slices));
+    tf32_gemm_kernel<BN, TA, TB><<<grid, kThreads + 32, Tile<BN>::kSmem, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <int BN>
+cudaError_t launch_bn(const TfGemmArgs &a, int slices, cudaStream_t s)
+{
+    if (a.ta) return a.tb ? launch<BN, true, true>(a, slices, s) : cudaErrorInvalidValue;
+    return a.tb ? launch<BN, false, true>(a, slices, s) : launch<BN, false, false>(a, slices, s);
+}
+
+}  // namespace
+
+// The widest tile that divides N and still gives kTfMinCtas CTAs: below that a
+// wider tile saves loads but leaves SMs idle.
+constexpr int64_t kTfMinCtas = 80;
 cudaError_t tf32_gemm(const TfGemmArgs &a, int slices, cudaStream_t s)
 {
-    // per device (the current one): set on every launch
-    const cudaError_t e = cudaFuncSetAttribute(mtf::tf32_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(mtf::kSmem));
-    if (e != cudaSuccess) return e;
-    const dim3 grid(static_cast<unsigned>((a.M + mtf::kBM - 1) / mtf::kBM),
-                    static_cast<unsigned>((a.N + mtf::kBN - 1) / mtf::kBN), static_cast<unsigned>(slices));
-    mtf::tf32_gemm_kernel<<<grid, mtf::kThreads + 32, mtf::kSmem, s>>>(a);
-    return cudaGetLastError();
+    const int64_t rows = (a.M + mtf::kBM - 1) / mtf::kBM * slices;
+    if (a.N % 256 == 0 && rows * (a.N / 256) >= kTfMinCtas) return launch_bn<256>(a, slices, s);
+    if (a.N % 128 == 0 && rows * (a.N / 128) >= kTfMinCtas) return launch_bn<128>(a, slices, s);
+    return launch_bn<64>(a, slices, s);
 }
 
 }  // namespace gbmc

@@ -80,10 +80,11 @@ __device__ __forceinline__ float silu_grad_f(float z)
 }
 
 // Tensor-core training GEMM (k_mlp_tf32.cu): C[M x N] = A[M x K] B[N x K]^T,
-// A and B K-major FP32 (row strides lda, ldb, multiples of 4 floats; 16-byte
-// aligned bases; any K), three-pass TF32 products with FP32
-// accumulation; grid M/128 x N/64 x slices, slice z covering K columns
-// [z kchunk, (z + 1) kchunk) (kchunk a multiple of 32).  Epilogues:
+// FP32 (row strides lda, ldb, multiples of 4 floats; 16-byte aligned bases; any
+// K), three-pass TF32 products with FP32 accumulation; A K-major, or [K x M]
+// (ta, with tb; M a multiple of 4); B K-major, or [K x N] (tb; N a multiple of
+// 4); slice z of the grid covers K columns [z kchunk, (z + 1) kchunk) (kchunk a
+// multiple of 32).  Epilogues:
 constexpr int kTfFwd = 0;   // Z = C + bias, H = silu(Z) ([M x ldc]), Ht = H^T ([N x ldt])
 constexpr int kTfBwd = 1;   // dZ = C * silu'(Zin) ([M x ldc]), dZt = dZ^T ([N x ldt])
 constexpr int kTfPart = 2;  // P[z][M][N] = C of slice z
@@ -94,6 +95,7 @@ struct TfGemmArgs {
     int64_t ldb;
     int64_t M;
     int N, K, kchunk;
+    bool ta, tb;
     int mode;
     const float *bias;
     float *Z, *H, *Ht;
@@ -104,7 +106,6 @@ struct TfGemmArgs {
     unsigned int *err;   // set to 1 when a bounded wait expires
     uint32_t cap;        // polls per wait
 };
-size_t tf32_gemm_smem();
 cudaError_t tf32_gemm(const TfGemmArgs &a, int slices, cudaStream_t s);
 
 }  // namespace gbmc
