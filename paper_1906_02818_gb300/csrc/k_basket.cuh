@@ -36,11 +36,6 @@ namespace basket_detail {
 
 constexpr int kMaxWarps = 20;  // warps of the largest block (one path per thread, 640 threads)
 
-// How a step's normals are read.
-constexpr int kReadAny = 0;      // NormalReader: materialised paths, and paths of more than 2^32 Philox blocks
-constexpr int kReadAligned = 1;  // d == D: every step is D / 4 whole blocks
-constexpr int kReadShifted = 2;  // any d: two blocks in registers, lanes picked by the step's place in the first
-
 __device__ __forceinline__ float elem(const f32x2 *v, int j) { return (j & 1) ? hi_of(v[j >> 1]) : lo_of(v[j >> 1]); }
 
 struct Stats {
@@ -58,45 +53,78 @@ __device__ __forceinline__ void accumulate_payoffs(AccSlot *s_acc, const PayoffS
     }
 }
 
-// Normals 4 kb .. 4 kb + 3 of the running step for a d that need not be a
-// multiple of 4: they lie in the two consecutive blocks held, from lane o on.
-// Where a step ends inside a block, the block is kept for the next step, so
-// every block is drawn once.  A branch per normal instead (NormalReader)
-// unrolls a copy of Philox for each of them: 4.13 ms for 100,003 paths x 100
-// steps of 50 assets.
-struct ShiftedReader {
-    PathStream ps;
-    float4 cur, nxt;
-    __device__ __forceinline__ void init(uint64_t n, const RoundKeys &rk)
-    {
-        ps.init(n, rk);
-        cur = ps.normals(0u, rk).f4();
-        nxt = ps.normals(1u, rk).f4();
+// Pathwise Greeks of the European payoff (Sec. I.A.3) of one path from x_a =
+// (Lhat W)_a: the price's term, delta_a = g w_a S_a / S0_a, vega_a = g w_a S_a
+// (-sigma_a T + x_a / (log2(e) sigma_a)) and rho = g U T - T f, g the payoff's
+// slope, into the warp's slots.  U adds four assets at a time and then those
+// sums as a tree over 32 of them, the order of the d > 64 kernel's lanes, so
+// that a basket has the same U there and here.
+template <int D>
+__device__ __forceinline__ void accumulate_basket_greeks(AccSlot *s_acc, const BasketArgs &a, const BasketConst<D> &c, bool valid,
+                                                         const f32x2 (&x)[D / 2])
+{
+    const float fM = static_cast<float>(a.run.steps);
+    float part[32];
+#pragma unroll
+    for (int g = 0; g < 32; ++g) {
+        part[g] = 0.0f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int j = 4 * g + e;
+            if (j < D) part[g] = fmaf(c.ws0[j], ex2_approx(fmaf(fM, c.drift[j], elem(x, j))), part[g]);
+        }
     }
-    __device__ __forceinline__ float4 group(int o) const
-    {
-        const bool two = (o & 2) != 0, one = (o & 1) != 0;
-        const float s0 = two ? cur.z : cur.x, s1 = two ? cur.w : cur.y, s2 = two ? nxt.x : cur.z, s3 = two ? nxt.y : cur.w,
-                    s4 = two ? nxt.z : nxt.x;
-        return make_float4(one ? s1 : s0, one ? s2 : s1, one ? s3 : s2, one ? s4 : s3);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int g = 0; g < o; ++g) part[g] += part[g + o];
+    const float U = part[0], K = a.pay.strike[0];
+    const bool put = a.pay.kind[0] == MC_PUT;
+    const float f = valid ? (put ? fmaxf(K - U, 0.0f) : fmaxf(U - K, 0.0f)) : 0.0f;
+    const float g = valid ? (put ? (U < K ? -1.0f : 0.0f) : (U > K ? 1.0f : 0.0f)) : 0.0f;
+    const int nv = 2 * a.d + 2;
+    warp_accumulate(s_acc, nv, 0, f);
+    warp_accumulate(s_acc, nv, nv - 1, g * U * a.T - a.T * f);
+    // four assets at a time: deltas at 1 + a, vegas at 1 + d + a
+#pragma unroll 1
+    for (int j0 = 0; j0 < a.d; j0 += 4) {
+        float dl[4], vg[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) dl[e] = vg[e] = 0.0f;
+#pragma unroll
+        for (int jj = 0; jj < D; jj += 4) {
+            if (jj != j0) continue;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int j = jj + e;
+                if (j < a.d) {
+                    const float S = c.s0[j] * ex2_approx(fmaf(fM, c.drift[j], elem(x, j)));
+                    dl[e] = g * c.w[j] * S / c.s0[j];
+                    vg[e] = g * c.w[j] * S * fmaf(-a.sigma[j], a.T, elem(x, j) / (kLog2e * a.sigma[j]));
+                }
+            }
+        }
+        const float v[8] = {dl[0], dl[1], dl[2], dl[3], vg[0], vg[1], vg[2], vg[3]};
+        warp_accumulate8_at(s_acc, nv, v, [&](int k) {
+            const int j = j0 + (k & 3);
+            return j < a.d ? (k < 4 ? 1 + j : 1 + a.d + j) : -1;
+        });
     }
-    // On to the next pair of blocks; b: the index of the block after them.
-    __device__ __forceinline__ void advance(uint32_t b, const RoundKeys &rk)
-    {
-        cur = nxt;
-        nxt = ps.normals(b, rk).f4();
-    }
-};
+}
 
 // ------------------------------ FP32 basket -------------------------------
-template <int D, int SCHEME, bool STATS, bool SAVE, int READ, int P>
+template <int D, int SCHEME, bool STATS, bool SAVE, int READ, int P, bool GREEKS>
 __global__ void __launch_bounds__(P == 1 ? 32 * kMaxWarps : basket_threads2(D), 1)
     basket_fp32_kernel(const __grid_constant__ BasketArgs a, const BasketConst<D> c)
 {
     static_assert(!SAVE || (READ == kReadAny && P == 1), "materialised paths: one per thread");
-    __shared__ AccSlot s_acc[kMaxWarps * MC_MAX_PAYOFFS * 2];
+    static_assert(!GREEKS || (SCHEME == MC_LOG_EULER && !STATS && !SAVE), "Greeks: European payoffs under log-Euler");
+    extern __shared__ AccSlot s_greeks[];  // GREEKS: the warps' slots of price, deltas, vegas, rho
+    __shared__ AccSlot s_pays[GREEKS ? 1 : kMaxWarps * MC_MAX_PAYOFFS * 2];
     __shared__ double s_red[32];
-    for (int i = threadIdx.x; i < kMaxWarps * a.pay.n * 2; i += blockDim.x) s_acc[i] = 0.0f;
+    AccSlot *const s_acc = GREEKS ? s_greeks : s_pays;
+    const int nvals = GREEKS ? 2 * a.d + 2 : a.pay.n;
+    for (int i = threadIdx.x; i < static_cast<int>(blockDim.x >> 5) * nvals * 2; i += blockDim.x) s_acc[i] = 0.0f;
     __syncthreads();
 
     constexpr int H = D / 2;
@@ -154,7 +182,7 @@ __global__ void __launch_bounds__(P == 1 ? 32 * kMaxWarps : basket_threads2(D), 
 #pragma unroll
                     for (int q = 0; q < H; ++q) {
                         if (SCHEME == MC_EULER) dw[p][q] = pack2(0.0f, 0.0f);
-                        else x[p][q] = fadd2(x[p][q], pack2(c.drift[2 * q], c.drift[2 * q + 1]));
+                        else if (!GREEKS) x[p][q] = fadd2(x[p][q], pack2(c.drift[2 * q], c.drift[2 * q + 1]));
                     }
                     if (READ == kReadAligned) znext[p] = ps[p].normals(static_cast<uint32_t>(i) * (D / 4), a.run.rk).f4();
                 }
@@ -245,6 +273,10 @@ __global__ void __launch_bounds__(P == 1 ? 32 * kMaxWarps : basket_threads2(D), 
             }
 #pragma unroll
             for (int p = 0; p < P; ++p) {
+                if (GREEKS) {
+                    if (it + p < a.run.ppt) accumulate_basket_greeks<D>(s_acc, a, c, valid[p], x[p]);
+                    continue;
+                }
                 float u = 0.0f;
 #pragma unroll
                 for (int j = 0; j < D; ++j) {
@@ -255,13 +287,13 @@ __global__ void __launch_bounds__(P == 1 ? 32 * kMaxWarps : basket_threads2(D), 
                 avg[p] = st[p].sum * inv_m;
             }
         }
-        if (a.pay.n > 0) {
+        if (!GREEKS && a.pay.n > 0) {
 #pragma unroll
             for (int p = 0; p < P; ++p)
                 if (it + p < a.run.ppt) accumulate_payoffs(s_acc, a.pay, valid[p], uT[p], avg[p], st[p]);
         }
     }
-    if (a.pay.n > 0) block_finish(s_acc, s_red, a.pay.n, a.red);
+    if (nvals > 0) block_finish(s_acc, s_red, nvals, a.red);
 }
 
 // European payoffs under log-Euler: each thread sums its path's normals into
@@ -269,9 +301,8 @@ __global__ void __launch_bounds__(P == 1 ? 32 * kMaxWarps : basket_threads2(D), 
 // once.  Bound by drawing: the contraction of every step took two thirds of
 // 8.0 ms at 2^18 paths x 252 steps of 64 assets.
 template <int D>
-__global__ void __launch_bounds__(kBasketSumBlock) basket_sum_kernel(const __grid_constant__ BasketArgs a, const BasketConst<D> c)
+__global__ void __launch_bounds__(kBasketSumBlock, 5) basket_sum_kernel(const __grid_constant__ BasketArgs a, const BasketConst<D> c)
 {
-    constexpr int kDraw = D >= 16 ? 4 : D / 4;  // blocks summed at a time
     __shared__ float s_w[D][kBasketSumBlock];
     __shared__ AccSlot s_acc[(kBasketSumBlock / 32) * MC_MAX_PAYOFFS * 2];
     __shared__ double s_red[32];
@@ -288,15 +319,18 @@ __global__ void __launch_bounds__(kBasketSumBlock) basket_sum_kernel(const __gri
         const uint64_t n = static_cast<uint64_t>(a.run.path_offset + nl);
         for (uint32_t p = 0; p < seg.period && seg.count(p) > 0; ++p) {
             const int o = seg.lane(p), nblk = (o + d + 3) >> 2;
-            for (int g = 0; g < nblk; g += kDraw) {
-                f32x2 w[2 * kDraw];
-                sum_blocks<kDraw>(w, n, a.run.rk, a.wide, seg.first_block(p) + g, 1, seg.count(p), seg.blocks, NoRounding{});
+            for (int g = 0; g < nblk; g += 4)
+                up_to_four(nblk - g, [&](auto nb) {
+                    constexpr int NB = decltype(nb)::value;
+                    f32x2 w[2 * NB];
+                    sum_blocks<NB>(w, n, a.run.rk, a.wide, seg.first_block(p) + g, 1, seg.count(p), seg.blocks, NoRounding{});
 #pragma unroll
-                for (int e = 0; e < 4 * kDraw; ++e) {
-                    const int k = 4 * g + e - o;
-                    if (k >= 0 && k < d) s_w[k][t] = (p == 0 ? 0.0f : s_w[k][t]) + ((e & 1) ? hi_of(w[e >> 1]) : lo_of(w[e >> 1]));
-                }
-            }
+                    for (int e = 0; e < 4 * NB; ++e) {
+                        const int k = 4 * g + e - o;
+                        if (k >= 0 && k < d)
+                            s_w[k][t] = (p == 0 ? 0.0f : s_w[k][t]) + ((e & 1) ? hi_of(w[e >> 1]) : lo_of(w[e >> 1]));
+                    }
+                });
         }
         f32x2 x[D / 2];
 #pragma unroll
@@ -318,30 +352,36 @@ __global__ void __launch_bounds__(kBasketSumBlock) basket_sum_kernel(const __gri
     block_finish(s_acc, s_red, a.pay.n, a.red);
 }
 
-template <int D, int SCHEME, bool STATS, bool SAVE, int READ, int P>
+template <int D, int SCHEME, bool STATS, bool SAVE, int READ, int P, bool GREEKS = false>
 const void *basket_fn()
 {
-    return reinterpret_cast<const void *>(&basket_fp32_kernel<D, SCHEME, STATS, SAVE, READ, P>);
+    return reinterpret_cast<const void *>(&basket_fp32_kernel<D, SCHEME, STATS, SAVE, READ, P, GREEKS>);
 }
 
-template <int D, int SCHEME, bool STATS>
+template <int D, int SCHEME, bool STATS, bool GREEKS = false>
 const void *basket_pick(const BasketArgs &a)
 {
-    if constexpr (D == 64) {  // runs of more than 2^32 Philox blocks per path take this width (basket_fp32_width)
+    if constexpr (D == 64 && !GREEKS) {  // runs of more than 2^32 Philox blocks per path take this width (basket_fp32_width)
         if (a.wide) return basket_fn<D, SCHEME, STATS, false, kReadAny, 1>();
     }
     if constexpr (basket_threads2(D) == 0)
-        return a.d == D ? basket_fn<D, SCHEME, STATS, false, kReadAligned, 1>() : basket_fn<D, SCHEME, STATS, false, kReadShifted, 1>();
+        return a.d == D ? basket_fn<D, SCHEME, STATS, false, kReadAligned, 1, GREEKS>()
+                        : basket_fn<D, SCHEME, STATS, false, kReadShifted, 1, GREEKS>();
     else if (a.d == D)
-        return a.two ? basket_fn<D, SCHEME, STATS, false, kReadAligned, 2>() : basket_fn<D, SCHEME, STATS, false, kReadAligned, 1>();
+        return a.two ? basket_fn<D, SCHEME, STATS, false, kReadAligned, 2, GREEKS>()
+                     : basket_fn<D, SCHEME, STATS, false, kReadAligned, 1, GREEKS>();
     else
-        return a.two ? basket_fn<D, SCHEME, STATS, false, kReadShifted, 2>() : basket_fn<D, SCHEME, STATS, false, kReadShifted, 1>();
+        return a.two ? basket_fn<D, SCHEME, STATS, false, kReadShifted, 2, GREEKS>()
+                     : basket_fn<D, SCHEME, STATS, false, kReadShifted, 1, GREEKS>();
 }
 
 template <int D, int SCHEME>
 const void *basket_select_impl(const BasketArgs &a)
 {
     if (a.run.save) return basket_fn<D, SCHEME, false, true, kReadAny, 1>();
+    if constexpr (SCHEME == MC_LOG_EULER) {
+        if (a.greeks) return basket_pick<D, SCHEME, false, true>(a);
+    }
     if (a.pay.need_avg || a.pay.need_max || a.pay.need_min) return basket_pick<D, SCHEME, true>(a);
     if constexpr (SCHEME == MC_LOG_EULER) return reinterpret_cast<const void *>(&basket_sum_kernel<D>);
     else return basket_pick<D, SCHEME, false>(a);

@@ -1,22 +1,25 @@
-// FP32 large baskets (64 < d <= 512) and the pathwise Greeks of every FP32
-// basket: European payoffs under log-Euler, the multivariate Euler step of
-// Sec. II.A.2 summed over the steps (Segments, mc_device.cuh: the terminal
-// log-prices need the contraction of the summed normals only).
+// FP32 large baskets (64 < d <= 512): European payoffs under log-Euler, the
+// multivariate Euler step of Sec. II.A.2, and their pathwise Greeks (of any d).
 //   * CTA = 64 paths x D assets (D = 128, 256 or 512, zero-padded), 512
-//     threads.  Drawing: thread (path t mod 64, t / 64) sums every eighth
-//     Philox block of its path over the steps, four blocks at a time in
-//     registers, into W[k][path] in shared memory.
-//   * Contraction, once per tile: thread (pg, ag) owns paths 4 pg .. 4 pg + 3
-//     and the assets 128 j + 4 ag .. + 3 (j < D / 128): 4 x D / 32 sums in
+//     threads.  Contraction: thread (pg, ag) owns paths 4 pg .. 4 pg + 3 and
+//     the assets 128 j + 4 ag .. + 3 (j < D / 128): 4 x D / 32 sums in
 //     registers as asset pairs (packed FP32x2 FMAs, one instruction for two
 //     assets of one path, each lane an FP32 fma), Lhat = log2(e) sqrt(dt)
 //     diag(sigma) Lrho streamed k-major in chunks of 16 rows (cp.async double
 //     buffer); 128-asset blocks above the chunk (zero in the lower-triangular
 //     factor) are skipped.
+//   * Prices: the terminal log-prices need the contraction of the summed
+//     normals only (Segments, mc_device.cuh).  Thread (path t mod 64, t / 64)
+//     sums every eighth Philox block of its path over the steps, up to four
+//     blocks at a time in registers, into W[k][path] in shared memory; one
+//     contraction per tile.  Bound by drawing; the contraction of every step
+//     took 141 ms for 2^16 paths x 252 steps at d = 512, this 6 ms.
+//   * Greeks: contracted every step.  The payoff's slope is an indicator of
+//     U > K, and one path that falls on the other side of K by a rounding
+//     moves the vegas, sums of large terms of both signs, by 1e-4; so the
+//     Greeks keep the sums they have always been formed from.
 //   * Epilogue: log2(S_a / S0_a) = M drift_a + (Lhat W)_a, the basket,
 //     European payoffs and the pathwise delta / vega / rho of payoff 0.
-// Bound by drawing; the contraction, which ran every step before, is 5 % of
-// a tile at d = 512 and 252 steps.
 #include "mc_kernels.cuh"
 
 namespace gbmc {
@@ -25,7 +28,6 @@ namespace {
 constexpr int kP = 64;       // paths per CTA
 constexpr int kThreads = 512;
 constexpr int kKC = 16;      // factor rows per chunk
-constexpr int kDraw = 4;     // Philox blocks a thread sums at a time
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
 {
@@ -38,7 +40,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // Element e (0..3) of a thread's four consecutive assets held as two pairs.
 __device__ __forceinline__ float accel(const f32x2 *pr, int e) { return (e & 1) ? hi_of(pr[e >> 1]) : lo_of(pr[e >> 1]); }
 
-template <int D>
+template <int D, bool GREEKS>
 __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_constant__ BigArgs a)
 {
     constexpr int J = D / 128;  // 4-asset groups per thread
@@ -52,7 +54,8 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
     const int pg = t >> 5, ag = t & 31;  // a warp = one path group, 32 asset groups
     const int d = a.d, nv = a.pay.n, M = a.run.steps;
     for (int i = t; i < nv * 2; i += kThreads) s_pay[i >> 1][i & 1] = 0.0f;
-    for (int i = t; i < (2 * d + 1) * 2; i += kThreads) s_g[i >> 1][i & 1] = 0.0f;
+    if (GREEKS)
+        for (int i = t; i < (2 * d + 1) * 2; i += kThreads) s_g[i >> 1][i & 1] = 0.0f;
     const int64_t ntiles = (a.run.paths + kP - 1) / kP;
     const int nchunks = (d + kKC - 1) / kKC;
     const Segments seg(M, d);
@@ -65,23 +68,6 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
         const uint32_t rq = static_cast<uint32_t>(t) >> 6;
         const int64_t rnl = tile * kP + rp;
         const uint64_t rn = static_cast<uint64_t>(a.run.path_offset + (rnl < a.run.paths ? rnl : 0));
-        for (uint32_t p = 0; p < seg.period && seg.count(p) > 0; ++p) {
-            const int o = seg.lane(p);
-            const uint32_t nblk = static_cast<uint32_t>(o + d + 3) >> 2;
-            for (uint32_t g = rq; g < nblk; g += 8 * kDraw) {
-                f32x2 w[2 * kDraw];
-                sum_blocks<kDraw>(w, rn, a.run.rk, a.wide, seg.first_block(p) + g, 8, seg.count(p), seg.blocks, NoRounding{});
-#pragma unroll
-                for (int e = 0; e < 4 * kDraw; ++e) {
-                    const int k = static_cast<int>(4 * (g + 8 * (e >> 2))) + (e & 3) - o;
-                    if (k >= 0 && k < d) {
-                        const float v = (e & 1) ? hi_of(w[e >> 1]) : lo_of(w[e >> 1]);
-                        zs[k * kP + rp] = p == 0 ? v : zs[k * kP + rp] + v;
-                    }
-                }
-            }
-            if (p + 1 < seg.period) __syncthreads();  // a column's sums of two segments lie with different threads
-        }
         f32x2 acc2[4][J][2];  // [path][asset group][asset pair]
 #pragma unroll
         for (int p = 0; p < 4; ++p)
@@ -89,36 +75,86 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
             for (int j = 0; j < J; ++j)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) acc2[p][j][e] = pack2(0.0f, 0.0f);
-        // first factor chunk
-        for (int e = t * 4; e < kKC * D; e += kThreads * 4) cp_async16(Ls + e, a.Lp + e);
-        cp_async_commit();
-        for (int c = 0; c < nchunks; ++c) {
-            cp_async_wait_all();
-            __syncthreads();  // chunk c (and, at c = 0, the summed normals) visible
-            const float *Lc = Ls + (c & 1) * kKC * D;
-            if (c + 1 < nchunks) {  // prefetch the next chunk into the other buffer
-                float *dst = Ls + ((c + 1) & 1) * kKC * D;
-                const float *src = a.Lp + static_cast<size_t>(c + 1) * kKC * D;
-                for (int e = t * 4; e < kKC * D; e += kThreads * 4) cp_async16(dst + e, src + e);
-                cp_async_commit();
-            }
-            const int k0 = c * kKC;
-#pragma unroll 4
-            for (int kk = 0; kk < kKC; ++kk) {
-                const float4 zv = *reinterpret_cast<const float4 *>(zs + (k0 + kk) * kP + 4 * pg);
-                const f32x2 zz[4] = {pack2(zv.x, zv.x), pack2(zv.y, zv.y), pack2(zv.z, zv.z), pack2(zv.w, zv.w)};
-#pragma unroll
-                for (int j = 0; j < J; ++j) {
-                    if (128 * j + 127 < k0) continue;  // block above the diagonal chunk: zero
-                    const ulonglong2 lv = *reinterpret_cast<const ulonglong2 *>(Lc + kk * D + 128 * j + 4 * ag);
-#pragma unroll
-                    for (int p = 0; p < 4; ++p) {
-                        acc2[p][j][0] = ffma2(lv.x, zz[p], acc2[p][j][0]);
-                        acc2[p][j][1] = ffma2(lv.y, zz[p], acc2[p][j][1]);
+        // acc2 += Lhat zs over the factor's chunks
+        auto contract = [&]() {
+            // first factor chunk
+            for (int e = t * 4; e < kKC * D; e += kThreads * 4) cp_async16(Ls + e, a.Lp + e);
+            cp_async_commit();
+            for (int c = 0; c < nchunks; ++c) {
+                cp_async_wait_all();
+                __syncthreads();  // chunk c (and, at c = 0, the summed normals) visible
+                const float *Lc = Ls + (c & 1) * kKC * D;
+                if (c + 1 < nchunks) {  // prefetch the next chunk into the other buffer
+                    float *dst = Ls + ((c + 1) & 1) * kKC * D;
+                    const float *src = a.Lp + static_cast<size_t>(c + 1) * kKC * D;
+                    for (int e = t * 4; e < kKC * D; e += kThreads * 4) cp_async16(dst + e, src + e);
+                    cp_async_commit();
+                }
+                const int k0 = c * kKC;
+    #pragma unroll 4
+                for (int kk = 0; kk < kKC; ++kk) {
+                    const float4 zv = *reinterpret_cast<const float4 *>(zs + (k0 + kk) * kP + 4 * pg);
+                    const f32x2 zz[4] = {pack2(zv.x, zv.x), pack2(zv.y, zv.y), pack2(zv.z, zv.z), pack2(zv.w, zv.w)};
+    #pragma unroll
+                    for (int j = 0; j < J; ++j) {
+                        if (128 * j + 127 < k0) continue;  // block above the diagonal chunk: zero
+                        const ulonglong2 lv = *reinterpret_cast<const ulonglong2 *>(Lc + kk * D + 128 * j + 4 * ag);
+    #pragma unroll
+                        for (int p = 0; p < 4; ++p) {
+                            acc2[p][j][0] = ffma2(lv.x, zz[p], acc2[p][j][0]);
+                            acc2[p][j][1] = ffma2(lv.y, zz[p], acc2[p][j][1]);
+                        }
                     }
                 }
+                __syncthreads();  // everyone done with chunk c before it is overwritten
             }
-            __syncthreads();  // everyone done with chunk c before it is overwritten
+        };
+        if (GREEKS) {
+            NormalReader rd;
+            rd.init(rn, a.run.rk);
+            PathStream ps;
+            ps.init(rn, a.run.rk);
+            for (int i = 0; i < M; ++i) {
+                __syncthreads();  // previous step done with zs
+                for (int k = static_cast<int>(rq) * (D / 8); k < (static_cast<int>(rq) + 1) * (D / 8) && k < d; k += 4) {
+                    float4 z;
+                    if (a.exact4) {
+                        z = ps.normals((static_cast<uint32_t>(i) * (d >> 2)) + (k >> 2), a.run.rk).f4();
+                    } else {
+                        const uint64_t j0 = static_cast<uint64_t>(i) * d + k;
+                        z.x = rd.get(j0);
+                        z.y = k + 1 < d ? rd.get(j0 + 1) : 0.f;
+                        z.z = k + 2 < d ? rd.get(j0 + 2) : 0.f;
+                        z.w = k + 3 < d ? rd.get(j0 + 3) : 0.f;
+                    }
+                    zs[(k + 0) * kP + rp] = z.x;
+                    zs[(k + 1) * kP + rp] = z.y;
+                    zs[(k + 2) * kP + rp] = z.z;
+                    zs[(k + 3) * kP + rp] = z.w;
+                }
+                contract();
+            }
+        } else {
+            for (uint32_t p = 0; p < seg.period && seg.count(p) > 0; ++p) {
+                const int o = seg.lane(p);
+                const uint32_t nblk = static_cast<uint32_t>(o + d + 3) >> 2;
+                for (uint32_t g = rq; g < nblk; g += 32)
+                    up_to_four(static_cast<int>((nblk - g + 7) / 8), [&](auto nb) {
+                        constexpr int NB = decltype(nb)::value;
+                        f32x2 w[2 * NB];
+                        sum_blocks<NB>(w, rn, a.run.rk, a.wide, seg.first_block(p) + g, 8, seg.count(p), seg.blocks, NoRounding{});
+    #pragma unroll
+                        for (int e = 0; e < 4 * NB; ++e) {
+                            const int k = static_cast<int>(4 * (g + 8 * (e >> 2))) + (e & 3) - o;
+                            if (k >= 0 && k < d) {
+                                const float v = (e & 1) ? hi_of(w[e >> 1]) : lo_of(w[e >> 1]);
+                                zs[k * kP + rp] = p == 0 ? v : zs[k * kP + rp] + v;
+                            }
+                        }
+                    });
+                if (p + 1 < seg.period) __syncthreads();  // a column's sums of two segments lie with different threads
+            }
+            contract();
         }
         // ---- epilogue ----
         float Ux[4] = {0.f, 0.f, 0.f, 0.f};
@@ -151,7 +187,7 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
                 }
             }
         }
-        if (a.greeks) {
+        if (GREEKS) {
             float gs[4];
 #pragma unroll
             for (int p = 0; p < 4; ++p) {
@@ -203,7 +239,7 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
         __syncthreads();
     }
     // per-CTA partials -> FP64 sum by the last CTA
-    const int nvals = nv + (a.greeks ? 2 * d + 1 : 0);
+    const int nvals = nv + (GREEKS ? 2 * d + 1 : 0);
     for (int i = t; i < nvals * 2; i += kThreads) {
         const int k = i >> 1, m = i & 1;
         a.partials[static_cast<size_t>(blockIdx.x) * nvals * 2 + i] = k < nv ? s_pay[k][m] : s_g[k - nv][m];
@@ -254,14 +290,17 @@ int wide_width(int d) { return d <= 128 ? 128 : (d <= 256 ? 256 : 512); }
 
 size_t wide_smem(int D) { return static_cast<size_t>(D) * kP * sizeof(float) + 2 * kKC * static_cast<size_t>(D) * sizeof(float); }
 
-const void *basket_wide_fn(int D)
+template <bool GREEKS>
+static const void *wide_fn(int D)
 {
     switch (D) {
-    case 128: return reinterpret_cast<const void *>(&basket_wide_kernel<128>);
-    case 256: return reinterpret_cast<const void *>(&basket_wide_kernel<256>);
-    default: return reinterpret_cast<const void *>(&basket_wide_kernel<512>);
+    case 128: return reinterpret_cast<const void *>(&basket_wide_kernel<128, GREEKS>);
+    case 256: return reinterpret_cast<const void *>(&basket_wide_kernel<256, GREEKS>);
+    default: return reinterpret_cast<const void *>(&basket_wide_kernel<512, GREEKS>);
     }
 }
+
+const void *basket_wide_fn(int D, bool greeks) { return greeks ? wide_fn<true>(D) : wide_fn<false>(D); }
 
 int basket_wide_block() { return kThreads; }
 

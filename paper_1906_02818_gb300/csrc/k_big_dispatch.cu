@@ -11,7 +11,7 @@ int basket_big_smem();
 template <int PREC>
 cudaError_t big_prep(int d, const double *L, const double *sigma, double cfac, double sdt, double r, double dt, int M,
                      uint8_t *bimg, float *cs, float *mdrift, float *vscale, cudaStream_t s);
-const void *basket_wide_fn(int D);
+const void *basket_wide_fn(int D, bool greeks);
 int basket_wide_block();
 int wide_width(int d);
 size_t wide_smem(int D);
@@ -20,7 +20,7 @@ namespace {
 
 constexpr int kBigThreads = 576;
 
-const void *select(int prec, int d, int *smem, int *threads)
+const void *select(int prec, int d, bool greeks, int *smem, int *threads)
 {
     *threads = kBigThreads;
     switch (prec) {
@@ -31,7 +31,7 @@ const void *select(int prec, int d, int *smem, int *threads)
         const int D = wide_width(d);
         *smem = static_cast<int>(wide_smem(D));
         *threads = basket_wide_block();
-        return basket_wide_fn(D);
+        return basket_wide_fn(D, greeks);
     }
     }
 }
@@ -44,7 +44,7 @@ size_t big_bimg_bytes(int prec) { return static_cast<size_t>(32) * (prec == MC_F
 cudaError_t launch_basket_big(int prec, const BigArgs &a, int grid, cudaStream_t s)
 {
     int smem = 0, threads = 0;
-    const void *fn = select(prec, a.d, &smem, &threads);
+    const void *fn = select(prec, a.d, a.greeks != 0, &smem, &threads);
     if (smem > 0) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;

@@ -26,7 +26,52 @@ constexpr int kThreads = 128;     // paths per tile
 constexpr int kQuarter = 32;      // paths staged per outer-product pass
 constexpr int kStride = kD + 4;   // shared row stride (floats; 16-B aligned rows)
 
-template <bool EXACT>
+// A path's normals, step after step, added to W (each entry in step order).
+template <int READ>
+struct StepAdder {
+    PathStream ps;     // kReadAligned
+    NormalReader rd;   // kReadAny
+    ShiftedReader sr;  // kReadShifted
+    uint32_t blk;
+    int o;
+    __device__ __forceinline__ void init(uint64_t n, const RoundKeys &rk)
+    {
+        if (READ == kReadAligned) ps.init(n, rk);
+        if (READ == kReadAny) rd.init(n, rk);
+        if (READ == kReadShifted) {
+            sr.init(n, rk);
+            blk = 1;
+            o = 0;
+        }
+    }
+    __device__ __forceinline__ void add(int i, int d, const RoundKeys &rk, float (&W)[kD])
+    {
+        const int nb = d >> 2, rest = d - 4 * ((d - 1) / 4);
+#pragma unroll
+        for (int kb = 0; kb < kD / 4; ++kb) {
+            if (READ == kReadAny) {
+#pragma unroll
+                for (int l = 0; l < 4; ++l)
+                    if (4 * kb + l < d) W[4 * kb + l] += rd.get(static_cast<uint64_t>(i) * d + 4 * kb + l);
+            } else if (4 * kb < d) {
+                float4 z;
+                if (READ == kReadAligned) {
+                    z = ps.normals(static_cast<uint32_t>(i) * nb + kb, rk).f4();
+                } else {
+                    z = sr.group(o);
+                    if (4 * kb + 4 < d || o + rest >= 4) sr.advance(++blk, rk);
+                }
+                W[4 * kb] += z.x;
+                W[4 * kb + 1] += READ == kReadAligned || 4 * kb + 1 < d ? z.y : 0.0f;
+                W[4 * kb + 2] += READ == kReadAligned || 4 * kb + 2 < d ? z.z : 0.0f;
+                W[4 * kb + 3] += READ == kReadAligned || 4 * kb + 3 < d ? z.w : 0.0f;
+            }
+        }
+        if (READ == kReadShifted) o = (o + d) & 3;
+    }
+};
+
+template <int READ>
 __global__ void __launch_bounds__(kThreads) corr_path_kernel(const __grid_constant__ CorrArgs a, const CorrConst c)
 {
     __shared__ __align__(16) float su[kQuarter * kStride];   // w_a S_a(T) of the staged paths
@@ -57,31 +102,9 @@ __global__ void __launch_bounds__(kThreads) corr_path_kernel(const __grid_consta
         float W[kD];
 #pragma unroll
         for (int k = 0; k < kD; ++k) W[k] = 0.0f;
-        if (EXACT) {
-            const int nb = d >> 2;
-            PathStream ps;
-            ps.init(n, a.run.rk);
-            for (int i = 0; i < M; ++i) {
-#pragma unroll
-                for (int kb = 0; kb < kD / 4; ++kb) {
-                    if (kb < nb) {
-                        const float4 z = ps.normals(static_cast<uint32_t>(i) * nb + kb, a.run.rk).f4();
-                        W[4 * kb] += z.x;
-                        W[4 * kb + 1] += z.y;
-                        W[4 * kb + 2] += z.z;
-                        W[4 * kb + 3] += z.w;
-                    }
-                }
-            }
-        } else {
-            NormalReader rd;
-            rd.init(n, a.run.rk);
-            for (int i = 0; i < M; ++i) {
-#pragma unroll
-                for (int k = 0; k < kD; ++k)
-                    if (k < d) W[k] += rd.get(static_cast<uint64_t>(i) * d + k);
-            }
-        }
+        StepAdder<READ> rd;
+        rd.init(n, a.run.rk);
+        for (int i = 0; i < M; ++i) rd.add(i, d, a.run.rk, W);
         // Four passes of 32 paths (one warp each): the staging warp forms its
         // paths' terminal prices, basket and payoff; all threads then add the
         // staged paths' u W^T to their H entries.
@@ -275,29 +298,7 @@ __global__ void corr_finish_kernel(int d, int B, const double *nb, const double 
 // in registers across the launch).
 constexpr int kAsianStride = kD + 4;  // staged row stride (floats; 16-B aligned rows)
 
-__device__ __forceinline__ void asian_draw(bool exact, int i, int d, const PathStream &ps, const RoundKeys &rk,
-                                           NormalReader &rd, float (&W)[kD])
-{
-    if (exact) {
-        const int nb = d >> 2;
-#pragma unroll
-        for (int kb = 0; kb < kD / 4; ++kb) {
-            if (kb < nb) {
-                const float4 z = ps.normals(static_cast<uint32_t>(i) * nb + kb, rk).f4();
-                W[4 * kb] += z.x;
-                W[4 * kb + 1] += z.y;
-                W[4 * kb + 2] += z.z;
-                W[4 * kb + 3] += z.w;
-            }
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < kD; ++k)
-            if (k < d) W[k] += rd.get(static_cast<uint64_t>(i) * d + k);
-    }
-}
-
-template <bool EXACT>
+template <int READ>
 __global__ void __launch_bounds__(kThreads) corr_asian_kernel(const __grid_constant__ CorrArgs a, const CorrConst c)
 {
     extern __shared__ __align__(16) float s_dyn[];
@@ -331,13 +332,11 @@ __global__ void __launch_bounds__(kThreads) corr_asian_kernel(const __grid_const
         float W[kD];
 #pragma unroll
         for (int k = 0; k < kD; ++k) W[k] = 0.0f;
-        NormalReader rd;
+        StepAdder<READ> rd;
         rd.init(n, a.run.rk);
-        PathStream ps;
-        ps.init(n, a.run.rk);
         float sumU = 0.0f;
         for (int i = 0; i < M; ++i) {
-            asian_draw(EXACT, i, d, ps, a.run.rk, rd, W);
+            rd.add(i, d, a.run.rk, W);
             const float fi = static_cast<float>(i + 1);
             float U = 0.0f;
 #pragma unroll
@@ -360,7 +359,7 @@ __global__ void __launch_bounds__(kThreads) corr_asian_kernel(const __grid_const
         for (int k = 0; k < kD; ++k) W[k] = 0.0f;
         rd.init(n, a.run.rk);
         for (int i = 0; any && i < M; ++i) {
-            asian_draw(EXACT, i, d, ps, a.run.rk, rd, W);
+            rd.add(i, d, a.run.rk, W);
             const float fi = static_cast<float>(i + 1);
             float *vr = sv + t * kAsianStride, *wr = sw + t * kAsianStride;
 #pragma unroll
@@ -407,7 +406,7 @@ size_t corr_asian_smem() { return 2 * static_cast<size_t>(kThreads) * kAsianStri
 // then dP/dLrho and the Cholesky adjoint per batch in FP64 (global memory).
 constexpr int kWChunk = 64;
 
-template <bool EXACT>
+template <int READ>
 __global__ void __launch_bounds__(128) corr_wsum_kernel(const __grid_constant__ CorrArgs a, float *__restrict__ Wbuf)
 {
     const int d = a.d, M = a.run.steps;
@@ -420,7 +419,7 @@ __global__ void __launch_bounds__(128) corr_wsum_kernel(const __grid_constant__ 
             float W[kWChunk];
 #pragma unroll
             for (int k = 0; k < kWChunk; ++k) W[k] = 0.0f;
-            if (EXACT) {  // d % 4 == 0: step i's normals are blocks i d/4 .. i d/4 + d/4 - 1
+            if (READ == kReadAligned) {  // d % 4 == 0: step i's normals are blocks i d/4 .. i d/4 + d/4 - 1
                 const uint32_t nb = static_cast<uint32_t>(d >> 2);
                 for (int i = 0; i < M; ++i) {
 #pragma unroll
@@ -431,6 +430,25 @@ __global__ void __launch_bounds__(128) corr_wsum_kernel(const __grid_constant__ 
                             W[4 * kb + 1] += z.y;
                             W[4 * kb + 2] += z.z;
                             W[4 * kb + 3] += z.w;
+                        }
+                    }
+                }
+            } else if (READ == kReadShifted) {  // a step's chunk: up to one block more than its normals fill
+                for (int i = 0; i < M; ++i) {
+                    const uint64_t j0 = static_cast<uint64_t>(i) * d + c0;
+                    const uint32_t q = static_cast<uint32_t>(j0 >> 2);
+                    const int o = static_cast<int>(j0 & 3);
+                    float4 cur = ps.normals(q, a.run.rk).f4();
+#pragma unroll
+                    for (int kb = 0; kb < kWChunk / 4; ++kb) {
+                        if (c0 + 4 * kb < d) {
+                            const float4 nxt = ps.normals(q + kb + 1, a.run.rk).f4();
+                            const float4 z = shifted4(cur, nxt, o);
+                            W[4 * kb] += z.x;
+                            W[4 * kb + 1] += z.y;
+                            W[4 * kb + 2] += z.z;
+                            W[4 * kb + 3] += z.w;  // past d: not stored
+                            cur = nxt;
                         }
                     }
                 }
@@ -594,10 +612,12 @@ bool corr_asian(const CorrArgs &a) { return a.kind == MC_ASIAN_CALL || a.kind ==
 const void *corr_select(const CorrArgs &a)
 {
     if (corr_asian(a))
-        return a.exact4 ? reinterpret_cast<const void *>(&corr_asian_kernel<true>)
-                        : reinterpret_cast<const void *>(&corr_asian_kernel<false>);
-    return a.exact4 ? reinterpret_cast<const void *>(&corr_path_kernel<true>)
-                    : reinterpret_cast<const void *>(&corr_path_kernel<false>);
+        return a.read == kReadAligned   ? reinterpret_cast<const void *>(&corr_asian_kernel<kReadAligned>)
+               : a.read == kReadShifted ? reinterpret_cast<const void *>(&corr_asian_kernel<kReadShifted>)
+                                        : reinterpret_cast<const void *>(&corr_asian_kernel<kReadAny>);
+    return a.read == kReadAligned   ? reinterpret_cast<const void *>(&corr_path_kernel<kReadAligned>)
+           : a.read == kReadShifted ? reinterpret_cast<const void *>(&corr_path_kernel<kReadShifted>)
+                                    : reinterpret_cast<const void *>(&corr_path_kernel<kReadAny>);
 }
 
 size_t corr_dyn_smem(const CorrArgs &a) { return corr_asian(a) ? corr_asian_smem() : 0; }
@@ -652,8 +672,9 @@ cudaError_t launch_corr_wide(const CorrArgs &a, const CorrWide &w, int grid, cud
     const int d = a.d, B = w.batches;
     const int64_t P = a.run.paths;
     if (P > INT32_MAX) return cudaErrorInvalidValue;
-    if (a.exact4) corr_wsum_kernel<true><<<grid, 128, 0, s>>>(a, w.Wbuf);
-    else corr_wsum_kernel<false><<<grid, 128, 0, s>>>(a, w.Wbuf);
+    if (a.read == kReadAligned) corr_wsum_kernel<kReadAligned><<<grid, 128, 0, s>>>(a, w.Wbuf);
+    else if (a.read == kReadShifted) corr_wsum_kernel<kReadShifted><<<grid, 128, 0, s>>>(a, w.Wbuf);
+    else corr_wsum_kernel<kReadAny><<<grid, 128, 0, s>>>(a, w.Wbuf);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // Y = W Lhat^T: Y[p][a] = sum_b W[p][b] Lhat[a][b]

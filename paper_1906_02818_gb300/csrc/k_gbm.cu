@@ -176,11 +176,17 @@ const void *basket_select(int D, const BasketArgs &a)
     }
 }
 
-int occupancy_of(const void *fn, int block)
+int occupancy_of(const void *fn, int block, size_t smem = 0)
 {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, 0) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, smem) != cudaSuccess) return 0;
     return nb;
+}
+
+// Dynamic shared memory of a basket launch: the warps' Greek slots.
+size_t greeks_slots(const BasketArgs &a, int block)
+{
+    return a.greeks ? static_cast<size_t>(block / 32) * (2 * a.d + 2) * 2 * sizeof(AccSlot) : 0;
 }
 
 }  // namespace
@@ -205,7 +211,7 @@ int basket_fp32_width(int d, bool wide)
 
 bool basket_fp32_sums(const BasketArgs &a)
 {
-    return a.scheme == MC_LOG_EULER && !a.run.save && !a.pay.need_avg && !a.pay.need_max && !a.pay.need_min;
+    return a.scheme == MC_LOG_EULER && !a.greeks && !a.run.save && !a.pay.need_avg && !a.pay.need_max && !a.pay.need_min;
 }
 
 size_t basket_const_bytes(int D)
@@ -254,14 +260,23 @@ cudaError_t launch_basket_fp32(int D, const BasketArgs &a, const void *cst, int 
 {
     const void *fn = basket_select(D, a);
     if (!fn) return cudaErrorInvalidValue;
+    const size_t smem = greeks_slots(a, block);
+    if (smem > 0) {
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
+    }
     void *args[] = {const_cast<BasketArgs *>(&a), const_cast<void *>(cst)};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, 0, s);
+    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, s);
 }
 
 int basket_fp32_occupancy(int D, const BasketArgs &a, int block)
 {
     const void *fn = basket_select(D, a);
-    return fn ? occupancy_of(fn, block) : 0;
+    if (!fn) return 0;
+    const size_t smem = greeks_slots(a, block);
+    if (smem > 0 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+        return 0;
+    return occupancy_of(fn, block, smem);
 }
 
 }  // namespace gbmc

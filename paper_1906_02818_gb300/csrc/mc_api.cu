@@ -588,6 +588,40 @@ int factor_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const Payof
     return MC_OK;
 }
 
+// Block of an FP32 basket launch (P->bk and P->D set).  The summed-normals
+// kernel: 128.  The stepping kernel: one block per SM, as large (in whole
+// warps) as an equal share of each round of paths asks for: two paths per
+// thread where the width allows it and an SM has more than 256, else one, of
+// up to 640 threads.  Runs of less than a round, or of so few paths that the
+// block would fall under 16 warps: blocks of 128, to spread them.
+void basket_block(mc_plan *P, int64_t paths, int sms)
+{
+    BasketArgs &b = P->bk;
+    const int64_t per_sm = (paths + sms - 1) / sms;
+    const int most = b.wide || b.run.save ? 0 : basket_threads2(P->D);
+    b.two = false;
+    if (basket_fp32_sums(b)) {
+        P->block = kBasketSumBlock;
+    } else if (most > 0 && per_sm > 256) {
+        b.two = true;
+        const int64_t rounds = (per_sm + 2 * most - 1) / (2 * most);
+        P->block = static_cast<int>((per_sm + 2 * rounds - 1) / (2 * rounds) + 31) / 32 * 32;
+    } else {
+        const int64_t rounds = (per_sm + 639) / 640;
+        const int trimmed = static_cast<int>(((per_sm + rounds - 1) / rounds + 31) / 32 * 32);
+        P->block = (per_sm >= 1280 || trimmed >= 512) && per_sm >= 640 ? trimmed : 128;
+    }
+}
+
+// Two paths per thread: whole rounds of them on every SM.
+void basket_grid(mc_plan *P, int64_t paths, int sms, int *ppt)
+{
+    if (!P->bk.two) return;
+    P->grid = static_cast<int>(std::min<int64_t>(sms, (paths + P->block - 1) / P->block));
+    const int64_t round = static_cast<int64_t>(P->grid) * P->block;
+    *ppt = static_cast<int>((paths + round - 1) / round);
+}
+
 // Shared set-up of mc_plan_create and mc_simulate.  save != nullptr selects
 // the materialising kernels (no payoffs, no reduction).
 int plan_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const mc_payoff *pays, int np,
@@ -741,25 +775,7 @@ int plan_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const mc_payo
             b.wide = wide;
             b.pay = ps;
             b.red = red;
-            // The stepping kernel: one block per SM, as large (in whole warps)
-            // as an equal share of each round of paths asks for: two paths per
-            // thread where the width allows it and an SM has more than 256,
-            // else one, of up to 640 threads.  Runs of less than a round, or
-            // of so few paths that the block would fall under 16 warps: blocks
-            // of 128, to spread them.
-            const int64_t per_sm = (c->paths + di.sms - 1) / di.sms;
-            const int most = wide || save ? 0 : basket_threads2(D);
-            if (basket_fp32_sums(b)) {
-                P->block = kBasketSumBlock;
-            } else if (most > 0 && per_sm > 256) {
-                b.two = true;
-                const int64_t rounds = (per_sm + 2 * most - 1) / (2 * most);
-                P->block = static_cast<int>((per_sm + 2 * rounds - 1) / (2 * rounds) + 31) / 32 * 32;
-            } else {
-                const int64_t rounds = (per_sm + 639) / 640;
-                const int trimmed = static_cast<int>(((per_sm + rounds - 1) / rounds + 31) / 32 * 32);
-                P->block = (per_sm >= 1280 || trimmed >= 512) && per_sm >= 640 ? trimmed : 128;
-            }
+            basket_block(P, c->paths, di.sms);
             MC_CUDA(launch_scale_factor(d, P->dL, P->dsig, cfac, sdt, m->r, dt, c->scheme, P->dLp, P->ddrift, s));
             std::vector<float> Lp(tri), drift(d);
             MC_CUDA(cudaMemcpyAsync(&status, P->dstatus, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -800,10 +816,7 @@ int plan_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const mc_payo
         P->grid = static_cast<int>(tiles < resident ? tiles : resident);
     } else {
         size_grid(c->paths, P->block, resident, &P->grid, &ppt);
-        if (P->kk == K_BASKET_FP32 && P->bk.two) {  // whole rounds of two paths per thread, on every SM
-            P->grid = static_cast<int>(std::min<int64_t>(di.sms, (c->paths + P->block - 1) / P->block));
-            ppt = static_cast<int>((c->paths + static_cast<int64_t>(P->grid) * P->block - 1) / (static_cast<int64_t>(P->grid) * P->block));
-        }
+        if (P->kk == K_BASKET_FP32) basket_grid(P, c->paths, di.sms, &ppt);
     }
     P->g1.run.ppt = ppt;
     P->bk.run.ppt = ppt;
@@ -1082,15 +1095,41 @@ int mc_greeks(const mc_model *m, const mc_sim_cfg *c, const mc_payoff *pays, int
         run.steps = c->steps;
         run.save_every = 1;
         mc_plan P;
-        if ((rc = big_setup(&P, m, c, ps, run, true, s))) return rc;
-        if ((rc = plan_launch(&P, P.dout, s))) return rc;
         const int G = 2 * m->d + 1;
+        if (m->d <= 64 && c->precision == MC_FP32 && c->scheme == MC_LOG_EULER && (ps.kind[0] == MC_CALL || ps.kind[0] == MC_PUT) &&
+            blocks_fit_32(c->steps, m->d)) {
+            // a path per thread (the stepping kernel); its reduction holds the price and the G Greeks
+            if ((rc = plan_setup(&P, m, c, pays, np, nullptr, 0, s))) return rc;
+            DeviceInfo di;
+            if ((rc = device_info(&di))) return rc;
+            BasketArgs &b = P.bk;
+            b.greeks = true;
+            b.T = static_cast<float>(c->T);
+            for (int k = 0; k < m->d; ++k) b.sigma[k] = static_cast<float>(m->sigma[k]);
+            basket_block(&P, c->paths, di.sms);
+            const int resident = basket_fp32_occupancy(P.D, b, P.block) * di.sms;
+            if (resident <= 0) return fail(MC_ECUDA, "basket Greeks kernel cannot be resident");
+            int ppt = 1;
+            size_grid(c->paths, P.block, resident, &P.grid, &ppt);
+            basket_grid(&P, c->paths, di.sms, &ppt);
+            b.run.ppt = ppt;
+            MC_CUDA(cudaStreamSynchronize(s));  // the set-up's blocks go back to the cache idle
+            dfree(P.partials);
+            dfree(P.dout);
+            MC_CUDA(dev_alloc(&P.partials, static_cast<size_t>(P.grid) * (1 + G) * 2 * sizeof(float)));
+            MC_CUDA(dev_alloc(&P.dout, static_cast<size_t>(1 + G) * sizeof(mc_result)));
+            b.red.partials = P.partials;
+            b.red.out = P.dout;
+        } else if ((rc = big_setup(&P, m, c, ps, run, true, s))) {
+            return rc;
+        }
+        if ((rc = plan_launch(&P, P.dout, s))) return rc;
         std::vector<mc_result> tmp(1 + G);
         MC_CUDA(cudaMemcpyAsync(tmp.data(), P.dout, tmp.size() * sizeof(mc_result), cudaMemcpyDeviceToHost, s));
         MC_CUDA(cudaStreamSynchronize(s));
         P.idle = true;
         unsigned int e = 0;
-        MC_CUDA(cudaMemcpy(&e, P.err, sizeof e, cudaMemcpyDeviceToHost));
+        if (P.err) MC_CUDA(cudaMemcpy(&e, P.err, sizeof e, cudaMemcpyDeviceToHost));
         if (e) return fail(MC_ETIMEOUT, "a bounded wait on the tensor-core pipeline gave up");
         if (prices) prices[0] = tmp[0];
         for (int k = 0; k < G; ++k) greeks[k] = tmp[1 + k];
@@ -1195,7 +1234,7 @@ static int corr_greeks_wide(const mc_model *m, const mc_sim_cfg *c, const mc_pay
     a.run.steps = c->steps;
     a.run.save_every = 1;
     a.d = d;
-    a.exact4 = d % 4 == 0 && blocks_fit_32(c->steps, d) ? 1 : 0;
+    a.read = !blocks_fit_32(c->steps, d) ? kReadAny : d % 4 == 0 ? kReadAligned : kReadShifted;
     a.kind = pay->kind;
     a.strike = static_cast<float>(pay->strike);
     // batches of kchunk paths (a multiple of 16) for the batch-means errors
@@ -1318,7 +1357,7 @@ int mc_corr_greeks(const mc_model *m, const mc_sim_cfg *c, const mc_payoff *pay,
     a.run.steps = c->steps;
     a.run.save_every = 1;
     a.d = d;
-    a.exact4 = d % 4 == 0 && blocks_fit_32(c->steps, d) ? 1 : 0;
+    a.read = !blocks_fit_32(c->steps, d) ? kReadAny : d % 4 == 0 ? kReadAligned : kReadShifted;
     a.kind = pay->kind;
     a.strike = static_cast<float>(pay->strike);
     const int occ = corr_occupancy(a);

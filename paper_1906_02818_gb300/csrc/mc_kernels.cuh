@@ -92,6 +92,9 @@ struct BasketArgs {
     int scheme;
     bool wide;  // a path's Philox blocks pass 2^32
     bool two;   // two paths per thread
+    bool greeks;  // price, delta_a, vega_a (a < d) and rho of payoff 0, European, log-Euler: 2 d + 2 reduced values
+    float T;
+    float sigma[64];
     PayoffSet pay;
     ReduceArgs red;
 };
@@ -278,7 +281,7 @@ struct CorrConst {
 struct CorrArgs {
     PathRun run;
     int d;
-    int exact4;         // d % 4 == 0: every step is d/4 whole Philox blocks
+    int read;           // how a step's normals are read (kReadAligned: d % 4 == 0)
     int kind;           // MC_CALL or MC_PUT on U = sum_a w_a S_a(T); MC_ASIAN_CALL or
                         // MC_ASIAN_PUT on the average of U over the steps (d <= 64)
     float strike;

@@ -43,6 +43,23 @@ def test_fp32_basket_greeks_summed_normals(gb, orc, d, steps):
         assert abs(g[0, k, 0] - m) <= 2e-5 * max(abs(m), scale, np.mean(np.abs(ref[k]))), (d, k, g[0, k, 0], m)
 
 
+@pytest.mark.parametrize("d,steps,paths", [(4, 3, 50000), (5, 6, 80001), (24, 2, 60000), (30, 3, 90000), (56, 2, 70000),
+                                           (63, 1, 100001), (64, 2, 33000)])
+def test_fp32_basket_greeks_many_paths(gb, d, steps, paths):
+    """One and two paths per thread, whole and ragged last rounds: the sums over
+    all paths are those of runs of at most 8192 of them (one path per thread)."""
+    w, pays = _case(d, 2, paths, steps)
+    pr, g = gb.greeks(gbm_model(w), cfg_of(w), pays[:1])
+    total = np.zeros(2 * d + 2)
+    for lo in range(0, paths, 8192):
+        n = min(8192, paths - lo)
+        p1, g1 = gb.greeks(gbm_model(w), cfg_of(dict(w, paths=n), path_offset=lo), pays[:1])
+        total += n * np.concatenate([[p1[0][0]], np.asarray(g1)[0, :, 0]])
+    got = np.concatenate([[pr[0][0]], np.asarray(g)[0, :, 0]])
+    # the same FP32 terms in FP64 sums, rounded once per block of paths to FP32
+    assert np.max(np.abs(got - total / paths)) <= 1e-6 * np.max(np.abs(got)), (d, got - total / paths)
+
+
 @pytest.mark.parametrize("d,steps,paths", [(2, 1, 130), (3, 5, 129), (5, 3, 257), (7, 6, 128), (10, 4, 500),
                                            (18, 7, 131), (33, 2, 129), (47, 9, 127), (57, 5, 130), (63, 4, 200),
                                            (64, 3, 129)])
