@@ -88,51 +88,97 @@ struct Stats {
     float sum, umax, umin;
 };
 
-// Draws Z_i of the path of ps / rd (row `row`) into the tile at `tile`; returns the
-// dequantisation factor of the row (1 unless E4M3).
-template <int PREC, bool EXACT>
-__device__ __forceinline__ float draw_row(uint32_t tile, int row, int i, int d, const PathStream &ps,
-                                          const RoundKeys &rk, NormalReader &rd, bool valid)
+// The normals of a path, step by step, in groups of four (4 kb ..): whole
+// blocks when d = 64, else two blocks in registers and the step's place in the
+// first.  A reader with a branch per normal unrolled 64 copies of Philox: d =
+// 27 FP16, 767,916 paths x 8 steps 584 us, so 285 us; d = 13 E4M3, 33,868 x
+// 169 with a barrier 1270 us, so 429 us (there the products and the read-back
+// of the accumulator that stop at d count too).
+template <int READ>
+struct RowReader {
+    PathStream ps;     // kReadAligned
+    ShiftedReader sr;  // kReadShifted
+    WideReader wr;     // kReadAny
+    uint32_t blk;      // kReadShifted: the last block held
+    int o;             // the step's first lane
+    __device__ __forceinline__ void init(uint64_t n, const RoundKeys &rk)
+    {
+        blk = 1;
+        o = 0;
+        if (READ == kReadAligned) ps.init(n, rk);
+        else if (READ == kReadShifted) sr.init(n, rk);
+        else wr.init(n, rk);
+    }
+    // Normals 4 kb .. 4 kb + 3 of step i (called for kb = 0, 1, ... in turn).
+    __device__ __forceinline__ float4 group(int i, int kb, int d, const RoundKeys &rk)
+    {
+        if (READ == kReadAligned) return ps.normals(static_cast<uint32_t>(i) * (kN / 4) + kb, rk).f4();
+        if (4 * kb >= d) return make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float4 z = READ == kReadShifted ? sr.group(o) : wr.group(o);
+        if (4 * kb + 4 < d || o + d - 4 * kb >= 4) {  // this group used up the first block
+            if (READ == kReadShifted) sr.advance(++blk, rk);
+            else wr.advance(rk);
+        }
+        // the next step's normals
+        if (4 * kb + 1 >= d) z.y = 0.0f;
+        if (4 * kb + 2 >= d) z.z = 0.0f;
+        if (4 * kb + 3 >= d) z.w = 0.0f;
+        return z;
+    }
+    __device__ __forceinline__ void step_done(int d)
+    {
+        if (READ != kReadAligned) o = (o + d) & 3;
+    }
+};
+
+// Columns the products run over: d rounded up to whole MMAs.
+template <int PREC>
+__device__ __forceinline__ int mma_columns(int d)
+{
+    return (d + Layout<PREC>::kKStep - 1) / Layout<PREC>::kKStep * Layout<PREC>::kKStep;
+}
+
+// Draws Z_i of rd's path (row `row`) into the tile at `tile`, as far as the
+// products read it; returns the dequantisation factor of the row (1 unless
+// E4M3).  Rows past the last path (not valid): anything finite; the branch
+// keeps the compiler from drawing chunks of d = 64 side by side, for which the
+// registers of eight CTAs per SM do not suffice.
+template <int PREC, int READ>
+__device__ __forceinline__ float draw_row(uint32_t tile, int row, int i, int d, const RoundKeys &rk, RowReader<READ> &rd,
+                                          bool valid)
 {
     using Ly = Layout<PREC>;
-    auto normal8 = [&](int c0, float (&z)[8]) {
-        if (!valid) {
-#pragma unroll
-            for (int l = 0; l < 8; ++l) z[l] = 0.0f;
-        } else if (EXACT) {
-            const uint32_t q = static_cast<uint32_t>(i) * (kN / 4) + c0 / 4;
-            const float4 a = ps.normals(q, rk).f4(), b = ps.normals(q + 1, rk).f4();
-            z[0] = a.x; z[1] = a.y; z[2] = a.z; z[3] = a.w; z[4] = b.x; z[5] = b.y; z[6] = b.z; z[7] = b.w;
-        } else {
-#pragma unroll
-            for (int l = 0; l < 8; ++l)
-                z[l] = (c0 + l < d) ? rd.get(static_cast<uint64_t>(i) * d + c0 + l) : 0.0f;
-        }
-    };
+    const int cols = READ == kReadAligned ? kN : mma_columns<PREC>(d);
     if (PREC != MC_FP8E4M3) {
 #pragma unroll
         for (int cb = 0; cb < Ly::kChunks; ++cb) {
-            float z[8];
-            normal8(cb * 8, z);
-            st_shared_v4(tile + Ly::chunk_off(row, cb), pack2<PREC>(z[0], z[1]), pack2<PREC>(z[2], z[3]),
-                         pack2<PREC>(z[4], z[5]), pack2<PREC>(z[6], z[7]));
+            if (8 * cb >= cols) break;
+            float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+            if (READ != kReadAligned || valid) {
+                a = rd.group(i, 2 * cb, d, rk);
+                b = rd.group(i, 2 * cb + 1, d, rk);
+            }
+            st_shared_v4(tile + Ly::chunk_off(row, cb), pack2<PREC>(a.x, a.y), pack2<PREC>(a.z, a.w),
+                         pack2<PREC>(b.x, b.y), pack2<PREC>(b.z, b.w));
         }
+        rd.step_done(d);
         return 1.0f;
     } else {
         float z[kN];
 #pragma unroll
-        for (int cb = 0; cb < kN / 8; ++cb) {
-            float t[8];
-            normal8(cb * 8, t);
-#pragma unroll
-            for (int l = 0; l < 8; ++l) z[cb * 8 + l] = t[l];
+        for (int kb = 0; kb < kN / 4; ++kb) {
+            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (READ != kReadAligned || valid) v = rd.group(i, kb, d, rk);
+            z[4 * kb] = v.x; z[4 * kb + 1] = v.y; z[4 * kb + 2] = v.z; z[4 * kb + 3] = v.w;
         }
+        rd.step_done(d);
         float amax = 0.0f;
 #pragma unroll
         for (int j = 0; j < kN; ++j) amax = fmaxf(amax, fabsf(z[j]));
         const float s = amax > 0.0f ? 448.0f / amax : 1.0f;
 #pragma unroll
         for (int cb = 0; cb < Ly::kChunks; ++cb) {
+            if (16 * cb >= cols) break;
             const float *q = z + cb * 16;
             st_shared_v4(tile + Ly::chunk_off(row, cb), pack4_e4m3(q[0] * s, q[1] * s, q[2] * s, q[3] * s),
                          pack4_e4m3(q[4] * s, q[5] * s, q[6] * s, q[7] * s),
@@ -144,11 +190,12 @@ __device__ __forceinline__ float draw_row(uint32_t tile, int row, int i, int d, 
 }
 
 template <int PREC>
-__device__ __forceinline__ void issue_mmas(uint32_t tmem_d, uint32_t ztile, uint32_t btile)
+__device__ __forceinline__ void issue_mmas(uint32_t tmem_d, uint32_t ztile, uint32_t btile, int cols)
 {
     using Ly = Layout<PREC>;
 #pragma unroll
     for (int kk = 0; kk < Ly::kMmas; ++kk) {
+        if (kk * Ly::kKStep >= cols) break;
         const uint64_t ad = tc::smem_desc(ztile + kk * 32, Ly::kGroupBytes, Ly::kSw);
         const uint64_t bd = tc::smem_desc(btile + kk * 32, Ly::kGroupBytes, Ly::kSw);
         if (PREC == MC_FP8E4M3) tc::mma_f8(tmem_d, ad, bd, tc::idesc_e4m3(kRows, kN), kk > 0 ? 1u : 0u);
@@ -156,7 +203,7 @@ __device__ __forceinline__ void issue_mmas(uint32_t tmem_d, uint32_t ztile, uint
     }
 }
 
-template <int PREC, int SCHEME, bool STATS, bool EXACT>
+template <int PREC, int SCHEME, bool STATS, int READ>
 __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_constant__ TcArgs a, const TcConst c)
 {
     using Ly = Layout<PREC>;
@@ -198,7 +245,8 @@ __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_consta
     bool aborted = __syncthreads_or(tc::mbar_wait_bounded(mbar + 8 - 8 * a.stall, 0, a.wait_cap) ? 0 : 1) != 0;
 
     uint32_t phase = 0;
-    const int M = a.run.steps, d = a.d;
+    const int M = a.run.steps, d = READ == kReadAligned ? kN : a.d;
+    const int cols = mma_columns<PREC>(d);  // past d: zero weight, zero increments
     const float inv_m = 1.0f / static_cast<float>(M);
     const int64_t ntiles = (a.run.paths + kRows - 1) / kRows;
     const uint32_t row_taddr = tmem + (static_cast<uint32_t>(warp * 32) << 16);
@@ -207,10 +255,8 @@ __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_consta
         const int64_t nl = tile * kRows + t;
         const bool valid = nl < a.run.paths;
         const uint64_t n = static_cast<uint64_t>(a.run.path_offset + (valid ? nl : 0));
-        NormalReader rd;
+        RowReader<READ> rd;
         rd.init(n, a.run.rk);
-        PathStream ps;
-        ps.init(n, a.run.rk);
         float x[kN];
 #pragma unroll
         for (int j = 0; j < kN; ++j) x[j] = (SCHEME == MC_LOG_EULER) ? 0.0f : c.s0[j];
@@ -218,18 +264,18 @@ __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_consta
 
         float deq_cur = 1.0f, deq_next = 1.0f;
         if (!aborted) {
-            deq_cur = draw_row<PREC, EXACT>(zt[0], t, 0, d, ps, a.run.rk, rd, valid);
+            deq_cur = draw_row<PREC, READ>(zt[0], t, 0, d, a.run.rk, rd, valid);
             tc::fence_proxy_async();
         }
         __syncthreads();
         if (t == 0 && !aborted) {
             tc::fence_after_sync();
-            issue_mmas<PREC>(tmem, zt[0], bt);
+            issue_mmas<PREC>(tmem, zt[0], bt, cols);
             tc::mma_commit(mbar);
         }
         for (int i = 0; i < M && !aborted; ++i) {
             if (i + 1 < M) {
-                deq_next = draw_row<PREC, EXACT>(zt[(i + 1) & 1], t, i + 1, d, ps, a.run.rk, rd, valid);
+                deq_next = draw_row<PREC, READ>(zt[(i + 1) & 1], t, i + 1, d, a.run.rk, rd, valid);
                 tc::fence_proxy_async();
             }
             const bool ok = tc::mbar_wait_bounded(mbar, phase & 1u, a.wait_cap);
@@ -239,6 +285,7 @@ __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_consta
             float u = 0.0f;
 #pragma unroll
             for (int cc = 0; cc < kN / 16; ++cc) {
+                if (cc * 16 >= d) break;
                 float v[16];
                 tc::tmem_ld16(row_taddr + cc * 16, v);
                 tc::tmem_wait_ld();
@@ -259,7 +306,7 @@ __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_consta
             if (__syncthreads_or(ok ? 0 : 1)) aborted = true;
             if (t == 0 && i + 1 < M && !aborted) {
                 tc::fence_after_sync();
-                issue_mmas<PREC>(tmem, zt[(i + 1) & 1], bt);
+                issue_mmas<PREC>(tmem, zt[(i + 1) & 1], bt, cols);
                 tc::mma_commit(mbar);
             }
             if (STATS) {
@@ -309,7 +356,7 @@ __global__ void __launch_bounds__(kThreads) basket_tc_kernel(const __grid_consta
 // small per-CTA footprint (64 TMEM columns, ~28 KB of shared memory, <= 64
 // registers) lets 8 CTAs share an SM, which hides each CTA's MMA wait behind
 // the others' normals.  Bounded waits as in basket_tc_kernel.
-template <int PREC, bool STATS, bool EXACT>
+template <int PREC, bool STATS, int READ>
 __global__ void __launch_bounds__(kThreads, 8) basket_tc_acc_kernel(const __grid_constant__ TcArgs a, const TcConst c)
 {
     using Ly = Layout<PREC>;
@@ -353,7 +400,8 @@ __global__ void __launch_bounds__(kThreads, 8) basket_tc_acc_kernel(const __grid
     bool aborted = __syncthreads_or(tc::mbar_wait_bounded(mbar + 8 - 8 * a.stall, 0, a.wait_cap) ? 0 : 1) != 0;
 
     uint32_t phase = 0;
-    const int M = a.run.steps, d = a.d;
+    const int M = a.run.steps, d = READ == kReadAligned ? kN : a.d;
+    const int cols = mma_columns<PREC>(d);  // past d: zero weight, zero increments
     const float inv_m = 1.0f / static_cast<float>(M);
     const int64_t ntiles = (a.run.paths + kRows - 1) / kRows;
     const uint32_t row_taddr = tmem + (static_cast<uint32_t>(warp * 32) << 16);
@@ -367,6 +415,7 @@ __global__ void __launch_bounds__(kThreads, 8) basket_tc_acc_kernel(const __grid
         const float4 *g4 = reinterpret_cast<const float4 *>(s_g[buf]);
 #pragma unroll
         for (int cc = 0; cc < kN / 16; ++cc) {
+            if (cc * 16 >= d) break;
             float v[16];
             tc::tmem_ld16(row_taddr + cc * 16, v);
             tc::tmem_wait_ld();
@@ -394,16 +443,14 @@ __global__ void __launch_bounds__(kThreads, 8) basket_tc_acc_kernel(const __grid
         const int64_t nl = tile * kRows + t;
         const bool valid = nl < a.run.paths;
         const uint64_t n = static_cast<uint64_t>(a.run.path_offset + (valid ? nl : 0));
-        NormalReader rd;
+        RowReader<READ> rd;
         rd.init(n, a.run.rk);
-        PathStream ps;
-        ps.init(n, a.run.rk);
         Stats st{0.0f, -INFINITY, INFINITY};
         bool ok = true;
         for (int i = 0; i < M; ++i) {
             // s_g[(i + 1) & 1] was last read before the previous step's barrier
             if (STATS || i + 1 == M) set_g(i + 1);
-            if (!aborted) draw_row<PREC, EXACT>(zt, t, i, d, ps, a.run.rk, rd, valid);
+            if (!aborted) draw_row<PREC, READ>(zt, t, i, d, a.run.rk, rd, valid);
             tc::fence_proxy_async();
             tc::fence_before_sync();  // this thread's accumulator reads precede the next MMA
             if (__syncthreads_or(ok ? 0 : 1)) aborted = true;
@@ -412,6 +459,7 @@ __global__ void __launch_bounds__(kThreads, 8) basket_tc_acc_kernel(const __grid
                 tc::fence_after_sync();
 #pragma unroll
                 for (int kk = 0; kk < Ly::kMmas; ++kk) {
+                    if (kk * Ly::kKStep >= cols) break;
                     const uint64_t ad = tc::smem_desc(zt + kk * 32, Ly::kGroupBytes, Ly::kSw);
                     const uint64_t bd = tc::smem_desc(bt + kk * 32, Ly::kGroupBytes, Ly::kSw);
                     tc::mma_f16(tmem, ad, bd, tc::idesc_f16(kRows, kN, PREC == MC_BF16), (i > 0 || kk > 0) ? 1u : 0u);
@@ -508,29 +556,36 @@ __global__ void tc_prep_kernel(int d, const double *L, const double *sigma, doub
 
 }  // namespace tcb
 
+namespace tcb {
+
+template <int PREC, int SCHEME, bool STATS, int READ>
+const void *entry()
+{
+    if constexpr (PREC != MC_FP8E4M3 && SCHEME == MC_LOG_EULER) return reinterpret_cast<const void *>(&basket_tc_acc_kernel<PREC, STATS, READ>);
+    else return reinterpret_cast<const void *>(&basket_tc_kernel<PREC, SCHEME, STATS, READ>);
+}
+
+template <int PREC, int SCHEME, bool STATS>
+const void *pick(const TcArgs &a)
+{
+    if (!blocks_fit_32(a.run.steps, a.d)) return entry<PREC, SCHEME, STATS, kReadAny>();
+    return a.d == kN ? entry<PREC, SCHEME, STATS, kReadAligned>() : entry<PREC, SCHEME, STATS, kReadShifted>();
+}
+
+}  // namespace tcb
+
 template <int PREC, int SCHEME>
 const void *basket_tc_select(const TcArgs &a, int *smem)
 {
     const bool stats = a.pay.need_avg || a.pay.need_max || a.pay.need_min;
-    const bool exact = a.d == tcb::kN && blocks_fit_32(a.run.steps, tcb::kN);
-    if constexpr (PREC != MC_FP8E4M3 && SCHEME == MC_LOG_EULER) {
-        // TMEM running sum: Z tile + factor tile + barriers + payoff slots
-        // (~27 KB with the static arrays and the per-block reservation: at
-        // most 8 CTAs, 8 x 64 TMEM columns, share an SM)
-        *smem = 1024 + tcb::Layout<PREC>::kTileBytes + tcb::Layout<PREC>::kBBytes + 32 +
-                (tcb::kThreads / 32) * a.pay.n * 2 * static_cast<int>(sizeof(AccSlot));
-        if (stats)
-            return exact ? reinterpret_cast<const void *>(&tcb::basket_tc_acc_kernel<PREC, true, true>)
-                         : reinterpret_cast<const void *>(&tcb::basket_tc_acc_kernel<PREC, true, false>);
-        return exact ? reinterpret_cast<const void *>(&tcb::basket_tc_acc_kernel<PREC, false, true>)
-                     : reinterpret_cast<const void *>(&tcb::basket_tc_acc_kernel<PREC, false, false>);
-    }
-    *smem = tcb::Layout<PREC>::kSmem;
-    if (stats)
-        return exact ? reinterpret_cast<const void *>(&tcb::basket_tc_kernel<PREC, SCHEME, true, true>)
-                     : reinterpret_cast<const void *>(&tcb::basket_tc_kernel<PREC, SCHEME, true, false>);
-    return exact ? reinterpret_cast<const void *>(&tcb::basket_tc_kernel<PREC, SCHEME, false, true>)
-                 : reinterpret_cast<const void *>(&tcb::basket_tc_kernel<PREC, SCHEME, false, false>);
+    // TMEM running sum: Z tile + factor tile + barriers + payoff slots (~27 KB
+    // with the static arrays and the per-block reservation: at most 8 CTAs,
+    // 8 x 64 TMEM columns, share an SM)
+    *smem = PREC != MC_FP8E4M3 && SCHEME == MC_LOG_EULER
+                ? 1024 + tcb::Layout<PREC>::kTileBytes + tcb::Layout<PREC>::kBBytes + 32 +
+                      (tcb::kThreads / 32) * a.pay.n * 2 * static_cast<int>(sizeof(AccSlot))
+                : tcb::Layout<PREC>::kSmem;
+    return stats ? tcb::pick<PREC, SCHEME, true>(a) : tcb::pick<PREC, SCHEME, false>(a);
 }
 
 template <int PREC>

@@ -277,6 +277,25 @@ struct ShiftedReader {
     }
 };
 
+// The same for paths of more than 2^32 Philox blocks (64-bit block indices).
+struct WideReader {
+    uint64_t n, b;
+    float4 cur, nxt;
+    __device__ __forceinline__ void init(uint64_t path, const RoundKeys &rk)
+    {
+        n = path;
+        b = 1;
+        cur = normals4(0, n, rk);
+        nxt = normals4(1, n, rk);
+    }
+    __device__ __forceinline__ float4 group(int o) const { return shifted4(cur, nxt, o); }
+    __device__ __forceinline__ void advance(const RoundKeys &rk)
+    {
+        cur = nxt;
+        nxt = normals4(++b, n, rk);
+    }
+};
+
 // ---------------------------------------------------------------------------
 // Summed normals.  Under log-Euler with constant coefficients the terminal
 // log-prices of a basket depend on a path's normals only through
