@@ -9,11 +9,13 @@
 // columns):
 //   warp 0   lane 0: TMA producer - streams the pre-swizzled 128 x 64 chunks
 //            of the quantised factor Lq (only chunks on or below the
-//            diagonal) into a ring of shared-memory slots;
+//            diagonal), two neighbouring row blocks at a time, into a ring of
+//            shared-memory slots;
 //   warp 1   lane 0: MMA issuer - for each 64-column panel p of Z and each
-//            128-row block b of Lq on or below the diagonal (p <= 2 b + 1):
-//            4 (2 for E4M3) tcgen05.mma of 128 x 128 x 16 (x32) into TMEM
-//            columns [128 b, 128 b + 128);
+//            pair of 128-row blocks b, b + 1 of Lq on or below the diagonal
+//            (p <= 2 b + 1; the last alone if their number is odd): 4 (2 for
+//            E4M3) tcgen05.mma of 128 x 256 x 16 (x32) into TMEM columns
+//            [128 b, 128 b + 256);
 //   warps 2..17: 512 threads; thread (warp w, lane l) owns path row
 //            32 (w mod 4) + l (its TMEM lane) and column group (w - 2) / 4;
 //            it draws 16 normals of every panel of its row per step
@@ -22,10 +24,12 @@
 //            at the end of a tile it reads its row's 128 columns of D,
 //            forms the terminal prices, the basket, the payoffs and the
 //            pathwise delta / vega / rho contributions.
-// The Z tile is split in two halves of panels with their own full / free
-// mbarriers, so drawing half A of step i+1 overlaps the MMAs of half B of
-// step i; the split balances the MMA work of the halves (the factor is
-// triangular: early panels meet more row blocks).  Every mbarrier wait is bounded; on expiry the CTA records an error
+// The panels of Z go through a ring of their own, so the workers draw up to a
+// ring ahead of the MMAs and the barriers of a step cost no round trip.  Two
+// halves of a whole step's Z with a barrier pair each, and single factor chunks
+// in 80 KB, left the MMA thread the longer chain of every half step: d = 512
+// BF16, 2^17 paths x 252 steps 20.7 ms, so 18.6.  Drawing alone would take 11.7.
+// Every mbarrier wait is bounded; on expiry the CTA records an error
 // word and stops issuing work (results become NaN).
 #pragma once
 
@@ -43,7 +47,6 @@ constexpr int kPanel = 64;        // K columns per panel
 constexpr int kBlk = 128;         // factor rows per chunk = UMMA N
 constexpr int kMaxPanels = 8;
 constexpr int kMaxBlocks = 4;
-constexpr int kRing = 5;          // factor-chunk slots (80 KB in flight for BF16)
 constexpr int kThreads = 576;     // 18 warps
 constexpr int kWorkers = 512;     // warps 2..17
 
@@ -57,11 +60,14 @@ struct L2 {
     static constexpr int kKStep = PREC == MC_FP8E4M3 ? 32 : 16;
     static constexpr int kMmas = kPanel / kKStep;
     static constexpr tc::Swizzle kSw = PREC == MC_FP8E4M3 ? tc::SW_64B : tc::SW_128B;
-    static constexpr int kZBytes = kMaxPanels * kPanelBytes;
+    static constexpr int kZ = PREC == MC_FP8E4M3 ? 8 : 5;     // panels of Z in the ring
+    static constexpr int kRing = PREC == MC_FP8E4M3 ? 6 : 4;  // factor slots, of two chunks (128 KB for BF16)
+    static constexpr int kSlotBytes = 2 * kChunkBytes;
+    static constexpr int kZBytes = kZ * kPanelBytes;
     // [pad 1024] Z | ring | barriers (256 B) | accumulators
-    static constexpr int kBarOff = kZBytes + kRing * kChunkBytes;
+    static constexpr int kBarOff = kZBytes + kRing * kSlotBytes;
     static constexpr int kSmem = 1024 + kBarOff + 256;
-    static_assert(32 + 16 * kRing + 32 <= 256, "mbarrier words exceed their area");
+    static_assert(16 * kZ + 16 * kRing + 32 <= 256, "mbarrier words exceed their area");
     __device__ static __forceinline__ uint32_t off(int row, int chunk)
     {
         const int phys = PREC == MC_FP8E4M3 ? (chunk ^ ((row >> 1) & 3)) : (chunk ^ (row & 7));
@@ -107,29 +113,51 @@ using tc::mbar_arrive;
 using tc::wait_or_fail;
 
 // One worker's 16 normals of a Z panel (columns c0 .. c0 + 15 of its path
-// row at step i), rounded to the operand type and stored swizzled.
-template <int PREC>
-__device__ __forceinline__ void draw_panel(uint32_t pan, int row, int grp, int c0, int i, int d, bool valid,
-                                           const PathStream &ps, int exact4, const RoundKeys &rk, NormalReader &rd)
+// row at step i; 0 past d).  c0 is a multiple of 16, so they are four whole
+// blocks when the step starts with one, else lie in up to five, o lanes into
+// the first.  A branch per normal unrolled 16 copies of Philox behind them:
+// d = 213 BF16, 59,318 paths x 68 steps 3.07 ms, so (and with the rings) 1.96.
+__device__ __forceinline__ void draw16(float (&z)[16], int c0, int i, int d, bool valid, const PathStream &ps, const BigArgs &a,
+                                       NormalReader &rd)
 {
-    using Ly = L2<PREC>;
-    float z[16];
 #pragma unroll
     for (int l = 0; l < 16; ++l) z[l] = 0.0f;
-    if (valid && c0 < d) {
-        if (exact4 && c0 + 16 <= d) {
-            const uint32_t q = static_cast<uint32_t>(i) * (d >> 2) + (c0 >> 2);
+    if (!valid || c0 >= d) return;
+    if (a.exact4 && c0 + 16 <= d) {
+        const uint32_t q = static_cast<uint32_t>(i) * (d >> 2) + (c0 >> 2);
 #pragma unroll
-            for (int bq = 0; bq < 4; ++bq) {
-                const float4 v = ps.normals(q + bq, rk).f4();
-                z[4 * bq] = v.x; z[4 * bq + 1] = v.y; z[4 * bq + 2] = v.z; z[4 * bq + 3] = v.w;
-            }
-        } else {
-#pragma unroll
-            for (int l = 0; l < 16; ++l)  // unrolled: z stays in registers
-                if (c0 + l < d) z[l] = rd.get(static_cast<uint64_t>(i) * d + c0 + l);
+        for (int bq = 0; bq < 4; ++bq) {
+            const float4 v = ps.normals(q + bq, a.run.rk).f4();
+            z[4 * bq] = v.x; z[4 * bq + 1] = v.y; z[4 * bq + 2] = v.z; z[4 * bq + 3] = v.w;
         }
+    } else if (!a.wide) {
+        const uint64_t j0 = static_cast<uint64_t>(i) * d + c0;
+        const uint32_t q = static_cast<uint32_t>(j0 >> 2);
+        const int o = static_cast<int>(j0 & 3), cols = min(16, d - c0), nb = (o + cols + 3) >> 2;
+        float4 cur = ps.normals(q, a.run.rk).f4();
+#pragma unroll
+        for (int bq = 0; bq < 4; ++bq) {
+            float4 nxt = cur;
+            if (bq + 1 < nb) nxt = ps.normals(q + bq + 1, a.run.rk).f4();
+            const float4 v = shifted4(cur, nxt, o);
+            if (4 * bq < cols) z[4 * bq] = v.x;
+            if (4 * bq + 1 < cols) z[4 * bq + 1] = v.y;
+            if (4 * bq + 2 < cols) z[4 * bq + 2] = v.z;
+            if (4 * bq + 3 < cols) z[4 * bq + 3] = v.w;
+            cur = nxt;
+        }
+    } else {
+#pragma unroll
+        for (int l = 0; l < 16; ++l)  // unrolled: z stays in registers
+            if (c0 + l < d) z[l] = rd.get(static_cast<uint64_t>(i) * d + c0 + l);
     }
+}
+
+// z rounded to the operand type, into the swizzled panel at `pan`.
+template <int PREC>
+__device__ __forceinline__ void store16(uint32_t pan, int row, int grp, const float (&z)[16])
+{
+    using Ly = L2<PREC>;
     if (PREC == MC_FP8E4M3) {
         stv4(pan + Ly::off(row, grp), pk4e(z[0], z[1], z[2], z[3]), pk4e(z[4], z[5], z[6], z[7]),
              pk4e(z[8], z[9], z[10], z[11]), pk4e(z[12], z[13], z[14], z[15]));
@@ -155,31 +183,23 @@ __global__ void __launch_bounds__(kThreads, 1) basket_big_kernel(const __grid_co
     const uint32_t raw = tc::smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const uint32_t zt = base, ring = base + Ly::kZBytes, bars = base + Ly::kBarOff;
-    // barrier words: zfull[2], zfree[2] (one pair per half of Z), lfull[R], lfree[R], ddone, dfree, tslot,
+    // barrier words: zfull[kZ], zfree[kZ], lfull[R], lfree[R], ddone, dfree, tslot,
     // xbar (the failure path's drain of the MMA issuer, and the test stall)
-    const uint32_t zfull = bars, zfree = bars + 16, lfull = bars + 32, lfree = lfull + 8 * kRing;
+    constexpr int kZ = Ly::kZ, kRing = Ly::kRing;
+    const uint32_t zfull = bars, zfree = zfull + 8 * kZ, lfull = zfree + 8 * kZ, lfree = lfull + 8 * kRing;
     const uint32_t ddone = lfree + 8 * kRing, dfree = ddone + 8, tslot = dfree + 8, xbar = dfree + 16;
     uint32_t *tslot_ptr = reinterpret_cast<uint32_t *>(smem_raw + (tslot - raw));
 
     const int d = a.d, NP = (d + kPanel - 1) / kPanel, NB = (NP + 1) / 2;
-    // Split of the Z panels into the two halves: the first half ends at the
-    // panel where the MMA chunks (NB - p / 2 for panel p) reach half the step's
-    // total, so each half's MMAs run while the workers draw the other half.
-    int half = 1;
-    {
-        int total = 0, cum = NB;
-        for (int p = 0; p < NP; ++p) total += NB - p / 2;
-        while (half < NP - 1 && 2 * cum < total) cum += NB - half++ / 2;
-    }
     const int M = a.run.steps;
     const int nv = a.pay.n;
     for (int i = t; i < nv * 2; i += kThreads) s_pay[i >> 1][i & 1] = 0.0f;
     for (int i = t; i < (2 * d + 1) * 2; i += kThreads) s_g[i >> 1][i & 1] = 0.0f;
     if (t == 0) {
         s_fail = 0;
-        for (int hh = 0; hh < 2; ++hh) {
-            tc::mbar_init(zfull + 8 * hh, kWorkers);
-            tc::mbar_init(zfree + 8 * hh, 1);
+        for (int r = 0; r < kZ; ++r) {
+            tc::mbar_init(zfull + 8 * r, kWorkers / 32);
+            tc::mbar_init(zfree + 8 * r, 1);
         }
         for (int r = 0; r < kRing; ++r) {
             tc::mbar_init(lfull + 8 * r, 1);
@@ -198,7 +218,6 @@ __global__ void __launch_bounds__(kThreads, 1) basket_big_kernel(const __grid_co
     tc::fence_after_sync();
     const uint32_t tmem = *tslot_ptr;
     const int64_t ntiles = (a.run.paths + kRows - 1) / kRows;
-    // chunks per step: sum over panels p of (NP - p)
     const uint32_t cap = tc::cap_polls(a.wait_cap);
     uint32_t issued = 0, lastpar = 0;  // producer: per ring slot, a copy was issued; its lfull parity
     if (tc::stall_requested(a.wait_cap)) {
@@ -214,14 +233,16 @@ __global__ void __launch_bounds__(kThreads, 1) basket_big_kernel(const __grid_co
             for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
                 for (int i = 0; i < M; ++i)
                     for (int p = 0; p < NP; ++p)
-                        for (int b = p / 2; b < NB; ++b) {
+                        for (int b = p / 2; b < NB; b += 2) {
                             const bool ok = primed < kRing ? (++primed, true)
                                                            : wait_or_fail(&s_fail, lfree + 8 * slot, phase ^ 1u, cap);
                             if (ok && !s_fail) {
-                                tc::mbar_arrive_expect_tx(lfull + 8 * slot, Ly::kChunkBytes);
-                                tc::bulk_g2s(ring + slot * Ly::kChunkBytes,
-                                             a.bimg + static_cast<size_t>(b * kMaxPanels + p) * Ly::kChunkBytes,
-                                             Ly::kChunkBytes, lfull + 8 * slot);
+                                const int two = b + 1 < NB ? 2 : 1;
+                                tc::mbar_arrive_expect_tx(lfull + 8 * slot, two * Ly::kChunkBytes);
+                                for (int e = 0; e < two; ++e)
+                                    tc::bulk_g2s(ring + slot * Ly::kSlotBytes + e * Ly::kChunkBytes,
+                                                 a.bimg + static_cast<size_t>((b + e) * kMaxPanels + p) * Ly::kChunkBytes,
+                                                 Ly::kChunkBytes, lfull + 8 * slot);
                                 issued |= 1u << slot;
                                 lastpar = (lastpar & ~(1u << slot)) | (phase << slot);
                             }
@@ -234,40 +255,46 @@ __global__ void __launch_bounds__(kThreads, 1) basket_big_kernel(const __grid_co
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
-            const uint32_t idesc = PREC == MC_FP8E4M3 ? tc::idesc_e4m3(kRows, kBlk)
-                                                      : tc::idesc_f16(kRows, kBlk, PREC == MC_BF16);
+            // one row block of the factor, two
+            const uint32_t idesc1 = PREC == MC_FP8E4M3 ? tc::idesc_e4m3(kRows, kBlk)
+                                                       : tc::idesc_f16(kRows, kBlk, PREC == MC_BF16);
+            const uint32_t idesc2 = PREC == MC_FP8E4M3 ? tc::idesc_e4m3(kRows, 2 * kBlk)
+                                                       : tc::idesc_f16(kRows, 2 * kBlk, PREC == MC_BF16);
             // descriptors change only in their 14-bit start-address field (address / 16)
             const uint64_t adesc0 = tc::smem_desc(zt, Ly::kGroup, Ly::kSw);
             const uint64_t bdesc0 = tc::smem_desc(ring, Ly::kGroup, Ly::kSw);
-            uint32_t slot = 0, phase = 0;
-            uint64_t g = 0, tl = 0;
+            uint32_t slot = 0, phase = 0, zslot = 0, zphase = 0;
+            uint64_t tl = 0;
             for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++tl) {
                 if (tl > 0) wait_or_fail(&s_fail, dfree, static_cast<uint32_t>((tl - 1) & 1), cap);
-                for (int i = 0; i < M; ++i, ++g) {
-                    for (int hh = 0; hh < 2; ++hh) {
-                        const bool zok = wait_or_fail(&s_fail, zfull + 8 * hh, static_cast<uint32_t>(g & 1), cap);
+                for (int i = 0; i < M; ++i) {
+                    for (int p = 0; p < NP; ++p) {
+                        const bool zok = wait_or_fail(&s_fail, zfull + 8 * zslot, zphase, cap);
                         tc::fence_after_sync();
-                        for (int p = hh ? half : 0; p < (hh ? NP : half); ++p) {
-                            const uint64_t ap = adesc0 + static_cast<uint32_t>(p * (Ly::kPanelBytes >> 4));
-                            for (int b = p / 2; b < NB; ++b) {
-                                if (zok && wait_or_fail(&s_fail, lfull + 8 * slot, phase, cap)) {
-                                    tc::fence_after_sync();
-                                    const uint64_t bp = bdesc0 + slot * static_cast<uint32_t>(Ly::kChunkBytes >> 4);
+                        const uint64_t ap = adesc0 + zslot * static_cast<uint32_t>(Ly::kPanelBytes >> 4);
+                        for (int b = p / 2; b < NB; b += 2) {
+                            if (zok && wait_or_fail(&s_fail, lfull + 8 * slot, phase, cap)) {
+                                tc::fence_after_sync();
+                                const uint64_t bp = bdesc0 + slot * static_cast<uint32_t>(Ly::kSlotBytes >> 4);
+                                const uint32_t id = b + 1 < NB ? idesc2 : idesc1;
 #pragma unroll
-                                    for (int kk = 0; kk < Ly::kMmas; ++kk) {
-                                        const uint32_t acc = (i == 0 && p == 0 && kk == 0) ? 0u : 1u;
-                                        if (PREC == MC_FP8E4M3) tc::mma_f8(tmem + b * kBlk, ap + 2 * kk, bp + 2 * kk, idesc, acc);
-                                        else tc::mma_f16(tmem + b * kBlk, ap + 2 * kk, bp + 2 * kk, idesc, acc);
-                                    }
-                                    tc::mma_commit(lfree + 8 * slot);
+                                for (int kk = 0; kk < Ly::kMmas; ++kk) {
+                                    const uint32_t acc = (i == 0 && p == 0 && kk == 0) ? 0u : 1u;
+                                    if (PREC == MC_FP8E4M3) tc::mma_f8(tmem + b * kBlk, ap + 2 * kk, bp + 2 * kk, id, acc);
+                                    else tc::mma_f16(tmem + b * kBlk, ap + 2 * kk, bp + 2 * kk, id, acc);
                                 }
-                                if (++slot == kRing) {
-                                    slot = 0;
-                                    phase ^= 1u;
-                                }
+                                tc::mma_commit(lfree + 8 * slot);
+                            }
+                            if (++slot == kRing) {
+                                slot = 0;
+                                phase ^= 1u;
                             }
                         }
-                        tc::mma_commit(zfree + 8 * hh);
+                        tc::mma_commit(zfree + 8 * zslot);
+                        if (++zslot == kZ) {
+                            zslot = 0;
+                            zphase ^= 1u;
+                        }
                     }
                 }
                 tc::mma_commit(ddone);
@@ -277,7 +304,8 @@ __global__ void __launch_bounds__(kThreads, 1) basket_big_kernel(const __grid_co
         // ---------------- RNG + epilogue workers ----------------
         const int row = 32 * (warp & 3) + lane;
         const int grp = (warp - 2) >> 2;  // column group 0..3
-        uint64_t g = 0, tl = 0;
+        uint32_t zslot = 0, zphase = 0, primed = 0;  // ring position; panels filled once
+        uint64_t tl = 0;
         for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++tl) {
             const int64_t nl = tile * kRows + row;
             const bool valid = nl < a.run.paths;
@@ -286,16 +314,20 @@ __global__ void __launch_bounds__(kThreads, 1) basket_big_kernel(const __grid_co
             rd.init(n, a.run.rk);
             PathStream ps;
             ps.init(n, a.run.rk);
-            for (int i = 0; i < M; ++i, ++g) {
-                for (int hh = 0; hh < 2; ++hh) {
-                    const bool ok = g == 0 || wait_or_fail(&s_fail, zfree + 8 * hh, static_cast<uint32_t>((g - 1) & 1), cap);
-                    if (ok && !s_fail) {
-                        for (int p = hh ? half : 0; p < (hh ? NP : half); ++p)
-                            draw_panel<PREC>(zt + p * Ly::kPanelBytes, row, grp, p * kPanel + grp * 16, i, d, valid, ps,
-                                             a.exact4, a.run.rk, rd);
-                        tc::fence_proxy_async();
+            for (int i = 0; i < M; ++i) {
+                for (int p = 0; p < NP; ++p) {
+                    float z[16];
+                    draw16(z, p * kPanel + grp * 16, i, d, valid && !s_fail, ps, a, rd);
+                    const bool ok = primed < kZ ? (++primed, true)
+                                                : wait_or_fail(&s_fail, zfree + 8 * zslot, zphase ^ 1u, cap);
+                    if (ok) store16<PREC>(zt + zslot * Ly::kPanelBytes, row, grp, z);
+                    tc::fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(zfull + 8 * zslot);  // always: the MMA issuer counts 16 warps
+                    if (++zslot == kZ) {
+                        zslot = 0;
+                        zphase ^= 1u;
                     }
-                    mbar_arrive(zfull + 8 * hh);  // always: the MMA issuer counts 512 arrivals
                 }
             }
             // ---- epilogue: terminal prices, basket, payoffs, pathwise Greeks ----
