@@ -13,7 +13,11 @@
 //
 // Warp roles (one CTA of 18 warps per SM; TMEM: 2 x 256 FP32 columns):
 //   warp 0   lane 0: TMA producer - streams the pre-swizzled weight chunks
-//            (W rows x 32 K columns, 64-byte swizzle) into a ring;
+//            (W rows x 32 K columns, 64-byte swizzle), two at a time, into a
+//            ring.  A slot's round trip (wait, MMAs, commit) costs some 300
+//            cycles beside its MMAs, whatever the copies do: slots of one
+//            chunk (256 cycles of MMAs) took 2.41 ms for 2^22 rows of the width-256
+//            network, these 2.15;
 //   warp 1   lane 0: MMA issuer - per layer and tile, K / 16 tcgen05.mma of
 //            128 x W x 16 into that tile's accumulator;
 //   warps 2..9 / 10..17: epilogue of tile lane X / Y (two tiles in flight,
@@ -36,7 +40,7 @@ constexpr int kKc = 32;                  // K columns per operand panel / weight
 constexpr int kMaxW = 256;
 constexpr int kMaxIn = 10;               // 3 n_in <= 32: layer 0 fits one K = 32 panel
 constexpr int kMaxLayers = 16;
-constexpr int kRing = 5;
+constexpr int kRing = 3;                 // slots of two chunks: 96 KB at W = 256
 static_assert(32 + 16 * kRing + 16 <= 128, "mbarrier words exceed their area");
 constexpr int kThreads = 576;
 constexpr int kLaneThreads = 256;        // epilogue threads of one tile lane
@@ -106,10 +110,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bf16_kernel(const Args a)
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int W = a.W, KC = W / kKc, NL = a.NL;
     const uint32_t raw = tc::smem_u32(smem_raw);
-    const uint32_t base = (raw + 1023u) & ~1023u;
+    const uint32_t base = (raw + 511u) & ~511u;  // the swizzle's period
     const uint32_t abytes = static_cast<uint32_t>(KC) * kPanelBytes;  // one tile's activations
     const uint32_t cbytes = static_cast<uint32_t>(W) * 64;            // one weight chunk
-    const uint32_t ring = base + 2 * abytes, bars = ring + kRing * cbytes;
+    const uint32_t sbytes = 2 * cbytes;                               // one ring slot
+    const uint32_t ring = base + 2 * abytes, bars = ring + kRing * sbytes;
     // barrier words: afull[2], dfull[2], lfull[R], lfree[R], tslot, xbar (the
     // failure path's drain of the MMA issuer, and the test stall)
     const uint32_t afull = bars, dfull = bars + 16, lfull = bars + 32, lfree = lfull + 8 * kRing;
@@ -154,13 +159,14 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bf16_kernel(const Args a)
                 const int lanes = tx + G < ntiles ? 2 : 1;
                 for (int l = 0; l < NL; ++l)
                     for (int T = 0; T < lanes; ++T)
-                        for (int kc = 0; kc < chunk_count(l, KC); ++kc) {
+                        for (int kc = 0; kc < chunk_count(l, KC); kc += 2) {
+                            const uint32_t bytes = kc + 1 < chunk_count(l, KC) ? sbytes : cbytes;
                             const bool ok = primed < kRing ? (++primed, true)
                                                            : tc::wait_or_fail(&s_fail, lfree + 8 * slot, phase ^ 1u, cap);
                             if (ok && !s_fail) {
-                                tc::mbar_arrive_expect_tx(lfull + 8 * slot, cbytes);
-                                tc::bulk_g2s(ring + slot * cbytes,
-                                             a.img + static_cast<size_t>(chunk_id(l, kc, KC)) * cbytes, cbytes,
+                                tc::mbar_arrive_expect_tx(lfull + 8 * slot, bytes);
+                                tc::bulk_g2s(ring + slot * sbytes,
+                                             a.img + static_cast<size_t>(chunk_id(l, kc, KC)) * cbytes, bytes,
                                              lfull + 8 * slot);
                                 issued |= 1u << slot;
                                 lastpar = (lastpar & ~(1u << slot)) | (phase << slot);
@@ -187,13 +193,19 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bf16_kernel(const Args a)
                         const bool aok = tc::wait_or_fail(&s_fail, afull + 8 * T, ph[T], cap);
                         ph[T] ^= 1u;
                         tc::fence_after_sync();
-                        for (int kc = 0; kc < chunk_count(l, KC); ++kc) {
+                        for (int kc = 0; kc < chunk_count(l, KC); kc += 2) {
                             if (aok && tc::wait_or_fail(&s_fail, lfull + 8 * slot, phase, cap)) {
                                 tc::fence_after_sync();
-                                const uint64_t ad = adesc0 + ((T * abytes + kc * kPanelBytes) >> 4);
-                                const uint64_t bd = bdesc0 + ((slot * cbytes) >> 4);
+                                uint64_t ad = adesc0 + ((T * abytes + kc * kPanelBytes) >> 4);
+                                uint64_t bd = bdesc0 + ((slot * sbytes) >> 4);
                                 tc::mma_f16(tmem + 256 * T, ad, bd, idesc, kc == 0 ? 0u : 1u);
                                 tc::mma_f16(tmem + 256 * T, ad + 2, bd + 2, idesc, 1u);  // K + 16: 32 bytes on
+                                if (kc + 1 < chunk_count(l, KC)) {
+                                    ad += kPanelBytes >> 4;
+                                    bd += cbytes >> 4;
+                                    tc::mma_f16(tmem + 256 * T, ad, bd, idesc, 1u);
+                                    tc::mma_f16(tmem + 256 * T, ad + 2, bd + 2, idesc, 1u);
+                                }
                                 tc::mma_commit(lfree + 8 * slot);
                             }
                             if (++slot == kRing) {
@@ -415,7 +427,7 @@ cudaError_t mlp_forward_bf16(const MlpLayout &L, const float *params, const uint
     a.err = err;
     const int KC = a.W / kKc;
     // at least half the SM's shared memory: one CTA per SM, which owns all 512 TMEM columns
-    int smem = 1024 + 2 * KC * kPanelBytes + kRing * a.W * 64 + 128;  // barriers: 16 + 16 + 16 R + 8 + 8 <= 128
+    int smem = 512 + 2 * KC * kPanelBytes + kRing * 2 * a.W * 64 + 128;  // barriers: 16 + 16 + 16 R + 8 + 8 <= 128
     if (smem < 120 * 1024) smem = 120 * 1024;
     cudaError_t e = cudaFuncSetAttribute(mlp_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
