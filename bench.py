@@ -450,7 +450,9 @@ def config_c5(torch, gb, orc, hw, flush, reps):
                "error_vs_oracle": {"paths": n_or, "per_price": _errors(orc, small, ref)},
                "roofline_sfu": hw.sfu(ps / t, normals=d, what=f"{d} normals")}
         if prec == "fp32":
-            rec["roofline"] = hw.fma(ps / t * d * (d + 1) / 2, f"{d * (d + 1) // 2} FMA per path-step (triangular)")
+            # a European price contracts the path's summed normals once
+            rec["roofline"] = rec["roofline_sfu"]
+            rec["roofline_fma"] = hw.fma(w["paths"] / t * d * (d + 1) / 2, f"{d * (d + 1) // 2} FMA per path (triangular)")
         else:
             rec["roofline"] = hw.tensor(ps / t * d * (d + 1), prec, f"{d * (d + 1)} flop per path-step (triangular)")
             tg, _, (_, g) = time_call(torch, lambda: gb.greeks(model, c, pays), 1)
