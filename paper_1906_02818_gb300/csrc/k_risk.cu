@@ -166,10 +166,23 @@ __global__ void outer_kernel(int64_t nscen, int64_t off, int d, const float *__r
 // remaining maturity; out[s*d + u] = sum_{o of u} pos_o (V_o(s) - base_o) in
 // FP64.  Options are sorted by maturity, so a path runs from one maturity to
 // the next without a test per date; the blocks that a maturity splits are
-// finished on the other side of it.  Few scenarios (the base date is one) are
-// cut into slices of paths, whose option sums nested_finish_kernel adds: the
-// base values of 32 underlyings on 32 CTAs took as long as the 16384 CTAs of
-// 512 scenarios (28.2 ms together for 1024 inner and 65536 base paths).
+// finished on the other side of it.
+// The paths fall into groups that depend on their number alone (nested_group):
+// thread t adds the group's paths t, t + 256, ... in FP32, the CTA adds its
+// threads in FP64, and the groups are added in FP64 in their order.  A slice is
+// a run of whole groups, so a scenario's value has the same bits however many
+// scenarios the call has and however many SMs share them (shards of a run).
+// Few scenarios (the base date is one) are cut into slices, whose group sums
+// nested_finish_kernel adds: the base values of 32 underlyings on 32 CTAs took
+// as long as the 16384 CTAs of 512 scenarios (28.2 ms together for 1024 inner
+// and 65536 base paths).
+
+// Paths of a group: 1024, four per thread, or the multiple of that which keeps
+// the groups at 256 (from 2^18 paths on).
+__host__ __device__ constexpr int nested_group(int paths)
+{
+    return paths <= (1 << 18) ? 1024 : (paths + (1 << 18) - 1) / (1 << 18) * 1024;
+}
 
 // Value of option j of underlying u at scenario price S1 from its payoff sum.
 __device__ __forceinline__ double nested_value(const RiskArgs &a, int o, int hs, float S1, double sum)
@@ -178,7 +191,7 @@ __device__ __forceinline__ double nested_value(const RiskArgs &a, int o, int hs,
     return exp(-static_cast<double>(a.r) * (a.rem[o] + hs) * a.dt) * sum / a.inner;
 }
 
-__global__ void __launch_bounds__(256) nested_kernel(const __grid_constant__ RiskArgs a, const float *__restrict__ Sp,
+__global__ void __launch_bounds__(256, 8) nested_kernel(const __grid_constant__ RiskArgs a, const float *__restrict__ Sp,
                                                      double *__restrict__ out, double *__restrict__ part, int slices)
 {
     __shared__ double s_v[kRiskMaxOptPerUnder];
@@ -205,73 +218,94 @@ __global__ void __launch_bounds__(256) nested_kernel(const __grid_constant__ Ris
     }
     __syncthreads();
     float acc[kRiskMaxOptPerUnder];
-#pragma unroll
-    for (int j = 0; j < kRiskMaxOptPerUnder; ++j) acc[j] = 0.0f;
     const uint64_t gpair = static_cast<uint64_t>(a.scen_off + s) * d + u;  // global (scenario, underlying)
     const uint64_t base_idx = Sp ? (gpair << 16) : (static_cast<uint64_t>(u) << 24);
     const uint64_t domain = Sp ? 3 : 5;
-    const int per = (a.inner + slices - 1) / slices, last = min(a.inner, (slice + 1) * per);
-    for (int path = slice * per + threadIdx.x; path < last; path += blockDim.x) {
-        PathStream ps;
-        ps.init(tag(domain, base_idx | static_cast<uint64_t>(path)), a.rk);
-        float y = 0.0f, mx = -INFINITY;  // log2(S/S1) and its running maximum over the dates
-        float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        auto step = [&](float zl) {
-            y += fmaf(bb, zl, aa);
-            mx = fmaxf(mx, y);
-        };
-        int q = 0, l = 0;  // next date 4 q + l + 1; z holds block q when l > 0
-        for (int j = 0; j < no;) {
-            const int t = s_t[j];
-            if (l > 0) {  // the rest of the block that the last maturity split
-                const int e = min(4, t - 4 * q);
-                if (l <= 1 && e > 1) step(z.y);
-                if (l <= 2 && e > 2) step(z.z);
-                if (e > 3) step(z.w);
-                l = e;
-                if (l == 4) {
-                    l = 0;
-                    ++q;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int group = nested_group(a.inner), groups = (a.inner + group - 1) / group, per = (groups + slices - 1) / slices;
+    double total = 0.0;  // threads below `no`: the option's sum over this slice's groups
+    for (int g = slice * per; g < min(groups, (slice + 1) * per); ++g) {
+        const int last = min(a.inner, (g + 1) * group);
+#pragma unroll
+        for (int j = 0; j < kRiskMaxOptPerUnder; ++j) acc[j] = 0.0f;
+        for (int path = g * group + threadIdx.x; path < last; path += blockDim.x) {
+            PathStream ps;
+            ps.init(tag(domain, base_idx | static_cast<uint64_t>(path)), a.rk);
+            float y = 0.0f, mx = -INFINITY;  // log2(S/S1) and its running maximum over the dates
+            float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            auto step = [&](float zl) {
+                y += fmaf(bb, zl, aa);
+                mx = fmaxf(mx, y);
+            };
+            int q = 0, l = 0;  // next date 4 q + l + 1; z holds block q when l > 0
+            for (int j = 0; j < no;) {
+                const int t = s_t[j];
+                if (l > 0) {  // the rest of the block that the last maturity split
+                    const int e = min(4, t - 4 * q);
+                    if (l <= 1 && e > 1) step(z.y);
+                    if (l <= 2 && e > 2) step(z.z);
+                    if (e > 3) step(z.w);
+                    l = e;
+                    if (l == 4) {
+                        l = 0;
+                        ++q;
+                    }
+                }
+                for (; 4 * q + 4 <= t; ++q) {
+                    z = ps.normals(static_cast<uint32_t>(q), a.rk).f4();
+                    step(z.x);
+                    step(z.y);
+                    step(z.z);
+                    step(z.w);
+                }
+                if (l == 0 && 4 * q < t) {
+                    z = ps.normals(static_cast<uint32_t>(q), a.rk).f4();
+                    l = t - 4 * q;
+                    step(z.x);
+                    if (l > 1) step(z.y);
+                    if (l > 2) step(z.z);
+                }
+                const float ST = S1 * ex2_approx(y), Smx = S1 * ex2_approx(mx);
+                for (; j < no && s_t[j] == t; ++j) {
+                    float f = s_kind[j] == MC_PUT ? fmaxf(s_K[j] - ST, 0.0f) : fmaxf(ST - s_K[j], 0.0f);
+                    if (s_kind[j] == MC_UO_CALL && Smx >= s_H[j]) f = 0.0f;
+                    acc[j] += f;
                 }
             }
-            for (; 4 * q + 4 <= t; ++q) {
-                z = ps.normals(static_cast<uint32_t>(q), a.rk).f4();
-                step(z.x);
-                step(z.y);
-                step(z.z);
-                step(z.w);
-            }
-            if (l == 0 && 4 * q < t) {
-                z = ps.normals(static_cast<uint32_t>(q), a.rk).f4();
-                l = t - 4 * q;
-                step(z.x);
-                if (l > 1) step(z.y);
-                if (l > 2) step(z.z);
-            }
-            const float ST = S1 * ex2_approx(y), Smx = S1 * ex2_approx(mx);
-            for (; j < no && s_t[j] == t; ++j) {
-                float f = s_kind[j] == MC_PUT ? fmaxf(s_K[j] - ST, 0.0f) : fmaxf(ST - s_K[j], 0.0f);
-                if (s_kind[j] == MC_UO_CALL && Smx >= s_H[j]) f = 0.0f;
-                acc[j] += f;
-            }
         }
+        // Block reduction per option (FP64).  Eight options share one exchange
+        // tree, in which a lane hands over the half of its values that it does
+        // not go on with: 9 FP64 additions for 40, each sum in warp_sum_d's order.
+        for (int j0 = 0; j0 < no; j0 += 8) {
+            double v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = acc[j0 + j];
+#pragma unroll
+            for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int j = 0; j < h; ++j) {
+                    const double keep = up ? v[j + h] : v[j], give = up ? v[j] : v[j + h];
+                    v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+            }
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+            if ((lane & 3) == 0) s_red[warp][j0 + (lane >> 2)] = v[0];
+        }
+        __syncthreads();
+        if (threadIdx.x < no) {
+            double t = 0.0;
+            for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) t += s_red[w][threadIdx.x];
+            if (slices > 1) part[(pair * groups + g) * kRiskMaxOptPerUnder + threadIdx.x] = t;
+            else total += t;
+        }
+        __syncthreads();  // s_red is free for the next group
     }
-    // block reduction per option (FP64)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = 0; j < no; ++j) {
-        const double v = warp_sum_d(static_cast<double>(acc[j]));
-        if (lane == 0) s_red[warp][j] = v;
-    }
+    if (slices > 1) return;
+    if (threadIdx.x < no) s_v[threadIdx.x] = nested_value(a, o0 + threadIdx.x, hs, S1, total);
     __syncthreads();
-    if (threadIdx.x < no) {
-        const int j = threadIdx.x;
-        double t = 0.0;
-        for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) t += s_red[w][j];
-        if (slices > 1) part[static_cast<int64_t>(blockIdx.x) * kRiskMaxOptPerUnder + j] = t;
-        else s_v[j] = nested_value(a, o0 + j, hs, S1, t);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && slices == 1) {
+    if (threadIdx.x == 0) {
         double t = 0.0;
         for (int j = 0; j < no; ++j) {
             if (Sp) t += a.pos[o0 + j] * (s_v[j] - a.base[o0 + j]);
@@ -281,9 +315,9 @@ __global__ void __launch_bounds__(256) nested_kernel(const __grid_constant__ Ris
     }
 }
 
-// One warp per (scenario, underlying): the option sums of its slices, then as above.
+// One warp per (scenario, underlying): its groups' option sums, then as above.
 __global__ void __launch_bounds__(32) nested_finish_kernel(const RiskArgs a, const float *__restrict__ Sp,
-                                                           double *__restrict__ out, const double *__restrict__ part, int slices)
+                                                           double *__restrict__ out, const double *__restrict__ part, int groups)
 {
     __shared__ double s_v[kRiskMaxOptPerUnder];
     const int64_t pair = blockIdx.x;
@@ -292,7 +326,7 @@ __global__ void __launch_bounds__(32) nested_finish_kernel(const RiskArgs a, con
     const float S1 = Sp ? Sp[pair] : a.s0[u];
     if (threadIdx.x < no) {
         double t = 0.0;
-        for (int k = 0; k < slices; ++k) t += part[(pair * slices + k) * kRiskMaxOptPerUnder + threadIdx.x];
+        for (int k = 0; k < groups; ++k) t += part[(pair * groups + k) * kRiskMaxOptPerUnder + threadIdx.x];
         s_v[threadIdx.x] = nested_value(a, o0 + threadIdx.x, hs, S1, t);
     }
     __syncthreads();
@@ -523,16 +557,19 @@ cudaError_t launch_outer(int64_t nscen, int64_t off, int d, const float *Lc, con
 }
 
 // Slices of the inner paths: none once the pairs alone are eight CTAs per SM,
-// else as many as reach that, each of at least one path per thread.
+// else as many as reach that, each of at least one group.
 int nested_slices(int64_t pairs, int inner, int sms)
 {
-    const int64_t want = (8 * static_cast<int64_t>(sms) + pairs - 1) / pairs, most = (inner + 255) / 256;
-    return static_cast<int>(std::max<int64_t>(1, std::min(want, most)));
+    const int group = nested_group(inner), groups = (inner + group - 1) / group;
+    const int64_t want = (8 * static_cast<int64_t>(sms) + pairs - 1) / pairs;
+    const int n = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, groups))), per = (groups + n - 1) / n;
+    return (groups + per - 1) / per;
 }
 
-size_t nested_part_doubles(int64_t pairs, int slices)
+size_t nested_part_doubles(int64_t pairs, int inner, int slices)
 {
-    return slices > 1 ? static_cast<size_t>(pairs) * slices * kRiskMaxOptPerUnder : 0;
+    const int group = nested_group(inner);
+    return slices > 1 ? static_cast<size_t>(pairs) * ((inner + group - 1) / group) * kRiskMaxOptPerUnder : 0;
 }
 
 cudaError_t launch_nested(const RiskArgs &a, int64_t nscen, const float *Sp, double *contrib, double *part, int slices,
@@ -542,7 +579,8 @@ cudaError_t launch_nested(const RiskArgs &a, int64_t nscen, const float *Sp, dou
     nested_kernel<<<static_cast<unsigned>(pairs * slices), 256, 0, s>>>(a, Sp, contrib, part, slices);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || slices == 1) return e;
-    nested_finish_kernel<<<static_cast<unsigned>(pairs), 32, 0, s>>>(a, Sp, contrib, part, slices);
+    const int group = nested_group(a.inner);
+    nested_finish_kernel<<<static_cast<unsigned>(pairs), 32, 0, s>>>(a, Sp, contrib, part, (a.inner + group - 1) / group);
     return cudaGetLastError();
 }
 

@@ -36,7 +36,7 @@ cudaError_t launch_outer(int64_t nscen, int64_t off, int d, const float *Lc, con
 // Inner paths of nscen scenarios (Sp == nullptr: the base date) in `slices`
 // CTAs per (scenario, underlying); part: nested_part_doubles scratch.
 int nested_slices(int64_t pairs, int inner, int sms);
-size_t nested_part_doubles(int64_t pairs, int slices);
+size_t nested_part_doubles(int64_t pairs, int inner, int slices);
 cudaError_t launch_nested(const RiskArgs &a, int64_t nscen, const float *Sp, double *contrib, double *part, int slices,
                           cudaStream_t s);
 cudaError_t launch_sum_under(int64_t nscen, int d, const double *contrib, double *pnl, cudaStream_t s);
