@@ -34,7 +34,7 @@ const void *basket_select_scheme(const BasketArgs &a);
 #ifdef GBMC_BASKET_IMPL
 namespace basket_detail {
 
-constexpr int kMaxWarps = 20;  // warps of the largest block (one path per thread, 640 threads)
+constexpr int kMaxWarps = kBasketMaxThreads / 32;
 
 __device__ __forceinline__ float elem(const f32x2 *v, int j) { return (j & 1) ? hi_of(v[j >> 1]) : lo_of(v[j >> 1]); }
 

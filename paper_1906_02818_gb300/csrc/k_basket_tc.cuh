@@ -585,6 +585,9 @@ const void *basket_tc_select(const TcArgs &a, int *smem)
     // TMEM running sum: Z tile + factor tile + barriers + payoff slots (~27 KB
     // with the static arrays and the per-block reservation: at most 8 CTAs,
     // 8 x 64 TMEM columns, share an SM)
+    static_assert(1024 + tcb::Layout<PREC>::kTileBytes + tcb::Layout<PREC>::kBBytes + 32 +
+                          (tcb::kThreads / 32) * MC_MAX_PAYOFFS * 2 * sizeof(AccSlot) + 4096 <= kSmemNoOptIn,
+                  "the running-sum kernel needs no shared-memory attribute for any number of payoffs");
     *smem = PREC != MC_FP8E4M3 && SCHEME == MC_LOG_EULER
                 ? 1024 + tcb::Layout<PREC>::kTileBytes + tcb::Layout<PREC>::kBBytes + 32 +
                       (tcb::kThreads / 32) * a.pay.n * 2 * static_cast<int>(sizeof(AccSlot))

@@ -637,7 +637,7 @@ int corr_occupancy(const CorrArgs &a)
 
 int corr_block() { return kThreads; }
 
-size_t corr_adjoint_smem(int d) { return (3 * static_cast<size_t>(d) * (d + 1) + d) * sizeof(double); }
+constexpr size_t corr_adjoint_smem(int d) { return (3 * static_cast<size_t>(d) * (d + 1) + d) * sizeof(double); }
 
 cudaError_t launch_corr(const CorrArgs &a, const CorrConst &c, int grid, int batches, const double *L,
                         const double *cfac, double *Hb, double *nb, double *out_dl, double *out_drho,
@@ -655,11 +655,9 @@ cudaError_t launch_corr(const CorrArgs &a, const CorrConst &c, int grid, int bat
     corr_batch_kernel<<<dim3(batches, kD * kD / 256), 256, 0, s>>>(a.partials, a.counts, grid, batches, Hb, nb);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const size_t smem = corr_adjoint_smem(a.d);
-    if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(corr_adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-    }
+    e = cudaFuncSetAttribute(corr_adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(corr_adjoint_smem(kD)));
+    if (e != cudaSuccess) return e;
     corr_adjoint_kernel<<<batches + 1, 256, smem, s>>>(a.d, batches, Hb, nb, L, cfac, out_dl, out_drho);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int dd2 = 2 * a.d * a.d;

@@ -282,11 +282,13 @@ const void *select(const FactorArgs &a)
 
 }  // namespace
 
-size_t factor_smem_bytes(const FactorArgs &a)
+static constexpr size_t factor_smem(int k, int G, int d, bool greeks)
 {
-    const int dp = 256 * a.G;
-    return static_cast<size_t>(a.k * dp + 3 * dp + kWarps * kP + (a.greeks ? (2 * a.d + 1) * 2 : 0)) * sizeof(float);
+    return static_cast<size_t>(k * 256 * G + 3 * 256 * G + kWarps * kP + (greeks ? (2 * d + 1) * 2 : 0)) * sizeof(float);
 }
+constexpr size_t kFactorSmem = factor_smem(kFactorMax, (kFactorMaxD + 255) / 256, kFactorMaxD, true);  // the largest
+
+size_t factor_smem_bytes(const FactorArgs &a) { return factor_smem(a.k, a.G, a.d, a.greeks != 0); }
 
 cudaError_t launch_factor_greeks_finish(const FactorArgs &a, int grid, double disc, mc_result *out, cudaStream_t s)
 {
@@ -299,7 +301,7 @@ cudaError_t launch_factor(const FactorArgs &a, int grid, cudaStream_t s)
 {
     const void *f = select(a);
     const size_t smem = factor_smem_bytes(a);
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kFactorSmem));
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<FactorArgs *>(&a)};
     return cudaLaunchKernel(f, dim3(grid), dim3(kBlock), args, smem, s);
@@ -309,7 +311,7 @@ int factor_occupancy(const FactorArgs &a)
 {
     const void *f = select(a);
     const size_t smem = factor_smem_bytes(a);
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kFactorSmem)) != cudaSuccess)
         return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, kBlock, smem) != cudaSuccess) return 0;

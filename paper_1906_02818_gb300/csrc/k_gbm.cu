@@ -183,7 +183,9 @@ int occupancy_of(const void *fn, int block, size_t smem = 0)
     return nb;
 }
 
-// Dynamic shared memory of a basket launch: the warps' Greek slots.
+// Dynamic shared memory of a basket launch: the warps' Greek slots.  They stay
+// within the 48 KB that no function attribute has to allow.
+static_assert(kBasketMaxThreads / 32 * (2 * 64 + 2) * 2 * sizeof(AccSlot) + 1024 <= kSmemNoOptIn, "Greek slots of the largest block");
 size_t greeks_slots(const BasketArgs &a, int block)
 {
     return a.greeks ? static_cast<size_t>(block / 32) * (2 * a.d + 2) * 2 * sizeof(AccSlot) : 0;
@@ -260,23 +262,14 @@ cudaError_t launch_basket_fp32(int D, const BasketArgs &a, const void *cst, int 
 {
     const void *fn = basket_select(D, a);
     if (!fn) return cudaErrorInvalidValue;
-    const size_t smem = greeks_slots(a, block);
-    if (smem > 0) {
-        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-    }
     void *args[] = {const_cast<BasketArgs *>(&a), const_cast<void *>(cst)};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, s);
+    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, greeks_slots(a, block), s);
 }
 
 int basket_fp32_occupancy(int D, const BasketArgs &a, int block)
 {
     const void *fn = basket_select(D, a);
-    if (!fn) return 0;
-    const size_t smem = greeks_slots(a, block);
-    if (smem > 0 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
-        return 0;
-    return occupancy_of(fn, block, smem);
+    return fn ? occupancy_of(fn, block, greeks_slots(a, block)) : 0;
 }
 
 }  // namespace gbmc

@@ -377,6 +377,8 @@ const void *greeks_kernel(int model, int K) {
                      : reinterpret_cast<const void *>(&heston_adjoint_kernel);
 }
 
+// The warps' slots: within the 48 KB that no function attribute has to allow.
+static_assert(kBlock / 32 * MC_MAX_PAYOFFS * 8 * 2 * sizeof(AccSlot) + 1024 <= kSmemNoOptIn, "Greek slots of the most payoffs");
 size_t greeks_smem(int model, int n_payoff)
 {
     const int per = model == MC_HESTON ? 8 : 4;
@@ -397,8 +399,6 @@ cudaError_t launch_greeks(const GreeksArgs &a, int grid, cudaStream_t s)
 {
     const void *fn = greeks_kernel(a.model, a.K);
     const size_t smem = greeks_smem(a.model, a.pay.n);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
     void *args[] = {const_cast<GreeksArgs *>(&a)};
     return cudaLaunchKernel(fn, dim3(grid), dim3(kBlock), args, smem, s);
 }
@@ -407,8 +407,6 @@ int greeks_occupancy(int model, int K, int n_payoff)
 {
     const void *fn = greeks_kernel(model, K);
     const size_t smem = greeks_smem(model, n_payoff);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
-        return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kBlock, smem) != cudaSuccess) return 0;
     return nb;

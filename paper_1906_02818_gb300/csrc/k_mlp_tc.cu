@@ -46,6 +46,13 @@ constexpr int kThreads = 576;
 constexpr int kLaneThreads = 256;        // epilogue threads of one tile lane
 constexpr int kPanelBytes = kRows * 64;  // one 128 x 32 bf16 panel
 constexpr int kSbo = 8 * 64;             // 8-row group stride
+// Dynamic shared memory at width W: at least half the SM's, so that one CTA per
+// SM owns all 512 TMEM columns.  Barriers: 16 + 16 + 16 R + 8 + 8 <= 128.
+constexpr int dyn_smem(int W)
+{
+    const int n = 512 + 2 * (W / kKc) * kPanelBytes + kRing * 2 * W * 64 + 128;
+    return n < 120 * 1024 ? 120 * 1024 : n;
+}
 
 struct Args {
     const float *x;        // [n][n_in]
@@ -432,11 +439,8 @@ cudaError_t mlp_forward_bf16(const MlpLayout &L, const float *params, const uint
     a.b_out = L.b_off[a.NL];
     a.cap = cap;
     a.err = err;
-    const int KC = a.W / kKc;
-    // at least half the SM's shared memory: one CTA per SM, which owns all 512 TMEM columns
-    int smem = 512 + 2 * KC * kPanelBytes + kRing * 2 * a.W * 64 + 128;  // barriers: 16 + 16 + 16 R + 8 + 8 <= 128
-    if (smem < 120 * 1024) smem = 120 * 1024;
-    cudaError_t e = cudaFuncSetAttribute(mlp_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int smem = dyn_smem(a.W);
+    cudaError_t e = cudaFuncSetAttribute(mlp_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_smem(kMaxW));
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -34,6 +34,14 @@ const void *select(int prec, const TcArgs &a, int *smem)
     }
 }
 
+// 4 KB: the static arrays.  The running-sum kernel's size goes with the payoffs
+// and stays below the line; the other's is the same in every call.
+cudaError_t allow_smem(const void *fn, int smem)
+{
+    if (static_cast<size_t>(smem) + 4096 <= kSmemNoOptIn) return cudaSuccess;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+}
+
 }  // namespace
 
 int tc_bimg_bytes(int prec) { return prec == MC_FP8E4M3 ? 64 * 64 : 64 * 64 * 2; }
@@ -43,7 +51,7 @@ cudaError_t launch_basket_tc(int prec, const TcArgs &a, const TcConst &c, int gr
     int smem = 0;
     const void *fn = select(prec, a, &smem);
     if (!fn) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<TcArgs *>(&a), const_cast<TcConst *>(&c)};
     return cudaLaunchKernel(fn, dim3(grid), dim3(kTcThreads), args, static_cast<size_t>(smem), s);
@@ -54,7 +62,7 @@ int basket_tc_occupancy(int prec, const TcArgs &a)
     int smem = 0;
     const void *fn = select(prec, a, &smem);
     if (!fn) return 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 0;
+    if (allow_smem(fn, smem) != cudaSuccess) return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kTcThreads, smem) != cudaSuccess) return 0;
     // The same bound computed from the kernel's resources: registers (per-warp

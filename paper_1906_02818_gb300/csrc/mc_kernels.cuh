@@ -42,6 +42,14 @@ inline void set_seed(PathRun &r, uint64_t seed)
     r.rk = round_keys(r.k0, r.k1);
 }
 
+// Dynamic shared memory a launch may ask for without
+// cudaFuncAttributeMaxDynamicSharedMemorySize.  A launch above the attribute
+// fails, and the attribute is the process's, so where it is needed every call
+// sets the same value, that of the function's largest launch: with each call's
+// own size, a call of another thread could lower it between this one's setting
+// and its launch.
+constexpr size_t kSmemNoOptIn = 48 * 1024;
+
 // Whether the Philox blocks of a path of `steps` steps all have index high
 // word 0 (PathStream's default); runs beyond that read through NormalReader.
 inline bool blocks_fit_32(int64_t steps, int64_t normals_per_step) { return steps * normals_per_step <= (int64_t(1) << 34); }
@@ -81,6 +89,7 @@ struct BasketConst {
     float s0[D];
 };
 
+constexpr int kBasketMaxThreads = 640;  // the stepping kernel's largest block (one path per thread)
 constexpr int kBasketSumBlock = 128;   // block of the summed-normals kernel
 // The largest block of two paths per thread: what the registers of D assets of
 // state leave (0: one path per thread only; at 64 assets two would leave an SM
@@ -291,7 +300,6 @@ struct CorrArgs {
 };
 int corr_occupancy(const CorrArgs &a);
 int corr_block();
-size_t corr_adjoint_smem(int d);
 // Path kernel, batch sums (Hb [B][64 x 64], nb [B]), the Cholesky adjoint per
 // batch and for all paths (out_dl, out_drho [B + 1][d x d]), and the means
 // with batch-means standard errors (res_dl, res_drho [d x d]).  L: FP64
