@@ -10,8 +10,11 @@
 // thread carries P paths, so that each factor pair that comes out of the
 // constant bank serves P instructions: that port, not the FMA pipe, is what
 // one path per thread waits for.  All warps of a block meet at a barrier after
-// every four columns, so that they read the same few hundred bytes of the
-// factor at a time.  A factor staged in shared memory instead was slower: each
+// every sixteen columns, so that they read the same few kilobytes of the factor
+// and of the code at a time; after every four, the barriers cost more than that
+// gave (64 assets, 2^18 paths x 252 steps with a barrier payoff 8.17 ms, every
+// eight 7.91, sixteen 7.84; 32 assets, 50,000 paths x 100 steps 298, 294 and
+// 265 us).  A factor staged in shared memory instead was slower: each
 // 16-byte shared load costs four cycles of the shared-memory port, a quarter
 // of the rate the packed FMAs need.  Every thread runs every step (threads
 // past the last path compute a path whose results are dropped), which keeps
@@ -35,6 +38,18 @@ const void *basket_select_scheme(const BasketArgs &a);
 namespace basket_detail {
 
 constexpr int kMaxWarps = kBasketMaxThreads / 32;
+
+// Path of this thread in round `round`, from the special registers each time:
+// held over the steps, the thread's index, its stride and the test against the
+// last path cost registers that 64 assets of state do not leave (52 bytes of
+// spills, so 32: 8.19 -> 8.07 ms at 2^18 paths x 252 steps with a barrier).
+__device__ __forceinline__ int64_t path_of(int round, int64_t gthreads)
+{
+    uint32_t t, b;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(b));
+    return static_cast<int64_t>(b) * blockDim.x + t + round * gthreads;
+}
 
 __device__ __forceinline__ float elem(const f32x2 *v, int j) { return (j & 1) ? hi_of(v[j >> 1]) : lo_of(v[j >> 1]); }
 
@@ -129,7 +144,6 @@ __global__ void __launch_bounds__(P == 1 ? 32 * kMaxWarps : basket_threads2(D), 
 
     constexpr int H = D / 2;
     const int64_t gthreads = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    const int64_t tid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     const int M = a.run.steps, d = a.d;
     const float inv_m = 1.0f / static_cast<float>(M);
     for (int it = 0; it < a.run.ppt; it += P) {
@@ -140,7 +154,7 @@ __global__ void __launch_bounds__(P == 1 ? 32 * kMaxWarps : basket_threads2(D), 
         int64_t nl = 0;
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            nl = tid + (it + p) * gthreads;
+            nl = path_of(it + p, gthreads);
             valid[p] = it + p < a.run.ppt && nl < a.run.paths;
             n[p] = static_cast<uint64_t>(a.run.path_offset + nl);
             uT[p] = avg[p] = 0.0f;
@@ -235,7 +249,7 @@ __global__ void __launch_bounds__(P == 1 ? 32 * kMaxWarps : basket_threads2(D), 
                             }
                         }
                     }
-                    if (!SAVE) __syncthreads();
+                    if (!SAVE && (kb & 3) == 3) __syncthreads();
                 }
                 if (READ == kReadShifted) o = (o + d) & 3;
 #pragma unroll
@@ -290,7 +304,7 @@ __global__ void __launch_bounds__(P == 1 ? 32 * kMaxWarps : basket_threads2(D), 
         if (!GREEKS && a.pay.n > 0) {
 #pragma unroll
             for (int p = 0; p < P; ++p)
-                if (it + p < a.run.ppt) accumulate_payoffs(s_acc, a.pay, valid[p], uT[p], avg[p], st[p]);
+                if (it + p < a.run.ppt) accumulate_payoffs(s_acc, a.pay, path_of(it + p, gthreads) < a.run.paths, uT[p], avg[p], st[p]);
         }
     }
     if (nvals > 0) block_finish(s_acc, s_red, nvals, a.red);
