@@ -588,38 +588,55 @@ int factor_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const Payof
     return MC_OK;
 }
 
-// Block of an FP32 basket launch (P->bk and P->D set).  The summed-normals
-// kernel: 128.  The stepping kernel: one block per SM, as large (in whole
-// warps) as an equal share of each round of paths asks for: two paths per
-// thread where the width allows it and an SM has more than 256, else one, of
-// up to 640 threads.  Runs of less than a round, or of so few paths that the
-// block would fall under 16 warps: blocks of 128, to spread them.
-void basket_block(mc_plan *P, int64_t paths, int sms)
+// Block, grid and paths per thread of an FP32 basket launch (P->bk and P->D
+// set).  The summed-normals kernel: blocks of 128.  The stepping kernel, one
+// path per thread: one block per SM, as large (in whole warps, up to 640
+// threads) as an equal share of each round of paths asks for; runs of less than
+// a round, or of so few paths that the block would fall under 16 warps: blocks
+// of 128, to spread them.  Two paths per thread, one block per SM, where the
+// width allows it and an SM has more than 256 paths (below, at most one warp
+// per scheduler would be left: 48 assets, 30,000 paths x 100 steps 597 us for
+// 496), if that is no more work for the fullest scheduler, in paths of a warp
+// over all rounds.  us for 100 steps, two against one path per thread: 8 assets
+// 40,000 paths (work 4 : 3) 73 : 64, 60,000 (4 : 4) 73 : 78, 90,000 (6 : 5)
+// 97 : 93, 2^18 (16 : 18) 227 : 257; 32 assets, the same, 326 : 264, 326 : 338,
+// 466 : 415, and 2^18 (16 : 15) 1182 : 1130; 50 assets, 100,003 (6 : 6)
+// 1063 : 1623; 56 assets, 2^18 (18 : 15) 2940 : 2548.  Euler holds two paths'
+// increments beside their states and spills from 24 assets on (24: up to 200
+// bytes a thread, 32: 550, 56: 1360): there equal work goes to one path (32
+// assets, 60,000: 405 : 344) unless two save a round (48 assets, 100,003:
+// 954 : 1497).  Greeks end every block with a reduction of 2 d + 2 values, so
+// never in blocks of 128 (16 assets, 90,000 paths 367 : 537).
+int basket_layout(mc_plan *P, int64_t paths, int sms, int *ppt)
 {
     BasketArgs &b = P->bk;
-    const int64_t per_sm = (paths + sms - 1) / sms;
-    const int most = b.wide || b.run.save ? 0 : basket_threads2(P->D);
+    auto up = [](int64_t n, int64_t unit) { return (n + unit - 1) / unit; };
+    const int64_t per_sm = up(paths, sms);
+    const bool sums = basket_fp32_sums(b);
     b.two = false;
-    if (basket_fp32_sums(b)) {
+    if (sums) {
         P->block = kBasketSumBlock;
-    } else if (most > 0 && per_sm > 256) {
-        b.two = true;
-        const int64_t rounds = (per_sm + 2 * most - 1) / (2 * most);
-        P->block = static_cast<int>((per_sm + 2 * rounds - 1) / (2 * rounds) + 31) / 32 * 32;
     } else {
-        const int64_t rounds = (per_sm + 639) / 640;
-        const int trimmed = static_cast<int>(((per_sm + rounds - 1) / rounds + 31) / 32 * 32);
-        P->block = (per_sm >= 1280 || trimmed >= 512) && per_sm >= 640 ? trimmed : 128;
+        const int64_t rounds = up(per_sm, kBasketMaxThreads);
+        const int trimmed = static_cast<int>(up(up(per_sm, rounds), 32) * 32);
+        P->block = (per_sm >= 2 * kBasketMaxThreads || trimmed >= 512) && per_sm >= kBasketMaxThreads ? trimmed : 128;
     }
-}
-
-// Two paths per thread: whole rounds of them on every SM.
-void basket_grid(mc_plan *P, int64_t paths, int sms, int *ppt)
-{
-    if (!P->bk.two) return;
-    P->grid = static_cast<int>(std::min<int64_t>(sms, (paths + P->block - 1) / P->block));
-    const int64_t round = static_cast<int64_t>(P->grid) * P->block;
-    *ppt = static_cast<int>((paths + round - 1) / round);
+    const int resident = basket_fp32_occupancy(P->D, b, P->block) * sms;
+    if (resident <= 0) return fail(MC_ECUDA, "kernel cannot be resident (occupancy query failed)");
+    size_grid(paths, P->block, resident, &P->grid, ppt);
+    const int most = sums || b.wide || b.run.save ? 0 : basket_threads2(P->D);
+    if (most == 0 || per_sm <= 256) return MC_OK;
+    const int64_t rounds = up(per_sm, 2 * most);
+    const int block = static_cast<int>(up(up(per_sm, 2 * rounds), 32) * 32);
+    const int64_t two = 2 * rounds * up(block, 128), one = *ppt * up(up(P->grid, sms) * P->block, 128);
+    const bool spills = b.scheme == MC_EULER && P->D > 16;
+    if (two < one || (two == one && (!spills || rounds < *ppt)) || (b.greeks && P->block == 128)) {
+        b.two = true;
+        P->block = block;
+        P->grid = static_cast<int>(std::min<int64_t>(sms, up(paths, block)));
+        *ppt = static_cast<int>(up(paths, static_cast<int64_t>(P->grid) * block));
+    }
+    return MC_OK;
 }
 
 // Shared set-up of mc_plan_create and mc_simulate.  save != nullptr selects
@@ -775,7 +792,6 @@ int plan_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const mc_payo
             b.wide = wide;
             b.pay = ps;
             b.red = red;
-            basket_block(P, c->paths, di.sms);
             MC_CUDA(launch_scale_factor(d, P->dL, P->dsig, cfac, sdt, m->r, dt, c->scheme, P->dLp, P->ddrift, s));
             std::vector<float> Lp(tri), drift(d);
             MC_CUDA(cudaMemcpyAsync(&status, P->dstatus, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -806,17 +822,18 @@ int plan_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const mc_payo
                 cW[a] = static_cast<float>(w);
                 cS[a] = static_cast<float>(m->s0[a]);
             }
-            resident = basket_fp32_occupancy(D, b, P->block) * di.sms;
         }
     }
-    if (resident <= 0) return fail(MC_ECUDA, "kernel cannot be resident (occupancy query failed)");
     int ppt = 1;
-    if (P->kk == K_BASKET_TC) {
+    if (P->kk == K_BASKET_FP32) {
+        if ((rc = basket_layout(P, c->paths, di.sms, &ppt))) return rc;
+    } else if (resident <= 0) {
+        return fail(MC_ECUDA, "kernel cannot be resident (occupancy query failed)");
+    } else if (P->kk == K_BASKET_TC) {
         const int64_t tiles = (c->paths + 127) / 128;
         P->grid = static_cast<int>(tiles < resident ? tiles : resident);
     } else {
         size_grid(c->paths, P->block, resident, &P->grid, &ppt);
-        if (P->kk == K_BASKET_FP32) basket_grid(P, c->paths, di.sms, &ppt);
     }
     P->g1.run.ppt = ppt;
     P->bk.run.ppt = ppt;
@@ -1106,13 +1123,7 @@ int mc_greeks(const mc_model *m, const mc_sim_cfg *c, const mc_payoff *pays, int
             b.greeks = true;
             b.T = static_cast<float>(c->T);
             for (int k = 0; k < m->d; ++k) b.sigma[k] = static_cast<float>(m->sigma[k]);
-            basket_block(&P, c->paths, di.sms);
-            const int resident = basket_fp32_occupancy(P.D, b, P.block) * di.sms;
-            if (resident <= 0) return fail(MC_ECUDA, "basket Greeks kernel cannot be resident");
-            int ppt = 1;
-            size_grid(c->paths, P.block, resident, &P.grid, &ppt);
-            basket_grid(&P, c->paths, di.sms, &ppt);
-            b.run.ppt = ppt;
+            if ((rc = basket_layout(&P, c->paths, di.sms, &b.run.ppt))) return rc;
             MC_CUDA(cudaStreamSynchronize(s));  // the set-up's blocks go back to the cache idle
             dfree(P.partials);
             dfree(P.dout);

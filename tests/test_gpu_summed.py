@@ -127,3 +127,16 @@ def test_nested_slices(gb, n_scen, inner):
     wide = gb.risk(pf, n_scen=1500, **kw)["pnl"][:n_scen]
     scale = np.abs(pf["strike"]).sum() * 0.1
     assert np.max(np.abs(alone - wide)) <= 2e-6 * scale, np.max(np.abs(alone - wide))
+
+
+@pytest.mark.parametrize("d,steps,paths", [(5, 5, 70000), (16, 3, 100003), (24, 3, 130000), (30, 3, 100003), (40, 4, 70000),
+                                           (50, 3, 100003), (56, 2, 100003), (48, 2, 160001)])
+def test_fp32_euler_basket_paths_per_thread(gb, orc, d, steps, paths):
+    """The Euler scheme, whose rule for two paths per thread is its own, on both
+    sides of that rule: prices equal the FP64 oracle's on the same paths."""
+    w, pays = _case(d, 2, paths, steps)
+    for group in ([pays[0]], [dict(kind="asian_call", strike=pays[0]["strike"])]):
+        got = gb.price(gbm_model(w), cfg_of(w, scheme="euler"), group)
+        m, se = orc.mean_se(oracle_gbm(orc, w, paths, group, scheme="euler")[0])
+        assert abs(got[0][0] - m) <= REL * abs(m), (d, group, got, m)
+        assert abs(got[0][1] - se) <= 1e-3 * se
