@@ -146,11 +146,14 @@ typedef struct {
 int mc_version(void);
 
 /* Device scratch of the set-up paths (model copies, Cholesky factors,
- * per-block partials, checkpoints) is taken from a per-device cache of blocks
- * that earlier calls released, so repeated calls of one shape allocate
- * nothing; a block is cached only once the call or plan that used it has
- * synchronised.  mc_release_cache frees every cached block (all devices) back
- * to CUDA; blocks held by live plans or running calls are not affected.
+ * per-block partials, checkpoints) and of the risk calls (mc_risk, mc_tail:
+ * buffers of up to 64 MiB) is taken from a per-device cache of blocks that
+ * earlier calls released, so repeated calls of one shape allocate nothing; a
+ * block is cached only once the call or plan that used it has synchronised.
+ * At most 8 GiB (and 1024 blocks) of a device lie idle there; past that the
+ * oldest are freed, and all of them are when the library runs short of device
+ * memory.  mc_release_cache frees every cached block (all devices) back to
+ * CUDA; blocks held by live plans or running calls are not affected.
  * Returns MC_OK. */
 int mc_release_cache(void);
 

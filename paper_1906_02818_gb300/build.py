@@ -32,7 +32,7 @@ def sources():
 
 
 def _inputs():
-    return sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + [
+    return sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + [
         os.path.join(ROOT, "include", "mc.h"), os.path.abspath(__file__)]
 
 

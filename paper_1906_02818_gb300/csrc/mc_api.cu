@@ -9,10 +9,10 @@
 #include <mutex>
 #include <new>
 #include <string>
-#include <unordered_map>
 #include <vector>
 
 #include "mc_kernels.cuh"
+#include "scratch_cache.h"
 
 using namespace gbmc;
 
@@ -167,85 +167,33 @@ void size_grid(int64_t paths, int block, int resident, int *grid, int *ppt)
     *ppt = static_cast<int>(p);
 }
 
-// Device allocations of the set-up paths come from a cache of freed blocks
-// (per device; sizes rounded up to 256 bytes; a request takes the smallest
-// free block of at least its size and at most twice it), so that repeated
-// calls of the same shape pay neither cudaMalloc nor cudaFree (which also
-// synchronises the device).  A block goes back to the cache only when no
-// launch can still use it (its owner has synchronised); mc_release_cache()
-// hands the cached blocks back to CUDA.
-struct CachedBlock {
-    void *p;
-    size_t size;
-    int dev;
-};
-std::mutex g_cache_mu;
-std::vector<CachedBlock> g_free_blocks;
-std::unordered_map<void *, CachedBlock> g_live_blocks;
-
-void release_cached(int dev)  // dev < 0: every device; caller holds g_cache_mu
-{
-    std::vector<CachedBlock> keep;
-    for (const CachedBlock &b : g_free_blocks) {
-        if (dev < 0 || b.dev == dev) {
-            int cur = -1;
-            cudaGetDevice(&cur);
-            if (cur != b.dev) cudaSetDevice(b.dev);
-            cudaFree(b.p);
-            if (cur != b.dev) cudaSetDevice(cur);
-        } else {
-            keep.push_back(b);
-        }
+struct DeviceOps {
+    static constexpr int kNoMemory = cudaErrorMemoryAllocation;
+    static int allocate(void **p, size_t n)
+    {
+        const cudaError_t e = cudaMalloc(p, n);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e;
     }
-    g_free_blocks.swap(keep);
-}
+    static void release(void *p, int dev)
+    {
+        int cur = -1;
+        cudaGetDevice(&cur);
+        if (cur != dev) cudaSetDevice(dev);
+        cudaFree(p);
+        if (cur != dev) cudaSetDevice(cur);
+    }
+};
+ScratchCache<DeviceOps> g_scratch;
 
 cudaError_t dev_alloc_raw(void **p, size_t n)
 {
     int dev = -1;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const size_t sz = n <= 256 ? 256 : (n + 255) & ~static_cast<size_t>(255);
-    std::lock_guard<std::mutex> g(g_cache_mu);
-    size_t best = static_cast<size_t>(-1), bi = 0;
-    for (size_t i = 0; i < g_free_blocks.size(); ++i) {
-        const CachedBlock &b = g_free_blocks[i];
-        if (b.dev == dev && b.size >= sz && b.size <= 2 * sz && b.size < best) {
-            best = b.size;
-            bi = i;
-        }
-    }
-    if (best != static_cast<size_t>(-1)) {
-        const CachedBlock b = g_free_blocks[bi];
-        g_free_blocks[bi] = g_free_blocks.back();
-        g_free_blocks.pop_back();
-        g_live_blocks[b.p] = b;
-        *p = b.p;
-        return cudaSuccess;
-    }
-    e = cudaMalloc(p, sz);
-    if (e == cudaErrorMemoryAllocation && !g_free_blocks.empty()) {
-        cudaGetLastError();
-        release_cached(dev);
-        e = cudaMalloc(p, sz);
-    }
-    if (e != cudaSuccess) return e;
-    g_live_blocks[*p] = CachedBlock{*p, sz, dev};
-    return cudaSuccess;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : static_cast<cudaError_t>(g_scratch.take(dev, n, p));
 }
 
-void dev_free_raw(void *p)
-{
-    if (!p) return;
-    std::lock_guard<std::mutex> g(g_cache_mu);
-    auto it = g_live_blocks.find(p);
-    if (it == g_live_blocks.end()) {
-        cudaFree(p);
-        return;
-    }
-    g_free_blocks.push_back(it->second);
-    g_live_blocks.erase(it);
-}
+void dev_free_raw(void *p) { g_scratch.give(p); }
 
 // Pinned blocks in which a pricing kernel leaves its results for the host: a
 // synchronising call then waits for its kernel alone, not for a copy behind
@@ -254,12 +202,13 @@ struct HostBlock {
     mc_result res[MC_MAX_PAYOFFS];
 };
 constexpr size_t kHostBlocks = 16;
-std::vector<HostBlock *> g_host_blocks;  // guarded by g_cache_mu
+std::mutex g_host_mu;
+std::vector<HostBlock *> g_host_blocks;  // guarded by g_host_mu
 
 HostBlock *host_block_take()
 {
     {
-        std::lock_guard<std::mutex> g(g_cache_mu);
+        std::lock_guard<std::mutex> g(g_host_mu);
         if (!g_host_blocks.empty()) {
             HostBlock *b = g_host_blocks.back();
             g_host_blocks.pop_back();
@@ -278,7 +227,7 @@ void host_block_give(HostBlock *b)  // no launch may still write it
 {
     if (!b) return;
     {
-        std::lock_guard<std::mutex> g(g_cache_mu);
+        std::lock_guard<std::mutex> g(g_host_mu);
         if (g_host_blocks.size() < kHostBlocks) {
             g_host_blocks.push_back(b);
             return;
@@ -380,6 +329,12 @@ void gbmc::debug_register(DebugReader fn) { debug_readers().push_back(fn); }
 
 cudaError_t gbmc::scratch_alloc(void **p, size_t bytes) { return dev_alloc_raw(p, bytes); }
 void gbmc::scratch_free(void *p) { dev_free_raw(p); }
+cudaError_t gbmc::device_alloc_raw(void **p, size_t bytes)
+{
+    int dev = -1;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : static_cast<cudaError_t>(g_scratch.take_uncached(dev, bytes, p));
+}
 
 int gbmc::set_last_error(int code, const char *msg)
 {
@@ -881,8 +836,8 @@ int mc_version(void) { return MC_VERSION; }
 
 int mc_release_cache(void)
 {
-    std::lock_guard<std::mutex> g(g_cache_mu);
-    release_cached(-1);
+    g_scratch.release(-1);
+    std::lock_guard<std::mutex> g(g_host_mu);
     for (HostBlock *b : g_host_blocks) cudaFreeHost(b);
     g_host_blocks.clear();
     return MC_OK;

@@ -344,6 +344,14 @@ cudaError_t launch_corr_wide(const CorrArgs &a, const CorrWide &w, int grid, cud
 // only when no launch can still use it.
 cudaError_t scratch_alloc(void **p, size_t bytes);
 void scratch_free(void *p);
+// Memory that outlives a call (freed with cudaFree), or is too large to keep:
+// cudaMalloc, tried again without the idle scratch where memory is short.
+cudaError_t device_alloc_raw(void **p, size_t bytes);
+template <class T>
+cudaError_t device_alloc(T **p, size_t bytes)
+{
+    return device_alloc_raw(reinterpret_cast<void **>(p), bytes);
+}
 
 // Records the thread-local message returned by mc_last_error(); returns code.
 int set_last_error(int code, const char *msg);

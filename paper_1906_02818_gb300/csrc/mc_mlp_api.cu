@@ -56,7 +56,7 @@ int ensure_work(mc_mlp *N, size_t floats)
     if (N->work) cudaFree(N->work);
     N->work = nullptr;
     N->work_floats = 0;
-    MLP_CUDA(cudaMalloc(&N->work, floats * sizeof(float)));
+    MLP_CUDA(device_alloc(&N->work, floats * sizeof(float)));
     N->work_floats = floats;
     return MC_OK;
 }
@@ -66,7 +66,7 @@ int loss_grad_batch(mc_mlp *N, const float *x, const float *t, int64_t n, cudaSt
 {
     if (N->train_mode == MC_MLP_TRAIN_TF32X3) {
         if (!N->err) {
-            MLP_CUDA(cudaMalloc(&N->err, sizeof(unsigned int)));
+            MLP_CUDA(device_alloc(&N->err, sizeof(unsigned int)));
             MLP_CUDA(cudaMemsetAsync(N->err, 0, sizeof(unsigned int), s));
         }
         MLP_CUDA(mlp_loss_grad_tc(N->L, N->params, x, t, n, N->work, N->grad, N->partial, kPartials, N->err,
@@ -95,10 +95,10 @@ int check_dloss(const mc_mlp *N, const mc_mlp_dloss *dl)
 int loss_grad_batch_d(mc_mlp *N, const float *x, const float *t, const float *g, int64_t n, const mc_mlp_dloss *dl,
                       cudaStream_t s)
 {
-    if (!N->dpartial) MLP_CUDA(cudaMalloc(&N->dpartial, (1 + kMlpMaxDirs) * kPartials * sizeof(double)));
+    if (!N->dpartial) MLP_CUDA(device_alloc(&N->dpartial, (1 + kMlpMaxDirs) * kPartials * sizeof(double)));
     if (N->train_mode == MC_MLP_TRAIN_TF32X3) {
         if (!N->err) {
-            MLP_CUDA(cudaMalloc(&N->err, sizeof(unsigned int)));
+            MLP_CUDA(device_alloc(&N->err, sizeof(unsigned int)));
             MLP_CUDA(cudaMemsetAsync(N->err, 0, sizeof(unsigned int), s));
         }
         MLP_CUDA(mlp_loss_grad_d_tc(N->L, N->params, x, t, g, n, dl->n_dir, dl->dir, dl->scale, dl->weight, N->work,
@@ -170,8 +170,8 @@ int mc_mlp_create(int32_t n_in, int32_t width, int32_t hidden, const float *init
     auto fail_free = [&](int code) { delete N; return code; };
     if (cudaGetDevice(&N->device) != cudaSuccess) return fail_free(set_last_error(MC_ECUDA, "no device"));
     for (float **p : {&N->params, &N->grad, &N->m, &N->v})
-        if (cudaMalloc(p, bytes) != cudaSuccess) return fail_free(set_last_error(MC_ENOMEM, "device allocation failed"));
-    if (cudaMalloc(&N->partial, kPartials * sizeof(double)) != cudaSuccess)
+        if (device_alloc(p, bytes) != cudaSuccess) return fail_free(set_last_error(MC_ENOMEM, "device allocation failed"));
+    if (device_alloc(&N->partial, kPartials * sizeof(double)) != cudaSuccess)
         return fail_free(set_last_error(MC_ENOMEM, "device allocation failed"));
     if (cudaMemcpy(N->params, init, bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(N->m, 0, bytes) != cudaSuccess || cudaMemset(N->v, 0, bytes) != cudaSuccess)
@@ -215,9 +215,9 @@ int mc_mlp_forward(mc_mlp *net, const float *dev_x, int64_t n, float *dev_y, int
         if (!mlp_bf16_supported(net->L))
             return set_last_error(MC_EUNSUPPORTED, "bf16 inference needs n_in <= 10 and equal hidden widths, a "
                                                    "multiple of 32 up to 256");
-        if (!net->img) MLP_CUDA(cudaMalloc(&net->img, mlp_bf16_image_bytes(net->L)));
+        if (!net->img) MLP_CUDA(device_alloc(&net->img, mlp_bf16_image_bytes(net->L)));
         if (!net->err) {
-            MLP_CUDA(cudaMalloc(&net->err, sizeof(unsigned int)));
+            MLP_CUDA(device_alloc(&net->err, sizeof(unsigned int)));
             MLP_CUDA(cudaMemset(net->err, 0, sizeof(unsigned int)));
         }
         if (net->img_version != net->version) {

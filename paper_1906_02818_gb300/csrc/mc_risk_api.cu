@@ -49,7 +49,7 @@ struct DevBufs {
     {
         const size_t bytes = n * sizeof(T) + 16;
         void *q = nullptr;
-        const cudaError_t e = bytes <= kKeep ? scratch_alloc(&q, bytes) : cudaMalloc(&q, bytes);
+        const cudaError_t e = bytes <= kKeep ? scratch_alloc(&q, bytes) : device_alloc(&q, bytes);
         if (e == cudaSuccess) (bytes <= kKeep ? cached : own).push_back(q);
         *p = static_cast<T *>(q);
         return e;
