@@ -232,8 +232,8 @@ int32_t mc_greek_count(const mc_model *model);
  * the prices.  d/dr includes the -T * price term of the discount factor.
  *   MC_HESTON: reverse-mode adjoint kernel; the path state is checkpointed
  *     every cfg->ckpt_every steps (0: 8, or 32 where checkpoints of 8 would
- *     pass 1 GiB; at most 64) in device scratch and
- *     each segment is recomputed from its checkpoint during the backward
+ *     pass 1 GiB or the device has no room for them; at most 64) in device
+ *     scratch and each segment is recomputed from its checkpoint during the backward
  *     sweep.  d sqrt(v+)/dv is taken as 0 where v <= 0.
  *   MC_GBM, d == 1: MC_LOG_EULER (the adjoint of log S is constant along
  *     the path and the sweep reduces to closed forms per path); European and

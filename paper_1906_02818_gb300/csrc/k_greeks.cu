@@ -388,11 +388,12 @@ size_t greeks_smem(int model, int n_payoff)
 int greeks_block() { return kBlock; }
 
 // Checkpoint stride where the caller leaves it open: the register kernel's,
-// unless its checkpoints would take more than 1 GiB (10,000 steps of a full grid).
+// unless its checkpoints would take more than 1 GiB (10,000 steps of a full
+// grid) or, which mc_greeks finds out, more than the device has left.
 int heston_stride(int steps, int64_t threads)
 {
     const int64_t bytes = (static_cast<int64_t>(steps) + kSeg - 1) / kSeg * 2 * threads * static_cast<int64_t>(sizeof(float));
-    return bytes <= (int64_t(1) << 30) ? kSeg : 32;
+    return bytes <= (int64_t(1) << 30) ? kSeg : kHestonStride;
 }
 
 cudaError_t launch_greeks(const GreeksArgs &a, int grid, cudaStream_t s)

@@ -1143,24 +1143,31 @@ int mc_greeks(const mc_model *m, const mc_sim_cfg *c, const mc_payoff *pays, int
     a.pay = ps;
     const int block = greeks_block();
     int grid = 0, ppt = 1;
-    if (m->kind == MC_HESTON && K == 0)
-        K = heston_stride(c->steps, std::min<int64_t>((c->paths + block - 1) / block, int64_t(16) * di.sms) * block);
-    a.K = K;
-    const int occ = greeks_occupancy(a.model, K, np);
-    if (occ <= 0) return fail(MC_ECUDA, "Greeks kernel cannot be resident");
-    size_grid(c->paths, block, occ * di.sms, &grid, &ppt);
-    a.run.ppt = ppt;
+    const bool open = m->kind == MC_HESTON && K == 0;
+    if (open) K = heston_stride(c->steps, std::min<int64_t>((c->paths + block - 1) / block, int64_t(16) * di.sms) * block);
 
     mc_plan P;  // owns the scratch buffers (freed on return)
     P.np = nv;
+    for (;;) {
+        a.K = K;
+        const int occ = greeks_occupancy(a.model, K, np);
+        if (occ <= 0) return fail(MC_ECUDA, "Greeks kernel cannot be resident");
+        size_grid(c->paths, block, occ * di.sms, &grid, &ppt);
+        if (m->kind != MC_HESTON) break;
+        const size_t nseg = (c->steps + K - 1) / K;
+        const cudaError_t e = dev_alloc(&P.ckpt, nseg * 2 * static_cast<size_t>(grid) * block * sizeof(float));
+        if (e == cudaErrorMemoryAllocation && open && K < kHestonStride) {
+            K = kHestonStride;  // a quarter of the checkpoints, in the slower kernel
+            continue;
+        }
+        MC_CUDA(e);
+        break;
+    }
+    a.run.ppt = ppt;
     MC_CUDA(dev_alloc(&P.partials, static_cast<size_t>(grid) * nv * 2 * sizeof(float)));
     MC_CUDA(dev_alloc(&P.ticket, sizeof(unsigned int)));
     MC_CUDA(cudaMemsetAsync(P.ticket, 0, sizeof(unsigned int), s));
     MC_CUDA(dev_alloc(&P.dout, static_cast<size_t>(nv) * sizeof(mc_result)));
-    if (m->kind == MC_HESTON) {
-        const size_t nseg = (c->steps + K - 1) / K;
-        MC_CUDA(dev_alloc(&P.ckpt, nseg * 2 * static_cast<size_t>(grid) * block * sizeof(float)));
-    }
     a.ckpt = P.ckpt;
     a.red.partials = P.partials;
     a.red.ticket = P.ticket;

@@ -189,6 +189,7 @@ struct GreeksArgs {
 };
 cudaError_t launch_greeks(const GreeksArgs &a, int grid, cudaStream_t s);
 int greeks_occupancy(int model, int K, int n_payoff);
+constexpr int kHestonStride = 32;  // checkpoint stride that saves memory
 int heston_stride(int steps, int64_t threads);
 int greeks_block();
 

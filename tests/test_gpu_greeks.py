@@ -131,3 +131,38 @@ def test_greeks_reject_barrier_and_euler(gb):
     with pytest.raises(native.MCError):
         gb.greeks(dict(kind="gbm", s0=[100.0], sigma=[0.2], r=0.05),
                   dict(steps=8, T=1.0, paths=64, scheme="euler"), [dict(kind="call", strike=100.0)])
+
+
+def test_heston_greeks_short_of_memory(gb):
+    """With the stride left open, checkpoints of eight steps that do not fit
+    give way to checkpoints of 32: the results are those of that stride."""
+    import torch
+    from paper_1906_02818_gb300 import native
+    model = dict(kind="heston", s0=100.0, v0=0.04, r=0.05, kappa=2.0, theta=0.04, xi=0.5, rho=-0.7)
+    pays = [dict(kind="call", strike=100.0)]
+    cfg = dict(steps=4096, T=1.0, paths=1 << 18)
+
+    def free():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return torch.cuda.mem_get_info()[0]
+
+    def call(c):  # results, and the device memory that the call leaves in the scratch cache
+        native.lib().mc_release_cache()
+        before = free()
+        r = gb.greeks(model, c, pays)
+        return r, before - free()
+
+    for k in (0, 32):  # both kernels are loaded
+        gb.greeks(model, dict(cfg, steps=8, ckpt_every=k), pays)
+    (p8, g8), need8 = call(cfg)
+    (p32, g32), need32 = call(dict(cfg, ckpt_every=32))
+    assert need8 > need32 + (64 << 20), (need8, need32)
+    native.lib().mc_release_cache()
+    room = torch.empty(free() - (need8 + need32) // 2, dtype=torch.uint8, device="cuda")
+    try:
+        p, g = gb.greeks(model, cfg, pays)
+    finally:
+        del room
+        free()
+    assert np.array_equal(np.array(p), np.array(p32)) and np.array_equal(g, g32)
