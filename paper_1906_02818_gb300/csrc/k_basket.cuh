@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kBasketSumBlock, 5) basket_sum_kernel(const __
                 up_to_four(nblk - g, [&](auto nb) {
                     constexpr int NB = decltype(nb)::value;
                     f32x2 w[2 * NB];
-                    sum_blocks<NB>(w, n, a.run.rk, a.wide, seg.first_block(p) + g, 1, seg.count(p), seg.blocks, NoRounding{});
+                    sum_blocks<NB>(w, n, a.run.rk, a.wide, seg.first_block(p) + g, 1, seg.count(p), seg.blocks);
 #pragma unroll
                     for (int e = 0; e < 4 * NB; ++e) {
                         const int k = 4 * g + e - o;

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
                     up_to_four(static_cast<int>((nblk - g + 7) / 8), [&](auto nb) {
                         constexpr int NB = decltype(nb)::value;
                         f32x2 w[2 * NB];
-                        sum_blocks<NB>(w, rn, a.run.rk, a.wide, seg.first_block(p) + g, 8, seg.count(p), seg.blocks, NoRounding{});
+                        sum_blocks<NB>(w, rn, a.run.rk, a.wide, seg.first_block(p) + g, 8, seg.count(p), seg.blocks);
     #pragma unroll
                         for (int e = 0; e < 4 * NB; ++e) {
                             const int k = static_cast<int>(4 * (g + 8 * (e >> 2))) + (e & 3) - o;

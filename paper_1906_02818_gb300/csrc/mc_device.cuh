@@ -325,12 +325,8 @@ struct Segments {
 };
 
 // w = the sums over `count` steps, `blocks` Philox blocks apart, of the
-// normals of blocks b, b + stride, ... (NB of them) of stream n, each normal
-// passed through `round` (the operand rounding of the reduced precisions).
-// wide: a block index may pass 2^32.
-struct NoRounding {
-    __device__ __forceinline__ f32x2 operator()(f32x2 z) const { return z; }
-};
+// normals of blocks b, b + stride, ... (NB of them) of stream n.  wide: a block
+// index may pass 2^32.
 // f(n) with n = min(left, 4) as a constant: the blocks a thread has left, at
 // most four of them summed at a time (a fixed four would draw the ones past
 // the end too: half of all for 64 assets over eight threads).
@@ -346,9 +342,9 @@ __device__ __forceinline__ void up_to_four(int left, const F &f)
     else if (left == 2) f(Blocks<2>{});
     else f(Blocks<1>{});
 }
-template <int NB, class Round>
+template <int NB>
 __device__ __forceinline__ void sum_blocks(f32x2 (&w)[2 * NB], uint64_t n, const RoundKeys &rk, bool wide, uint64_t b,
-                                           uint32_t stride, int count, uint32_t blocks, const Round &round)
+                                           uint32_t stride, int count, uint32_t blocks)
 {
 #pragma unroll
     for (int j = 0; j < 2 * NB; ++j) w[j] = pack2(0.0f, 0.0f);
@@ -360,15 +356,15 @@ __device__ __forceinline__ void sum_blocks(f32x2 (&w)[2 * NB], uint64_t n, const
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
                 const Normals4 z = ps.normals(q + stride * j, rk);
-                w[2 * j] = fadd2(w[2 * j], round(z.a));
-                w[2 * j + 1] = fadd2(w[2 * j + 1], round(z.b));
+                w[2 * j] = fadd2(w[2 * j], z.a);
+                w[2 * j + 1] = fadd2(w[2 * j + 1], z.b);
             }
     } else {
         for (int s = 0; s < count; ++s)
 #pragma unroll 1
             for (int j = 0; j < NB; ++j) {
                 const float4 z = normals4(static_cast<uint64_t>(s) * blocks + b + stride * j, n, rk);
-                const f32x2 za = round(pack2(z.x, z.y)), zb = round(pack2(z.z, z.w));
+                const f32x2 za = pack2(z.x, z.y), zb = pack2(z.z, z.w);
 #pragma unroll
                 for (int k = 0; k < NB; ++k) {
                     if (k == j) {

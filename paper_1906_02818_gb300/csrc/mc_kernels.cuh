@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cstdlib>
 #include <cuda_runtime.h>
 
 #include "mc_device.cuh"
@@ -51,8 +52,17 @@ inline void set_seed(PathRun &r, uint64_t seed)
 constexpr size_t kSmemNoOptIn = 48 * 1024;
 
 // Whether the Philox blocks of a path of `steps` steps all have index high
-// word 0 (PathStream's default); runs beyond that read through NormalReader.
-inline bool blocks_fit_32(int64_t steps, int64_t normals_per_step) { return steps * normals_per_step <= (int64_t(1) << 34); }
+// word 0 (PathStream's default); runs beyond that read with 64-bit block
+// indices.  No run in reach of a test has 2^34 normals in a path, so a debug
+// build answers no for every run when GBMC_DEBUG_WIDE=1 is set.
+inline bool blocks_fit_32(int64_t steps, int64_t normals_per_step)
+{
+#ifdef GBMC_DEBUG
+    const char *e = std::getenv("GBMC_DEBUG_WIDE");
+    if (e && e[0] == '1') return false;
+#endif
+    return steps * normals_per_step <= (int64_t(1) << 34);
+}
 
 // Single-asset GBM.  log-Euler: y = log2(S/S0) += a + b z with
 // a = log2(e) (r - sigma^2/2) dt, b = log2(e) sigma sqrt(dt).
