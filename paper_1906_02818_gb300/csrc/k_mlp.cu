@@ -735,7 +735,7 @@ __global__ void __launch_bounds__(256) col_parts_kernel(int blocks, int C, const
         s = 0.0f;
         for (int q = 0; q < 8; ++q) s += s_part[q][lane];
         if (p == 0) out[c] = s;
-        else gW0[static_cast<int64_t>(ds.dir[p - 1]) * C + c] += s;
+        else atomicAdd(gW0 + static_cast<int64_t>(ds.dir[p - 1]) * C + c, s);  // directions may share an input
     }
 }
 

@@ -62,3 +62,28 @@ def test_loss_selection(gb, n, alpha):
     var, cvar, nt = orisk.var_cvar(pnl, alpha)
     assert got["var"] == var and got["n_tail"] == nt, (n, alpha, got, var, nt)
     assert abs(got["cvar"] - cvar) <= 1e-12 * max(1.0, abs(cvar))
+
+
+@pytest.mark.parametrize("mode", ["fp32", "tf32x3"])
+@pytest.mark.parametrize("dirs", [[0, 0], [1, 0, 1], [2, 2, 2, 2], [4, 3, 3, 4]])
+def test_directions_that_share_an_input(gb, mode, dirs):
+    """Every direction's share of the first layer's gradient arrives where
+    several name the same input."""
+    import torch
+    width, hidden, n, k = 128, 2, 515, len(dirs)
+    sizes = [5] + [width] * hidden + [1]
+    init = workloads.mlp_init(5, width, hidden, seed=5)
+    net = gb.Mlp(5, width, hidden, init)
+    net.set_train_mode(mode)
+    rng = np.random.default_rng(k)
+    x = rng.uniform(-1, 1, (n, 5)).astype(np.float32)
+    t = rng.uniform(0, 0.5, n).astype(np.float32)
+    g = rng.uniform(-1, 1, (n, k)).astype(np.float32)
+    sc, wt = np.array([1.5, 0.7, 2.0, 1.0][:k]), np.array([0.5, 2.0, 1.0, 0.3][:k])
+    parts, grad = net.loss_grad_d(torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda(), torch.from_numpy(g).cuda(),
+                                  dirs, list(sc), list(wt))
+    loss, p_ref, G = omlp.dloss_and_grads(omlp.unpack(init.astype(np.float64), sizes), x.astype(np.float64),
+                                          t.astype(np.float64), g.astype(np.float64) / sc, dirs, list(wt * sc * sc))
+    ref = omlp.pack(G)
+    assert np.max(np.abs(grad - ref)) <= 1e-4 * np.max(np.abs(ref))
+    net.close()
