@@ -416,9 +416,11 @@ __global__ void sum_under_kernel(int64_t nscen, int d, const double *contrib, do
 // found so far, and its last CTA picks the digit that holds the k-th; then one
 // pass adds up what lies above.  Seven reads of n values over the SMs, in
 // launches of a few microseconds; a sort of all losses in one CTA took 6.5 ms
-// of a 2^16-scenario run.
+// of a 2^16-scenario run.  What one CTA reads anyway (kTailSmall losses) goes
+// through the same passes in one launch: 1000 losses 47 us a call for 84.
 constexpr int kTailBits = 11, kTailBins = 1 << kTailBits, kTailPasses = 6;  // 5 x 11 + 9 bits
-constexpr int kTailBlock = 512, kTailMaxGrid = 304;
+constexpr int kTailBlock = 512, kTailMaxGrid = 304, kTailSmall = 2 * kTailBlock;
+constexpr int kTailPer = kTailBins / kTailBlock;
 struct TailState {
     unsigned long long prefix;       // the digits found
     unsigned int k;                  // rank among the losses that share them, from the largest
@@ -434,44 +436,32 @@ __device__ __forceinline__ unsigned long long loss_key(double l)
     return (u >> 63) ? ~u : u | 0x8000000000000000ull;
 }
 
-// Whether this CTA is the last of the launch to arrive (the others' writes are then visible).
-__device__ __forceinline__ bool last_cta(unsigned int *ticket)
+__device__ __forceinline__ double key_loss(unsigned long long key)
 {
-    __shared__ unsigned int s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1u : 0u;
-    __syncthreads();
-    if (s_last) __threadfence();
-    return s_last != 0u;
+    return __longlong_as_double(static_cast<long long>((key >> 63) ? key & 0x7fffffffffffffffull : ~key));
 }
 
-__global__ void __launch_bounds__(kTailBlock) tail_pass_kernel(int64_t n, const double *__restrict__ pnl, int pass,
-                                                               unsigned int k0, TailState *st)
+// The digit that pass `pass` looks at: `width` bits above `shift`, under the 64 - below bits found.
+struct TailDigit {
+    int below, width, shift;
+    __device__ __forceinline__ explicit TailDigit(int pass)
+        : below(64 - kTailBits * pass), width(below < kTailBits ? below : kTailBits), shift(below - width)
+    {
+    }
+    __device__ __forceinline__ unsigned int of(unsigned long long key) const
+    {
+        return static_cast<unsigned int>((key >> shift) & ((1ull << width) - 1ull));
+    }
+};
+
+// c: counts of the bins kTailBins - 1 - kTailPer t - j of thread t.  True in the one thread whose bins hold the k-th
+// value from the top: *bin, and its rank there.
+__device__ __forceinline__ bool tail_pick(const unsigned int (&c)[kTailPer], unsigned int k, unsigned int *bin, unsigned int *rank)
 {
-    __shared__ unsigned int h[kTailBins];
     __shared__ unsigned int scan[kTailBlock];
     const int t = threadIdx.x;
-    const int below = 64 - kTailBits * pass;                             // bits below the digits found
-    const int width = below < kTailBits ? below : kTailBits, shift = below - width;
-    const unsigned long long prefix = pass ? st->prefix : 0ull;
-    for (int b = t; b < kTailBins; b += kTailBlock) h[b] = 0u;
-    __syncthreads();
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(kTailBlock) + t; i < n; i += static_cast<int64_t>(gridDim.x) * kTailBlock) {
-        const unsigned long long key = loss_key(-pnl[i]);
-        if (pass == 0 || (key >> below) == prefix) atomicAdd(&h[(key >> shift) & ((1ull << width) - 1ull)], 1u);
-    }
-    __syncthreads();
-    for (int b = t; b < kTailBins; b += kTailBlock)
-        if (h[b]) atomicAdd(&st->hist[pass][b], h[b]);
-    if (!last_cta(&st->ticket[pass])) return;
-    // thread t: the bins from kTailBins - 1 - 4 t down; counts from the top
-    constexpr int kPer = kTailBins / kTailBlock;
-    unsigned int c[kPer], own = 0u;
-    for (int j = 0; j < kPer; ++j) {
-        c[j] = *reinterpret_cast<volatile unsigned int *>(&st->hist[pass][kTailBins - 1 - kPer * t - j]);
-        own += c[j];
-    }
+    unsigned int own = 0u;
+    for (int j = 0; j < kTailPer; ++j) own += c[j];
     scan[t] = own;
     __syncthreads();
     for (int o = 1; o < kTailBlock; o <<= 1) {
@@ -480,25 +470,24 @@ __global__ void __launch_bounds__(kTailBlock) tail_pass_kernel(int64_t n, const 
         scan[t] += v;
         __syncthreads();
     }
-    const unsigned int k = pass ? st->k : k0;
     unsigned int above = scan[t] - own;
     __syncthreads();
-    if (above < k && k <= above + own)
-        for (int j = 0; j < kPer; ++j) {
-            if (k <= above + c[j]) {
-                st->prefix = (prefix << width) | static_cast<unsigned long long>(kTailBins - 1 - kPer * t - j);
-                st->k = k - above;
-                break;
-            }
-            above += c[j];
+    if (!(above < k && k <= above + own)) return false;
+    for (int j = 0; j < kTailPer; ++j) {
+        if (k <= above + c[j]) {
+            *bin = static_cast<unsigned int>(kTailBins - 1 - kTailPer * t - j);
+            *rank = k - above;
+            break;
         }
+        above += c[j];
+    }
+    return true;
 }
 
-__global__ void __launch_bounds__(kTailBlock) tail_sum_kernel(int64_t n, const double *__restrict__ pnl, TailState *st, double *res)
+// This CTA's share of the losses above var: their sum and number, in thread 0.
+__device__ __forceinline__ void tail_above(int64_t n, const double *__restrict__ pnl, double var, double *sum, double *count)
 {
     __shared__ double s_red[2][kTailBlock / 32];
-    const unsigned long long key = st->prefix;
-    const double var = __longlong_as_double(static_cast<long long>((key >> 63) ? key & 0x7fffffffffffffffull : ~key));
     double t = 0.0, c = 0.0;
     for (int64_t i = blockIdx.x * static_cast<int64_t>(kTailBlock) + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * kTailBlock) {
         const double l = -pnl[i];
@@ -520,6 +509,94 @@ __global__ void __launch_bounds__(kTailBlock) tail_sum_kernel(int64_t n, const d
             t += s_red[0][w];
             c += s_red[1][w];
         }
+        *sum = t;
+        *count = c;
+    }
+}
+
+// All passes of up to kTailSmall losses in one CTA.
+__global__ void __launch_bounds__(kTailBlock) tail_small_kernel(int n, const double *__restrict__ pnl, unsigned int k0, double *res)
+{
+    __shared__ unsigned int h[kTailBins];
+    __shared__ unsigned long long s_prefix;
+    __shared__ unsigned int s_k;
+    const int t = threadIdx.x;
+    if (t == 0) {
+        s_prefix = 0ull;
+        s_k = k0;
+    }
+    for (int pass = 0; pass < kTailPasses; ++pass) {
+        const TailDigit dg(pass);
+        for (int b = t; b < kTailBins; b += kTailBlock) h[b] = 0u;
+        __syncthreads();
+        const unsigned long long prefix = s_prefix;
+        for (int i = t; i < n; i += kTailBlock) {
+            const unsigned long long key = loss_key(-pnl[i]);
+            if (pass == 0 || (key >> dg.below) == prefix) atomicAdd(&h[dg.of(key)], 1u);
+        }
+        __syncthreads();
+        unsigned int c[kTailPer], bin, rank;
+        for (int j = 0; j < kTailPer; ++j) c[j] = h[kTailBins - 1 - kTailPer * t - j];
+        if (tail_pick(c, s_k, &bin, &rank)) {
+            s_prefix = (prefix << dg.width) | bin;
+            s_k = rank;
+        }
+        __syncthreads();
+    }
+    const double var = key_loss(s_prefix);
+    double sum = 0.0, count = 0.0;
+    tail_above(n, pnl, var, &sum, &count);
+    if (t == 0) {
+        res[0] = var;
+        res[1] = count > 0.0 ? sum / count : var;
+        res[2] = count;
+    }
+}
+
+// Whether this CTA is the last of the launch to arrive (the others' writes are then visible).
+__device__ __forceinline__ bool last_cta(unsigned int *ticket)
+{
+    __shared__ unsigned int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1u : 0u;
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last != 0u;
+}
+
+__global__ void __launch_bounds__(kTailBlock) tail_pass_kernel(int64_t n, const double *__restrict__ pnl, int pass,
+                                                               unsigned int k0, TailState *st)
+{
+    __shared__ unsigned int h[kTailBins];
+    const int t = threadIdx.x;
+    const TailDigit dg(pass);
+    const unsigned long long prefix = pass ? st->prefix : 0ull;
+    for (int b = t; b < kTailBins; b += kTailBlock) h[b] = 0u;
+    __syncthreads();
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(kTailBlock) + t; i < n; i += static_cast<int64_t>(gridDim.x) * kTailBlock) {
+        const unsigned long long key = loss_key(-pnl[i]);
+        if (pass == 0 || (key >> dg.below) == prefix) atomicAdd(&h[dg.of(key)], 1u);
+    }
+    __syncthreads();
+    for (int b = t; b < kTailBins; b += kTailBlock)
+        if (h[b]) atomicAdd(&st->hist[pass][b], h[b]);
+    if (!last_cta(&st->ticket[pass])) return;
+    unsigned int c[kTailPer], bin, rank;
+    for (int j = 0; j < kTailPer; ++j) c[j] = *reinterpret_cast<volatile unsigned int *>(&st->hist[pass][kTailBins - 1 - kTailPer * t - j]);
+    const unsigned int k = pass ? st->k : k0;
+    if (tail_pick(c, k, &bin, &rank)) {
+        st->prefix = (prefix << dg.width) | bin;
+        st->k = rank;
+    }
+}
+
+__global__ void __launch_bounds__(kTailBlock) tail_sum_kernel(int64_t n, const double *__restrict__ pnl, TailState *st, double *res)
+{
+    const double var = key_loss(st->prefix);
+    double t = 0.0, c = 0.0;
+    tail_above(n, pnl, var, &t, &c);
+    if (threadIdx.x == 0) {
         st->sum[blockIdx.x] = t;
         st->count[blockIdx.x] = c;
     }
@@ -610,6 +687,10 @@ cudaError_t launch_tail(int64_t n, const double *pnl, void *scratch, double alph
     TailState *st = static_cast<TailState *>(scratch);
     int64_t k = static_cast<int64_t>(std::ceil((1.0 - alpha) * static_cast<double>(n) - 1e-9));
     if (k < 1) k = 1;
+    if (n <= kTailSmall) {
+        tail_small_kernel<<<1, kTailBlock, 0, s>>>(static_cast<int>(n), pnl, static_cast<unsigned int>(k), res);
+        return cudaGetLastError();
+    }
     cudaError_t e = cudaMemsetAsync(st, 0, sizeof(TailState), s);
     if (e != cudaSuccess) return e;
     const int grid = static_cast<int>(std::min<int64_t>(kTailMaxGrid, (n + 2 * kTailBlock - 1) / (2 * kTailBlock)));
