@@ -13,7 +13,7 @@
 //     sums every eighth Philox block of its path over the steps, up to four
 //     blocks at a time in registers, into W[k][path] in shared memory; one
 //     contraction per tile.  Bound by drawing; the contraction of every step
-//     took 141 ms for 2^16 paths x 252 steps at d = 512, this 6 ms.
+//     took 141 ms for 2^16 paths x 252 steps at d = 512, this 6.8 ms.
 //   * Greeks: contracted every step.  The payoff's slope is an indicator of
 //     U > K, and one path that falls on the other side of K by a rounding
 //     moves the vegas, sums of large terms of both signs, by 1e-4; so the
@@ -110,27 +110,40 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
             }
         };
         if (GREEKS) {
-            NormalReader rd;
-            rd.init(rn, a.run.rk);
+            // thread (path t mod 64, t / 64) draws an eighth of the columns: whole blocks when 4 | d, else the lanes
+            // that the step's place in its first block picks from two blocks in registers
             PathStream ps;
             ps.init(rn, a.run.rk);
+            const int k0 = static_cast<int>(rq) * (D / 8), k1 = min(k0 + D / 8, d);
+            auto put = [&](int k, const float4 &z) {
+                zs[(k + 0) * kP + rp] = z.x;
+                zs[(k + 1) * kP + rp] = z.y;
+                zs[(k + 2) * kP + rp] = z.z;
+                zs[(k + 3) * kP + rp] = z.w;
+            };
             for (int i = 0; i < M; ++i) {
                 __syncthreads();  // previous step done with zs
-                for (int k = static_cast<int>(rq) * (D / 8); k < (static_cast<int>(rq) + 1) * (D / 8) && k < d; k += 4) {
-                    float4 z;
-                    if (a.exact4) {
-                        z = ps.normals((static_cast<uint32_t>(i) * (d >> 2)) + (k >> 2), a.run.rk).f4();
-                    } else {
-                        const uint64_t j0 = static_cast<uint64_t>(i) * d + k;
-                        z.x = rd.get(j0);
-                        z.y = k + 1 < d ? rd.get(j0 + 1) : 0.f;
-                        z.z = k + 2 < d ? rd.get(j0 + 2) : 0.f;
-                        z.w = k + 3 < d ? rd.get(j0 + 3) : 0.f;
+                const uint64_t j0 = static_cast<uint64_t>(i) * d + k0;
+                if (a.wide) {
+                    NormalReader rd;
+                    rd.init(rn, a.run.rk);
+                    for (int k = k0; k < k1; ++k) zs[k * kP + rp] = rd.get(j0 + k - k0);
+                } else if (a.exact4) {
+                    const uint32_t q = static_cast<uint32_t>(j0 >> 2) - (k0 >> 2);
+                    for (int k = k0; k < k1; k += 4) put(k, ps.normals(q + (k >> 2), a.run.rk).f4());
+                } else if (k0 < k1) {
+                    uint32_t q = static_cast<uint32_t>(j0 >> 2);
+                    const int o = static_cast<int>(j0 & 3);
+                    float4 cur = ps.normals(q, a.run.rk).f4();
+                    for (int k = k0; k < k1; k += 4) {
+                        const float4 nxt = ps.normals(++q, a.run.rk).f4();
+                        float4 z = shifted4(cur, nxt, o);
+                        if (k + 1 >= d) z.y = 0.0f;
+                        if (k + 2 >= d) z.z = 0.0f;
+                        if (k + 3 >= d) z.w = 0.0f;
+                        put(k, z);
+                        cur = nxt;
                     }
-                    zs[(k + 0) * kP + rp] = z.x;
-                    zs[(k + 1) * kP + rp] = z.y;
-                    zs[(k + 2) * kP + rp] = z.z;
-                    zs[(k + 3) * kP + rp] = z.w;
                 }
                 contract();
             }
