@@ -19,7 +19,8 @@
 //     moves the vegas, sums of large terms of both signs, by 1e-4; so the
 //     Greeks keep the sums they have always been formed from.
 //   * Epilogue: log2(S_a / S0_a) = M drift_a + (Lhat W)_a, the basket,
-//     European payoffs and the pathwise delta / vega / rho of payoff 0.
+//     European payoffs and the pathwise delta / vega / rho of payoff 0.  Every
+//     sum has a fixed order: a run's results have the same bits each time.
 #include "mc_kernels.cuh"
 
 namespace gbmc {
@@ -50,6 +51,7 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
     __shared__ float s_pay[MC_MAX_PAYOFFS][2];
     __shared__ float s_g[kBigMaxD * 2 + 1][2];
     __shared__ float s_u[kP];
+    __shared__ float s_w[2][MC_MAX_PAYOFFS + 1][2];  // sums of the two warps that hold a tile's payoffs; last: rho
     const int t = threadIdx.x, lane = t & 31;
     const int pg = t >> 5, ag = t & 31;  // a warp = one path group, 32 asset groups
     const int d = a.d, nv = a.pay.n, M = a.run.steps;
@@ -195,8 +197,8 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
                 const float f = valid ? payoff_eval(a.pay.kind[q], a.pay.strike[q], INFINITY, s_u[t], 0.f, 0.f, 0.f) : 0.f;
                 const float s1 = warp_sum(f), s2 = warp_sum(f * f);
                 if (lane == 0) {
-                    atomicAdd(&s_pay[q][0], s1);
-                    atomicAdd(&s_pay[q][1], s2);
+                    s_w[pg][q][0] = s1;
+                    s_w[pg][q][1] = s2;
                 }
             }
         }
@@ -210,8 +212,12 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
                                                          : (U > a.pay.strike[0] ? 1.f : 0.f))
                               : 0.f;
             }
+            // the warps' sums of delta, delta^2, vega, vega^2 per column, [4][16 warps][D], over the normals (read no
+            // more); then added in the warps' order
+            float *red = zs;
 #pragma unroll
-            for (int j = 0; j < J; ++j)
+            for (int j = 0; j < J; ++j) {
+                float4 sums[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int col = 128 * j + 4 * ag + e;
@@ -226,14 +232,14 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
                             d1 += dl; d2 += dl * dl; v1 += vg; v2 += vg * vg;
                         }
                     }
-                    // each lane holds its own columns: one atomic per (warp, column)
-                    if (col < d) {
-                        atomicAdd(&s_g[col][0], d1);
-                        atomicAdd(&s_g[col][1], d2);
-                        atomicAdd(&s_g[d + col][0], v1);
-                        atomicAdd(&s_g[d + col][1], v2);
-                    }
+                    reinterpret_cast<float *>(&sums[0])[e] = d1;
+                    reinterpret_cast<float *>(&sums[1])[e] = d2;
+                    reinterpret_cast<float *>(&sums[2])[e] = v1;
+                    reinterpret_cast<float *>(&sums[3])[e] = v2;
                 }
+#pragma unroll
+                for (int v = 0; v < 4; ++v) *reinterpret_cast<float4 *>(red + (v * 16 + pg) * D + 128 * j + 4 * ag) = sums[v];
+            }
             if (t < kP) {
                 const float U = s_u[t];
                 const bool valid = tile * kP + t < a.run.paths;
@@ -244,13 +250,27 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
                 const float rr = g * U * a.T - a.T * f;
                 const float r1 = warp_sum(rr), r2 = warp_sum(rr * rr);
                 if (lane == 0) {
-                    atomicAdd(&s_g[2 * d][0], r1);
-                    atomicAdd(&s_g[2 * d][1], r2);
+                    s_w[pg][nv][0] = r1;
+                    s_w[pg][nv][1] = r2;
                 }
             }
         }
         __syncthreads();
+        if (t < 2 * nv) s_pay[t >> 1][t & 1] += s_w[0][t >> 1][t & 1] + s_w[1][t >> 1][t & 1];
+        if (GREEKS) {
+            if (t < 2) s_g[2 * d][t] += s_w[0][nv][t] + s_w[1][nv][t];
+            for (int i = t; i < 4 * d; i += kThreads) {
+                const int v = i / d, col = i - v * d;
+                float sum = 0.0f;
+#pragma unroll
+                for (int w = 0; w < kThreads / 32; ++w) sum += zs[(v * 16 + w) * D + col];
+                s_g[(v >> 1) * d + col][v & 1] += sum;
+            }
+            __syncthreads();
+            for (int i = d * kP + t; i < nchunks * kKC * kP; i += kThreads) zs[i] = 0.0f;
+        }
     }
+    __syncthreads();
     // per-CTA partials -> FP64 sum by the last CTA
     const int nvals = nv + (GREEKS ? 2 * d + 1 : 0);
     for (int i = t; i < nvals * 2; i += kThreads) {

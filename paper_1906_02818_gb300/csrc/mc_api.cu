@@ -557,8 +557,8 @@ int factor_setup(mc_plan *P, const mc_model *m, const mc_sim_cfg *c, const Payof
 // 97 : 93, 2^18 (16 : 18) 227 : 257; 32 assets, the same, 326 : 264, 326 : 338,
 // 466 : 415, and 2^18 (16 : 15) 1182 : 1130; 50 assets, 100,003 (6 : 6)
 // 1063 : 1623; 56 assets, 2^18 (18 : 15) 2940 : 2548.  Euler holds two paths'
-// increments beside their states and spills from 24 assets on (24: up to 200
-// bytes a thread, 32: 550, 56: 1360): there equal work goes to one path (32
+// increments beside their states and spills from 24 assets on (24: up to 128
+// bytes a thread, 32: 364, 56: 904): there equal work goes to one path (32
 // assets, 60,000: 405 : 344) unless two save a round (48 assets, 100,003:
 // 954 : 1497).  Greeks end every block with a reduction of 2 d + 2 values, so
 // never in blocks of 128 (16 assets, 90,000 paths 367 : 537).
@@ -592,6 +592,25 @@ int basket_layout(mc_plan *P, int64_t paths, int sms, int *ppt)
         *ppt = static_cast<int>(up(paths, static_cast<int64_t>(P->grid) * block));
     }
     return MC_OK;
+}
+
+// Whether the FP32 Greeks of a basket of d <= 64 assets are formed by the
+// large-basket kernel (a path's assets over eight threads) and not by the
+// stepping kernel (a path per thread).  The latter pays more per path and block
+// at the end (2 d + 2 values), and its steps last as long for few paths as for
+// a full SM.  us, large-basket : stepping kernel: 64 assets, up to 9,728 paths
+// (one round of tiles) 755 : 1130 at 120 steps, 236 : 295 at 8; 20,000 paths (3
+// rounds) 348 : 416 at 8, 659 : 585 at 30; 80,000 (9) 604 : 784 at 8, 1526 :
+// 1052 at 30.  50 assets, one round 757 : 1049 at 120, 20,000 paths 234 : 271 at
+// 2, 324 : 321 at 8, 80,000 329 : 300 at 2; 48 assets, one round 631 : 642 at
+// 120; 40 assets, one round 172 : 187 at 2, 603 : 364 at 120, 40,000 paths
+// 238 : 271 at 2.
+bool greeks_wide(int d, int steps, int64_t paths, int sms)
+{
+    const int64_t rounds = (paths + 64 * static_cast<int64_t>(sms) - 1) / (64 * static_cast<int64_t>(sms));
+    if (d > 56) return rounds == 1 || steps <= 13 + 34 / ((rounds - 1) * (rounds - 1));
+    if (d > 40 && rounds == 1) return true;
+    return d > 16 && rounds <= 5 && steps <= 5;
 }
 
 // Shared set-up of mc_plan_create and mc_simulate.  save != nullptr selects
@@ -1068,12 +1087,12 @@ int mc_greeks(const mc_model *m, const mc_sim_cfg *c, const mc_payoff *pays, int
         run.save_every = 1;
         mc_plan P;
         const int G = 2 * m->d + 1;
+        DeviceInfo di;
+        if ((rc = device_info(&di))) return rc;
         if (m->d <= 64 && c->precision == MC_FP32 && c->scheme == MC_LOG_EULER && (ps.kind[0] == MC_CALL || ps.kind[0] == MC_PUT) &&
-            blocks_fit_32(c->steps, m->d)) {
+            blocks_fit_32(c->steps, m->d) && !greeks_wide(m->d, c->steps, c->paths, di.sms)) {
             // a path per thread (the stepping kernel); its reduction holds the price and the G Greeks
             if ((rc = plan_setup(&P, m, c, pays, np, nullptr, 0, s))) return rc;
-            DeviceInfo di;
-            if ((rc = device_info(&di))) return rc;
             BasketArgs &b = P.bk;
             b.greeks = true;
             b.T = static_cast<float>(c->T);

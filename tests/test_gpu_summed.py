@@ -140,3 +140,20 @@ def test_fp32_euler_basket_paths_per_thread(gb, orc, d, steps, paths):
         m, se = orc.mean_se(oracle_gbm(orc, w, paths, group, scheme="euler")[0])
         assert abs(got[0][0] - m) <= REL * abs(m), (d, group, got, m)
         assert abs(got[0][1] - se) <= 1e-3 * se
+
+
+@pytest.mark.parametrize("d,steps,paths", [(17, 5, 3000), (17, 6, 3000), (40, 2, 20000), (48, 6, 9000), (48, 6, 9800),
+                                           (57, 20, 31000), (64, 30, 30000)])
+def test_fp32_basket_greeks_either_kernel(gb, orc, d, steps, paths):
+    """Both sides of the rule that sends short or small runs to the
+    large-basket kernel, against the FP64 oracle on the same paths.  One path
+    whose basket value lies within rounding of the strike may fall on its other
+    side: its whole term is allowed for."""
+    w, pays = _case(d, 2, paths, steps)
+    pr, g = gb.greeks(gbm_model(w), cfg_of(w), pays[:1])
+    ref = orc.gbm_greeks(w["s0"], w["sigma"], w["r"], w["T"], steps, paths, pays[:1], corr=w["corr"], weights=w["weights"])[0]
+    scale = np.max(np.abs(ref.mean(axis=1)[:d]))
+    for k in range(2 * d + 1):
+        m = ref[k].mean()
+        tol = 2e-5 * max(abs(m), scale, np.mean(np.abs(ref[k]))) + np.max(np.abs(ref[k])) / paths
+        assert abs(g[0, k, 0] - m) <= tol, (d, k, g[0, k, 0], m, tol)
