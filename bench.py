@@ -328,7 +328,7 @@ def config_c3(torch, gb, orc, hw, flush, reps):
             "error_vs_oracle": {"paths": n_or, "max_rel": max(e["rel"] for e in _errors(orc, small, ref)),
                                 "per_price": _errors(orc, small, ref)},
             "greeks": {"ms": tg * 1e3, "wall_ms": tg_wall * 1e3, "value": ps / tg, "unit": UNIT,
-                       "what": "7 pathwise Greeks of 18 options, adjoint with checkpoints every 32 steps",
+                       "what": "7 pathwise Greeks of 18 options, adjoint with checkpoints every 8 steps",
                        "call_K80": {nm: [float(g[0, k, 0]), float(g[0, k, 1])] for k, nm in enumerate(names)},
                        "error_vs_oracle_forward_mode": {"paths": n_g, "call_K80": gerr},
                        "cpu_baseline": {"value": n_g * w["steps"] / tg_or, "unit": UNIT, "cores": os.cpu_count(),

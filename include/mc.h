@@ -213,6 +213,11 @@ int mc_simulate(const mc_model *model, const mc_sim_cfg *cfg, int32_t save_every
  * mc_price -- discounted Monte Carlo prices of n_payoff payoffs on the same
  * simulated paths (Eq. 3), with standard errors.
  *   out: host [n_payoff] results.  1 <= n_payoff <= MC_MAX_PAYOFFS.
+ * The last digits of a European price may depend on the payoffs beside it:
+ * under MC_LOG_EULER with MC_FP32 (d <= 64), European payoffs among themselves
+ * are priced from the path's summed normals, beside one on the path from the
+ * state stepped through the dates.  The paths and the estimator are the same;
+ * the FP32 sums round in another order (about 1e-7 relative).
  * Synchronises `stream` before returning.
  */
 int mc_price(const mc_model *model, const mc_sim_cfg *cfg, const mc_payoff *payoffs,
