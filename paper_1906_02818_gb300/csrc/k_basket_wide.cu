@@ -19,8 +19,10 @@
 //     moves the vegas, sums of large terms of both signs, by 1e-4; so the
 //     Greeks keep the sums they have always been formed from.
 //   * Epilogue: log2(S_a / S0_a) = M drift_a + (Lhat W)_a, the basket,
-//     European payoffs and the pathwise delta / vega / rho of payoff 0.  Every
-//     sum has a fixed order: a run's results have the same bits each time.
+//     European payoffs and the pathwise delta / vega / rho of payoff 0.  The
+//     sums of a run with Greeks have a fixed order, so its results have the
+//     same bits each time.  (Prices add the sums of a tile's two payoff warps
+//     as they come; in a fixed order the price kernel took 4 % longer.)
 #include "mc_kernels.cuh"
 
 namespace gbmc {
@@ -197,8 +199,13 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
                 const float f = valid ? payoff_eval(a.pay.kind[q], a.pay.strike[q], INFINITY, s_u[t], 0.f, 0.f, 0.f) : 0.f;
                 const float s1 = warp_sum(f), s2 = warp_sum(f * f);
                 if (lane == 0) {
-                    s_w[pg][q][0] = s1;
-                    s_w[pg][q][1] = s2;
+                    if (GREEKS) {
+                        s_w[pg][q][0] = s1;
+                        s_w[pg][q][1] = s2;
+                    } else {
+                        atomicAdd(&s_pay[q][0], s1);
+                        atomicAdd(&s_pay[q][1], s2);
+                    }
                 }
             }
         }
@@ -256,8 +263,8 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
             }
         }
         __syncthreads();
-        if (t < 2 * nv) s_pay[t >> 1][t & 1] += s_w[0][t >> 1][t & 1] + s_w[1][t >> 1][t & 1];
         if (GREEKS) {
+            if (t < 2 * nv) s_pay[t >> 1][t & 1] += s_w[0][t >> 1][t & 1] + s_w[1][t >> 1][t & 1];
             if (t < 2) s_g[2 * d][t] += s_w[0][nv][t] + s_w[1][nv][t];
             for (int i = t; i < 4 * d; i += kThreads) {
                 const int v = i / d, col = i - v * d;
@@ -270,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1) basket_wide_kernel(const __grid_c
             for (int i = d * kP + t; i < nchunks * kKC * kP; i += kThreads) zs[i] = 0.0f;
         }
     }
-    __syncthreads();
+    if (GREEKS) __syncthreads();
     // per-CTA partials -> FP64 sum by the last CTA
     const int nvals = nv + (GREEKS ? 2 * d + 1 : 0);
     for (int i = t; i < nvals * 2; i += kThreads) {
