@@ -601,14 +601,15 @@ int basket_layout(mc_plan *P, int64_t paths, int sms, int *ppt)
 // a full SM.  us, large-basket : stepping kernel: 64 assets, up to 9,728 paths
 // (one round of tiles) 755 : 1130 at 120 steps, 236 : 295 at 8; 20,000 paths (3
 // rounds) 348 : 416 at 8, 659 : 585 at 30; 80,000 (9) 604 : 784 at 8, 1526 :
-// 1052 at 30.  50 assets, one round 757 : 1049 at 120, 20,000 paths 234 : 271 at
+// 1052 at 30; from 640 paths per SM on the latter has one block per SM and less
+// to add up (200,000 paths 1071 : 567 at 8).  50 assets, one round 757 : 1049 at 120, 20,000 paths 234 : 271 at
 // 2, 324 : 321 at 8, 80,000 329 : 300 at 2; 48 assets, one round 631 : 642 at
 // 120; 40 assets, one round 172 : 187 at 2, 603 : 364 at 120, 40,000 paths
 // 238 : 271 at 2.
 bool greeks_wide(int d, int steps, int64_t paths, int sms)
 {
     const int64_t rounds = (paths + 64 * static_cast<int64_t>(sms) - 1) / (64 * static_cast<int64_t>(sms));
-    if (d > 56) return rounds == 1 || steps <= 13 + 34 / ((rounds - 1) * (rounds - 1));
+    if (d > 56) return rounds == 1 || (paths < static_cast<int64_t>(kBasketMaxThreads) * sms && steps <= 13 + 34 / ((rounds - 1) * (rounds - 1)));
     if (d > 40 && rounds == 1) return true;
     return d > 16 && rounds <= 5 && steps <= 5;
 }
