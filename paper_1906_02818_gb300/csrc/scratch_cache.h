@@ -16,9 +16,12 @@
 #pragma once
 
 #include <cstddef>
+#include <iterator>
+#include <list>
+#include <map>
 #include <mutex>
 #include <unordered_map>
-#include <vector>
+#include <utility>
 
 namespace gbmc {
 
@@ -35,17 +38,16 @@ public:
     {
         const size_t size = n <= 256 ? 256 : (n + 255) & ~static_cast<size_t>(255);
         std::lock_guard<std::mutex> g(mu_);
-        auto best = idle_.end();
-        for (auto b = idle_.begin(); b != idle_.end(); ++b)
-            if (b->dev == dev && b->size >= size && b->size <= 2 * size && (best == idle_.end() || b->size < best->size)) best = b;
-        if (best != idle_.end()) {
-            *p = best->p;
-            live_[best->p] = *best;
-            idle_.erase(best);
+        const auto best = by_size_.lower_bound({dev, size});
+        if (best != by_size_.end() && best->first.first == dev && best->first.second <= 2 * size) {
+            const Block b = *best->second;
+            drop(best->second);
+            live_[b.p] = b;
+            *p = b.p;
             return 0;
         }
         const int e = allocate(dev, size, p);
-        if (e == 0) live_[*p] = Block{*p, size, dev};
+        if (e == 0) live_[*p] = Block{*p, size, dev, {}};
         return e;
     }
 
@@ -70,21 +72,16 @@ public:
             return;
         }
         idle_.push_back(given);
-        size_t bytes = 0, blocks = 0;
-        for (const Block &b : idle_)
-            if (b.dev == dev) {
-                bytes += b.size;
-                ++blocks;
-            }
-        for (auto b = idle_.begin(); b != idle_.end() && (bytes > kIdleBytes || blocks > kIdleBlocks);) {
-            if (b->dev != dev) {
-                ++b;
-                continue;
-            }
-            bytes -= b->size;
-            --blocks;
-            Ops::release(b->p, b->dev);
-            b = idle_.erase(b);
+        idle_.back().at = by_size_.insert({{dev, given.size}, std::prev(idle_.end())});
+        Total &t = total_[dev];
+        t.bytes += given.size;
+        ++t.blocks;
+        for (auto b = idle_.begin(); t.bytes > kIdleBytes || t.blocks > kIdleBlocks;) {
+            const auto old = b++;
+            if (old->dev != dev) continue;
+            const Block gone = *old;
+            drop(old);
+            Ops::release(gone.p, dev);
         }
     }
 
@@ -96,15 +93,32 @@ public:
     }
 
 private:
+    struct Block;
+    using Idle = std::list<Block>;  // oldest first
+    using Index = std::multimap<std::pair<int, size_t>, typename Idle::iterator>;  // by device and size
     struct Block {
         void *p;
         size_t size;
         int dev;
+        typename Index::iterator at;  // idle blocks: the entry of the index
+    };
+    struct Total {
+        size_t bytes = 0, blocks = 0;
     };
     std::mutex mu_;
-    std::vector<Block> idle_;  // oldest first
+    Idle idle_;
+    Index by_size_;
+    std::map<int, Total> total_;  // idle, by device
     std::unordered_map<void *, Block> live_;
 
+    void drop(typename Idle::iterator b)
+    {
+        Total &t = total_[b->dev];
+        t.bytes -= b->size;
+        --t.blocks;
+        by_size_.erase(b->at);
+        idle_.erase(b);
+    }
     int allocate(int dev, size_t n, void **p)
     {
         int e = Ops::allocate(p, n);
@@ -115,12 +129,11 @@ private:
     {
         bool any = false;
         for (auto b = idle_.begin(); b != idle_.end();) {
-            if (dev >= 0 && b->dev != dev) {
-                ++b;
-                continue;
-            }
-            Ops::release(b->p, b->dev);
-            b = idle_.erase(b);
+            const auto old = b++;
+            if (dev >= 0 && old->dev != dev) continue;
+            const Block gone = *old;
+            drop(old);
+            Ops::release(gone.p, gone.dev);
             any = true;
         }
         return any;
