@@ -253,9 +253,10 @@ int mc_risk(const mc_portfolio *pf, const mc_risk_cfg *cf, mc_risk_result *res, 
         int dev = 0, sms = 0;
         RK_CUDA(cudaGetDevice(&dev));
         RK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int bsl = nested_slices(d, cf->base_paths, sms), isl = nested_slices(ns * d, cf->inner_paths, sms);
+        const int bsl = nested_slices(d, cf->base_paths, true, sms), isl = nested_slices(ns * d, cf->inner_paths, false, sms);
         RK_CUDA(B.alloc(&d_contrib, ns * d));
-        RK_CUDA(B.alloc(&d_part, std::max(nested_part_doubles(d, cf->base_paths, bsl), nested_part_doubles(ns * d, cf->inner_paths, isl))));
+        RK_CUDA(B.alloc(&d_part, std::max(nested_part_doubles(d, cf->base_paths, true, bsl),
+                                         nested_part_doubles(ns * d, cf->inner_paths, false, isl))));
         a.inner = cf->base_paths;
         RK_CUDA(launch_nested(a, 1, nullptr, nullptr, d_part, bsl, s));  // base values at S0, full maturities
         a.inner = cf->inner_paths;

@@ -35,8 +35,8 @@ cudaError_t launch_outer(int64_t nscen, int64_t off, int d, const float *Lc, con
                          const RoundKeys &rk, float *Sp, cudaStream_t s);
 // Inner paths of nscen scenarios (Sp == nullptr: the base date) in `slices`
 // CTAs per (scenario, underlying); part: nested_part_doubles scratch.
-int nested_slices(int64_t pairs, int inner, int sms);
-size_t nested_part_doubles(int64_t pairs, int inner, int slices);
+int nested_slices(int64_t pairs, int inner, bool base, int sms);
+size_t nested_part_doubles(int64_t pairs, int inner, bool base, int slices);
 cudaError_t launch_nested(const RiskArgs &a, int64_t nscen, const float *Sp, double *contrib, double *part, int slices,
                           cudaStream_t s);
 cudaError_t launch_sum_under(int64_t nscen, int d, const double *contrib, double *pnl, cudaStream_t s);
